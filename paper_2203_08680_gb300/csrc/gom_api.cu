@@ -526,17 +526,14 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
     {
         const int R = tabs.max_abs_w < (int64_t(1) << 12) ? 12 : 16;
         if (coop && variant == kVarNarrow && max_w <= 255 && tabs.max_abs_w < (int64_t(1) << 16)) {
-            const int sm = static_cast<int>(std::max<int64_t>(tabs.max_s, 1) | 1); // odd row stride: no bank conflicts
             const int S = static_cast<int>(std::max<int64_t>(tabs.max_s, 1));
-            const int epw = 32 / S, E0 = 32 / c->W;
-            const int nc = (E0 + epw - 1) / epw;
-            const int64_t ww = gom_bs_warp_words(sm, nc, c->W);
+            const int64_t ww = gom_bs_warp_words(S);
             const int wpb = static_cast<int>(std::min<int64_t>(kBsThreads / 32, kSmemBudget / (ww * 4)));
             // the block's fitness accumulators (32 W int64), then the warps' regions
             const size_t smem = std::max(static_cast<size_t>(256 * c->W + ww * 4 * wpb), keys_smem);
             // the kernels without the learned filter's code, and with it (same grids)
-            const void *rf = gom_run_bs_kernel(R, false), *mf = gom_mix_bs_kernel(R, false);
-            const void *rfl = gom_run_bs_kernel(R, true), *mfl = gom_mix_bs_kernel(R, true);
+            const void *rf = gom_run_bs_kernel(S, R, false), *mf = gom_mix_bs_kernel(S, R, false);
+            const void *rfl = gom_run_bs_kernel(S, R, true), *mfl = gom_mix_bs_kernel(S, R, true);
             if (wpb >= 1 && smem <= static_cast<size_t>(kSmemBudget) && rf && mf && rfl && mfl) {
                 const int E = 32 / c->W;
                 const int64_t items = (max_group + E - 1) / E;
@@ -559,10 +556,7 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
                     c->bs_grid_run = static_cast<int>(std::min<int64_t>(static_cast<int64_t>(c->sms) * occ_r, need));
                     c->bs_grid_mix = static_cast<int>(std::min<int64_t>(
                         std::min<int64_t>(static_cast<int64_t>(c->sms) * occ_m, need), kMaxMixBlocks));
-                    c->prm.bs_sm = sm;
                     c->prm.bs_S = S;
-                    c->prm.bs_epw = epw;
-                    c->prm.bs_nc = nc;
                     c->prm.bs_words = static_cast<int32_t>(ww);
                     // the default where the largest group gives at least a quarter of the
                     // resident warps an item, and a variable row has at most 16 words: with

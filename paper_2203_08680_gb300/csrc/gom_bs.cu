@@ -1,6 +1,7 @@
-// gom_bs.cu -- the kernels of the bit-sliced mixing path (gom_bs.cuh): the
-// persistent generation kernel, the per-group mixing kernel of the
-// per-generation graph, and the Forced Improvement kernels of that graph.
+// gom_bs.cu -- the bit-sliced mixing path's kernels by element class (their
+// instances are in gom_bs8.cu, gom_bs16.cu and gom_bs32.cu, so that they
+// compile in parallel) and the Forced Improvement kernels of the
+// per-generation graph.
 #include <climits>
 #include <cuda_runtime.h>
 
@@ -9,39 +10,6 @@
 #include "gom_kernels.cuh"
 
 namespace {
-
-// Persistent path on the bit-sliced phase: up to G generations in one
-// cooperative launch (bs_generations on the whole grid).  The dynamic shared
-// memory holds the block's fitness accumulators, then the warps' regions (the
-// k group keys of the order phase overlay them).
-template <int R, bool LEARN>
-__global__ void __launch_bounds__(kBsThreads, 5) k_run_bs(GomParams P, int G, int64_t target)
-{
-    extern __shared__ __align__(16) uint32_t s_dyn[];
-    __shared__ unsigned long long s_cnt[4], s_fc[4];
-    bs_generations<R, LEARN>(P, whole_grid(), P.bar, G, target, reinterpret_cast<unsigned long long *>(s_dyn),
-                             bs_warp_region(P, s_dyn), reinterpret_cast<long long *>(s_dyn), s_cnt, s_fc);
-}
-
-// Per-launch path: the mixing of the group at position t (one launch per
-// group in the per-generation CUDA graph).
-template <int R, bool LEARN>
-__global__ void __launch_bounds__(kBsThreads, 5) k_mix_bs(GomParams P, int t)
-{
-    extern __shared__ __align__(16) uint32_t s_dyn[];
-    __shared__ unsigned long long s_cnt[4], s_fc[4];
-    long long *s_f = reinterpret_cast<long long *>(s_dyn);
-    if (P.st->done) return;
-    fc_zero(s_fc);
-    acc_zero(P, s_f, s_cnt);
-    BsLane L;
-    bs_lane_zero(L);
-    uint32_t *wsm = bs_warp_region(P, s_dyn);
-    phase_mix_bs<R, LEARN>(P, whole_grid(), t, P.order[t], P.st->g, wsm, L, s_f, s_fc);
-    bs_finish_generation(P, L, s_f, s_cnt);
-    acc_flush(P, s_f, s_cnt);
-    if (LEARN) fc_flush(P, s_fc);
-}
 
 // Forced Improvement on the per-launch path (one CUDA graph per
 // generation): the elitist update of its start (one block), the start
@@ -118,16 +86,14 @@ const void *gom_fi_kernel(int which, int r)
     }
 }
 
-int gom_bs_warp_words(int sm, int nc, int w) { return bs_warp_words(sm, nc, w); }
-
-const void *gom_run_bs_kernel(int r, bool learn)
+const void *gom_run_bs_kernel(int s, int r, bool learn)
 {
-    if (learn) return r <= 12 ? (const void *)k_run_bs<12, true> : r <= 16 ? (const void *)k_run_bs<16, true> : nullptr;
-    return r <= 12 ? (const void *)k_run_bs<12, false> : r <= 16 ? (const void *)k_run_bs<16, false> : nullptr;
+    return bs_class(s) == 8 ? gom_run_bs8(r, learn) : bs_class(s) == 16 ? gom_run_bs16(r, learn) : gom_run_bs32(r, learn);
 }
 
-const void *gom_mix_bs_kernel(int r, bool learn)
+const void *gom_mix_bs_kernel(int s, int r, bool learn)
 {
-    if (learn) return r <= 12 ? (const void *)k_mix_bs<12, true> : r <= 16 ? (const void *)k_mix_bs<16, true> : nullptr;
-    return r <= 12 ? (const void *)k_mix_bs<12, false> : r <= 16 ? (const void *)k_mix_bs<16, false> : nullptr;
+    return bs_class(s) == 8 ? gom_mix_bs8(r, learn) : bs_class(s) == 16 ? gom_mix_bs16(r, learn) : gom_mix_bs32(r, learn);
 }
+
+int gom_bs_warp_words(int s) { return bs_warp_words(s); }

@@ -12,18 +12,22 @@
 // A warp takes an item of E = 32 / W elements of the colour group (W = words
 // per variable row); lane k owns the pair (element slot k / W, word k mod W),
 // i.e. 32 individuals of one element.  Per item:
-//   phase 0  (lane = pair) the parent's current rows on F_j and the
-//            generation-start rows of P on F_j into shared memory, the run
-//            starts of P's patterns on F_j, and the Philox donor starts of
-//            all 1024 trials (one Philox call per 4 individuals); then, by
-//            32 x 32 bit transposes, the patterns of P and of the parents on
-//            the item's elements packed side by side per individual
-//   phase 1  (lane = individual, one word after the other) the donor search
-//            of Sec. 4.2: one lookup of the start candidate's packed pattern
-//            and of the next run start after it, the run-start walk and the
-//            word-parallel scan for the rare rest; the packed flips (donor ^
-//            parent) go back through transposes into flip planes F_a (bit b:
-//            individual b flips variable a)
+//   phase 0  (lane = pair) the parent's current rows on F_j into shared
+//            memory, the generation-start rows of P on F_j in registers; the
+//            run starts of P's patterns (bit d: pattern d differs from pattern
+//            d - 1, cyclically); then, by a bit transpose inside the lane, the
+//            pattern P_d of each of its 32 individuals, and by one backward
+//            walk over them the pattern N_d of the next run start after d: one
+//            table entry (P_d, N_d) per individual
+//   phase 1  (lane = 4 individuals of a pair) the donor search of Sec. 4.2: one
+//            Philox call gives 4 starts; one table entry per trial holds the
+//            start's pattern and the pattern the search falls through to when
+//            the start equals the parent.  (Lane = pair) the 32 entries come
+//            back through the inverse transpose as bit-planes T1_a (the
+//            starts' bits) and T2_a (the fall-through's), and the flip planes
+//            F_a (bit b: individual b flips variable a) are a plane select;
+//            the rare individuals whose own column is the run start the
+//            search falls through to are resolved one by one
 //   phase 2  (lane = pair) the partial evaluation (Sec. 2.2, Alg. 4) as
 //            bit-plane arithmetic: an edge e that a trial toggles (t_e = F_a
 //            for an edge leaving F_j, F_a ^ F_b inside) changes the cut by
@@ -41,6 +45,11 @@
 // (gom_filter_dev.cuh) decides which elements run and lists them in order, the
 // groups run only the listed elements, and each item records its elements'
 // history and training samples.
+// What bounds it: instruction issue and the integer ALU.  Donor tables made and
+// read inside the lane took a generation of the 1000x1000 torus (p = 256) from
+// 2.27 to 1.31 ms against tables of packed patterns transposed across the warp
+// with a run-start search per trial.
+//
 // Elements of one colour group share no variable and no edge (LMIG
 // colouring), so the rows a pair reads and writes belong to it alone during
 // the group.
@@ -61,61 +70,32 @@
 
 namespace {
 
-// Four independent 32 x 32 bit-matrix transposes across the warp, interleaved
-// step by step (their shuffles and logic overlap instead of waiting on one
-// another): lane r holds row r of each matrix (bit c = entry (r, c)) on entry
-// and column r (bit c = entry (c, r)) on return.  Five steps; step j swaps
-// the off-diagonal j x j blocks of each 2j x 2j block between lanes l and
-// l ^ j, branch-free: a lane keeps its own half of each block (mask `keep`)
-// and takes the partner's other half rotated into place (left by j for the
-// lower lane of a pair, right by j for the upper one).
-__device__ __forceinline__ void transpose32x4(uint32_t (&x)[4])
+// Transposes the NR x NR bit blocks of NR registers inside the lane (NR = 8:
+// four blocks, one per byte column; 16: two; 32: one): bit NR c + r of x[a]
+// on entry is bit NR c + a of x[r] on return.  log2(NR) steps; step j swaps
+// the off-diagonal j x j blocks of each 2j x 2j block.  3 * 4 * 4 = 48
+// instructions transpose 8 variables of 32 individuals in each of 32 lanes,
+// where shuffle transposes across the warp took 15 for one word of 32
+// individuals, used 20 of 32 rows, and kept the shuffle unit busy.
+template <int NR, int J = NR / 2>
+__device__ __forceinline__ void transpose_lane(uint32_t (&x)[NR])
 {
-    const int lane = threadIdx.x & 31;
+    constexpr uint32_t m = J == 16 ? 0x0000FFFFu : J == 8 ? 0x00FF00FFu : J == 4 ? 0x0F0F0F0Fu : J == 2 ? 0x33333333u
+                                                                                                    : 0x55555555u;
 #pragma unroll
-    for (int j = 16; j; j >>= 1) {
-        const uint32_t m = j == 16 ? 0x0000FFFFu : j == 8 ? 0x00FF00FFu : j == 4 ? 0x0F0F0F0Fu : j == 2 ? 0x33333333u
-                                                                                                  : 0x55555555u;
-        const uint32_t up = 0u - (uint32_t)((lane >> (31 - __clz(j))) & 1);
-        const uint32_t keep = m ^ up;
-        const int sh = up ? 32 - j : j;
-        uint32_t y[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) y[q] = __shfl_xor_sync(0xFFFFFFFFu, x[q], j);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) x[q] = (x[q] & keep) | (__funnelshift_l(y[q], y[q], sh) & ~keep);
+    for (int r = 0; r < NR; ++r) {
+        if (r & J) continue;
+        const uint32_t a = x[r], b = x[r + J];
+        x[r] = (a & m) | ((b << J) & ~m);
+        x[r + J] = ((a >> J) & m) | (b & ~m);
     }
+    if constexpr (J > 1) transpose_lane<NR, J / 2>(x); // (a loop over J would stay a loop, with x in local memory)
 }
 
 // Brings the 128-byte line holding *ptr into L2 (a hint: no data returned).
 __device__ __forceinline__ void prefetch_l2(const void *ptr)
 {
     asm volatile("prefetch.global.L2 [%0];" ::"l"(ptr));
-}
-
-// Word-parallel donor scan over the staged rows (32 candidates per step):
-// the first individual in cyclic order from `start`, skipping `self`, whose
-// generation-start bits on F_j differ from the parent's bits xf; -1 if none.
-__device__ int scan_rows(const uint32_t *sP, int SM, int e, int W, int Wv, int p, int s, uint32_t xf, int start,
-                         int self)
-{
-    const int ws = start >> 5, bs = start & 31;
-    for (int step = 0; step <= Wv; ++step) {
-        int wc = ws + step;
-        if (wc >= Wv) wc -= Wv;
-        const uint32_t *row = sP + (e * W + wc) * SM;
-        uint32_t diff = 0;
-        for (int a = 0; a < s; ++a) diff |= row[a] ^ (0u - ((xf >> a) & 1u));
-        const int lim = p - 32 * wc;
-        uint32_t mk = diff & (lim >= 32 ? 0xFFFFFFFFu : ((1u << lim) - 1u));
-        if (wc == (self >> 5)) mk &= ~(1u << (self & 31));
-        if (step == 0)
-            mk &= 0xFFFFFFFFu << bs;
-        else if (step == Wv)
-            mk &= ~(0xFFFFFFFFu << bs);
-        if (mk) return 32 * wc + __ffs(mk) - 1;
-    }
-    return -1;
 }
 
 // First position at or after x, in cyclic order over [0, p), whose bit is set
@@ -133,58 +113,22 @@ __device__ __forceinline__ int next_run_start(const uint32_t *rs, uint32_t nz, i
     return 32 * w2 + __ffs(rs[w2]) - 1;
 }
 
-// The donor of individual `self` (Sec. 4.2): the first candidate in cyclic
-// order from `start`, skipping self, whose generation-start bits on F_j
-// differ from the parent's current bits xf, or -1.  The search resumes at
-// candidate `cur`, whose pattern is known to equal xf (start, or the one
-// after it).  Candidates' patterns come from the packed table tc of P (the
-// element's field at offset `off`); rs are the run starts of the element's
-// patterns (bit d: pattern d differs from pattern d - 1, cyclically), so the
-// candidates strictly inside a run equal to the parent are passed in one
-// step (a run start after such a run differs from xf); after a few steps the
-// word-parallel scan over the staged rows finishes the search.  *pd receives
-// the donor's pattern.  Divergent code.
-__device__ int find_donor_packed(const uint32_t *tc, int off, uint32_t fmask, const uint32_t *sP, const uint32_t *rs,
-                                 uint32_t nz, int SM, int e, int W, int Wv, int p, int s, uint32_t xf, int start,
-                                 int cur, int self, uint32_t *pd)
-{
-    int d = cur; // pattern d == xf here
-    for (int it = 0; it < 4; ++it) {
-        const int d2 = next_run_start(rs, nz, d + 1 == p ? 0 : d + 1);
-        if (d2 < 0) return -1; // one run: every candidate equals the parent
-        const int dist_d = d - start + (d < start ? p : 0);
-        const int dist_2 = d2 - start + (d2 < start ? p : 0);
-        if (dist_2 <= dist_d) return -1; // the jump passed the start
-        if (d2 != self) {
-            *pd = (tc[d2] >> off) & fmask;
-            return d2;
-        }
-        d = d2 + 1 == p ? 0 : d2 + 1; // skip the parent's own column
-        if (d == start) return -1;
-        const uint32_t pat = (tc[d] >> off) & fmask;
-        if (pat != xf) {
-            *pd = pat;
-            return d;
-        }
-    }
-    const int d3 = d + 1 == p ? 0 : d + 1;
-    if (d3 == start) return -1;
-    const int r = scan_rows(sP, SM, e, W, Wv, p, s, xf, d3, self);
-    if (r >= 0) *pd = (tc[r] >> off) & fmask;
-    return r;
-}
+// Shared-memory words of one pair's table entries, by the class SB of the
+// largest element (8, 16 or 32 variables): 32 entries of 2 bytes (P_d in the
+// low byte, N_d in the high one), 4 bytes (halves) or 8 bytes (P_d, N_d).
+__host__ __device__ constexpr int bs_entry_words(int SB) { return 2 * SB; }
 
-// Shared-memory words of one warp's region (SM = P.bs_sm, odd, so that the
-// 32 lanes reading word a of their own rows hit 32 different banks; NC
-// chunks of packed patterns): rows of O on F_j [32 pairs][SM], rows of P
-// [32][SM], flip planes [32][SM], donor starts [32 pairs][32 individuals] as
-// 16-bit values, run starts [32 pairs], packed patterns of P [NC][W][32],
-// packed patterns of O [NC][W][32] (their slots reused for the packed flips),
-// the item's element sizes [32] and the masks of their non-empty run-start
-// words [32].
-__host__ __device__ __forceinline__ int bs_warp_words(int SM, int NC, int W)
+// The class of the largest element S.
+__host__ __device__ constexpr int bs_class(int S) { return S <= 8 ? 8 : S <= 16 ? 16 : 32; }
+
+// Shared-memory words of one warp's region: the donor tables [32 pairs], the
+// trials' entries [32 pairs] (their slots reused for the flip planes
+// [S][32 pairs]), the rows of O on F_j [S][32 pairs] and the run starts [32
+// pairs].  Row arrays are variable-major: lane l reads word 32 a + l, free of
+// bank conflicts for any a.
+__host__ __device__ __forceinline__ int bs_warp_words(int S)
 {
-    return 96 * SM + 16 * 32 + 32 + 64 * NC * W + 64;
+    return 64 * bs_entry_words(bs_class(S)) + 32 * S + 32;
 }
 
 // The dynamic shared memory of the bit-sliced kernels: the block's fitness
@@ -236,16 +180,52 @@ __device__ __noinline__ void bs_record(const GomParams &P, int q, bool ke, bool 
     __syncwarp();
 }
 
+// Individual i of element j (its pairs from b2 on in the table), possibly the
+// run start its own search falls through to: its start is drawn again, and if
+// the next run start after it is not i, the result is false.  Otherwise the
+// search goes on behind i, and *fl receives the donor's flips: the donor is
+// i + 1 if its pattern differs from the parent's (xf, the pattern of the run
+// before i, which holds the start), else the first run start after i + 1 --
+// unless the element has no more than two run starts: then the run of i + 1
+// reaches round to i, everyone but i equals the parent, and there is no donor.
+template <int SB>
+__device__ __noinline__ bool self_hit(uint32_t *fl, const uint32_t *tab, const uint32_t *rs, uint32_t nz, int b2, int j,
+                                      int i, uint32_t g, int p, uint64_t seed)
+{
+    const uint4 r4 = philox10(make_uint4((uint32_t)j, (uint32_t)(i >> 2), g, kTagDonor), (uint32_t)seed,
+                              (uint32_t)(seed >> 32));
+    const uint32_t d = (uint32_t)(i + 1) + __umulhi(pick(r4, i & 3), (uint32_t)(p - 1));
+    const int st = (int)min(d, d - (uint32_t)p);
+    if (next_run_start(rs, nz, st + 1 == p ? 0 : st + 1) != i) return false;
+    const auto entry = [&](int x, uint32_t *next) -> uint32_t {
+        if constexpr (SB == 8) {
+            const uint32_t en = reinterpret_cast<const uint16_t *>(tab)[32 * b2 + x];
+            *next = en >> 8;
+            return en & 0xFFu;
+        } else {
+            const int k3 = b2 + (x >> 5), at = 32 * k3 + ((x + k3) & 31);
+            *next = SB == 16 ? tab[at] >> 16 : tab[1024 + at];
+            return SB == 16 ? tab[at] & 0xFFFFu : tab[at];
+        }
+    };
+    uint32_t unused, nn;
+    const uint32_t xf = entry(i == 0 ? p - 1 : i - 1, &unused), pn = entry(i + 1 == p ? 0 : i + 1, &nn);
+    int starts = 0;
+    for (uint32_t m = nz; m; m &= m - 1) starts += __popc(rs[__ffs(m) - 1]);
+    *fl = pn != xf ? pn ^ xf : starts == 2 ? 0u : nn ^ xf;
+    return true;
+}
+
 // One item of colour group c at position t: entries [k0, k1) (at most E) of
 // the group's elements -- positions k0 .. k1 - 1, or with the learned filter
 // skipping, the positions qlist[k0 .. k1) of the compacted list -- with every
 // word, all trials of Alg. 2.
-template <int R, bool LEARN>
+template <int SB, int R, bool LEARN>
 __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist, int k0, int k1, uint32_t g,
                                         uint32_t *wsm, BsLane &L, long long *s_f, unsigned long long *s_fc)
 {
     const int lane = threadIdx.x & 31;
-    const int W = P.W, Wv = P.Wv, p = P.p, SM = P.bs_sm;
+    const int W = P.W, Wv = P.Wv, p = P.p, S = P.bs_S;
     const int lw = __ffs(W) - 1;
     const int e = lane >> lw, w = lane & (W - 1);
     const bool ke = k0 + e < k1; // this lane's element exists
@@ -257,11 +237,14 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
         audited = en < 0;
     }
     const bool kv = ke && w < Wv; // this lane's pair exists
-    uint32_t *sO = wsm, *sP = wsm + 32 * SM, *sD = wsm + 64 * SM;
-    uint16_t *sStart = reinterpret_cast<uint16_t *>(wsm + 96 * SM); // p <= 1024: a start fits 16 bits
-    uint32_t *sRS = wsm + 96 * SM + 16 * 32;
+    constexpr int EW = bs_entry_words(SB);
+    uint32_t *tab = wsm, *res = wsm + 32 * EW;
+    uint32_t *sF = res; // flip planes, once every lane has read its entries back
+    uint32_t *sX = wsm + 64 * EW, *sRS = sX + 32 * S;
+    const int lim = p - 32 * w;
+    const uint32_t vm = lim >= 32 ? 0xFFFFFFFFu : lim > 0 ? (1u << lim) - 1u : 0u; // this word's individuals
 
-    // ---- phase 0: the pair's rows, run starts, donor starts
+    // ---- phase 0: the pair's rows, run starts, donor table
     int j = 0, s = 0, f0 = 0, d0 = 0, n_in = 0, n_out = 0;
     if (ke) {
         const int4 a = __ldg(P.hdr + 2 * q), b = __ldg(P.hdr + 2 * q + 1);
@@ -283,183 +266,253 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
             prefetch_l2(P.seg + f0 + q + s);
         }
     }
-    for (int a4 = 0; a4 < SM; a4 += 4) {
-        uint32_t xo[4], xp[4];
+    uint32_t xp[SB];
+    uint32_t chg = 0; // individuals that changed on F_j since the generation start
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            xo[c] = xp[c] = 0;
-            if (kv && a4 + c < s) {
-                const int64_t v = __ldg(P.fv + f0 + a4 + c);
-                xo[c] = P.O[v * W + w];
-                xp[c] = P.P[v * W + w];
+    for (int a = 0; a < SB; ++a) xp[a] = 0;
+#pragma unroll
+    for (int a8 = 0; a8 < SB; a8 += 8) {
+        if (a8 < S) {
+            int at[8];
+            uint32_t xo[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) at[c] = kv && a8 + c < s ? __ldg(P.fv + f0 + a8 + c) * W + w : -1;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                xo[c] = at[c] >= 0 ? P.O[at[c]] : 0u;
+                xp[a8 + c] = at[c] >= 0 ? P.P[at[c]] : 0u;
+            }
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                chg |= xo[c] ^ xp[a8 + c];
+                if (a8 + c < S) sX[32 * (a8 + c) + lane] = xo[c];
             }
         }
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-            if (a4 + c < SM) {
-                sO[lane * SM + a4 + c] = xo[c];
-                sP[lane * SM + a4 + c] = xp[c];
-            }
     }
-    __syncwarp();
+    uint32_t rs = 0, fst = 0, nz;
     {   // run starts of the element's patterns in word w: bit b set iff the
-        // pattern of individual 32 w + b differs from the one before it (cyclically)
-        uint32_t rsw = 0;
-        if (kv) {
-            const uint32_t *cur = sP + lane * SM;
-            const uint32_t *prev = sP + (e * W + (w == 0 ? Wv - 1 : w - 1)) * SM;
-            const int pb = w == 0 ? (p - 1) & 31 : 31;
-            for (int a = 0; a < s; ++a) {
-                const uint32_t x = cur[a];
-                rsw |= x ^ ((x << 1) | ((prev[a] >> pb) & 1u));
-            }
-            const int lim = p - 32 * w;
-            rsw &= lim >= 32 ? 0xFFFFFFFFu : ((1u << lim) - 1u);
-        }
-        sRS[lane] = rsw;
+        // pattern of individual 32 w + b differs from the one before it
+        // (cyclically: the word before's last individual, by a shuffle of the
+        // packed last bits); fst: the pattern at the word's first run start
+        const int lastb = lim >= 32 ? 31 : lim > 0 ? lim - 1 : 0;
+        uint32_t lst = 0;
+#pragma unroll
+        for (int a = 0; a < SB; ++a)
+            if (a < S) lst |= ((xp[a] >> lastb) & 1u) << a;
+        const uint32_t prv = __shfl_sync(kFull, lst, e * W + (w == 0 ? Wv - 1 : w - 1));
+#pragma unroll
+        for (int a = 0; a < SB; ++a)
+            if (a < S) rs |= xp[a] ^ __funnelshift_l(prv << (31 - a), xp[a], 1);
+        rs = kv ? rs & vm : 0u;
+        sRS[lane] = rs;
+        const int fb = rs ? __ffs(rs) - 1 : 0;
+#pragma unroll
+        for (int a = 0; a < SB; ++a)
+            if (a < S) fst |= ((xp[a] >> fb) & 1u) << a;
         // element e's words with a run start: bits e W .. e W + W - 1 of the ballot
-        const uint32_t nzb = __ballot_sync(0xFFFFFFFFu, rsw != 0);
-        if (w == 0)
-            wsm[96 * SM + 16 * 32 + 32 + 64 * P.bs_nc * W + 32 + e] = W == 32 ? nzb : (nzb >> (e * W)) & ((1u << W) - 1u);
+        const uint32_t nzb = __ballot_sync(kFull, rs != 0);
+        nz = W == 32 ? nzb : (nzb >> (e * W)) & ((1u << W) - 1u);
     }
-    {   // donor starts: call (pair k2, c) covers individuals 32 w2 + 4c .. + 3
-#pragma unroll 1
-        for (int r = 0; r < 8; ++r) {
-            const int k2 = 4 * r + (lane >> 3), c = lane & 7;
-            const int w2 = k2 & (W - 1);
-            const int j2 = __shfl_sync(0xFFFFFFFFu, j, k2);
-            const bool v2 = __shfl_sync(0xFFFFFFFFu, kv ? 1 : 0, k2) && 32 * w2 + 4 * c < p;
-            if (v2) {
-                const uint4 r4 = philox10_rk(make_uint4((uint32_t)j2, (uint32_t)(8 * w2 + c), g, kTagDonor), P.rk);
-                const int i0 = 32 * w2 + 4 * c;
-                int st[4];
+    // the first run start after word w (cyclically): its pattern carries into
+    // the word's last individuals; without any run start every pattern is the same
+    const uint32_t later = nz & ~((2u << w) - 1u); // words after w
+    const uint32_t any = later ? later : nz;        // else wrap round
+    uint32_t nx = __shfl_sync(kFull, fst, e * W + (any ? __ffs(any) - 1 : w));
+    {
+        uint32_t x[SB];
 #pragma unroll
-                for (int cc = 0; cc < 4; ++cc) {
-                    const int d = i0 + cc + 1 + (int)__umulhi(pick(r4, cc), (uint32_t)(p - 1));
-                    st[cc] = d >= p ? d - p : d;
+        for (int a = 0; a < SB; ++a) x[a] = xp[a];
+        transpose_lane<SB>(x); // block column c of x[r]: the pattern of individual 32 w + SB c + r
+        if (SB < 32) nx <<= 32 - SB;
+        if constexpr (SB == 8) {
+#pragma unroll
+            for (int c = 3; c >= 0; --c) {
+                uint32_t ent[4]; // two entries each
+#pragma unroll
+                for (int r = 6; r >= 0; r -= 2) {
+                    const uint32_t hi = __byte_perm(x[r + 1], nx, c | (c + 4) << 4);
+                    if ((rs >> (8 * c + r + 1)) & 1u) nx = x[r + 1];
+                    const uint32_t lo = __byte_perm(x[r], nx, c | (c + 4) << 4);
+                    if ((rs >> (8 * c + r)) & 1u) nx = x[r];
+                    ent[r / 2] = __byte_perm(lo, hi, 0x5410);
                 }
-                *reinterpret_cast<uint2 *>(sStart + k2 * 32 + 4 * c) =
-                    make_uint2((uint32_t)st[0] | ((uint32_t)st[1] << 16), (uint32_t)st[2] | ((uint32_t)st[3] << 16));
+                nx >>= 8;
+                *reinterpret_cast<uint4 *>(tab + 16 * lane + 4 * c) = make_uint4(ent[0], ent[1], ent[2], ent[3]);
             }
-        }
-    }
-    // packed patterns: for chunk c (elements c EPW .. c EPW + EPW - 1 of the
-    // item) and word w2, lane b receives the bits of individual 32 w2 + b on
-    // the chunk's elements side by side (element e_c at bit offset e_c S), by
-    // one transpose of the rows (row r = variable r mod S of element r / S);
-    // four words at a time, interleaved
-    const int S = P.bs_S, EPW = P.bs_epw, NC = P.bs_nc;
-    const int E = 32 >> lw;
-    uint32_t *tabP = wsm + 96 * SM + 16 * 32 + 32, *tabO = tabP + 32 * NC * W;
-    uint32_t *sFM = tabO; // a lane reads its entry of tabO before it writes the same entry of sFM
-    int *sS = reinterpret_cast<int *>(tabO + 32 * NC * W);
-    const uint32_t *sNZ = tabO + 32 * NC * W + 32; // per element slot: its non-empty run-start words
-    const uint32_t fmask = S >= 32 ? 0xFFFFFFFFu : ((1u << S) - 1u);
-    if (w == 0) sS[e] = s; // the item's element sizes, by slot
-    const int er = lane / S, ar = lane - er * S; // this lane's row in a transpose: element er of a chunk, variable ar
-    for (int c = 0; c < NC; ++c) {
-        const int e3 = c * EPW + er;
-        const bool row = er < EPW && e3 < E;
-        for (int w2 = 0; w2 < Wv; w2 += 4) {
-            uint32_t tp[4], to[4];
+        } else if constexpr (SB == 16) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int at = (e3 * W + w2 + j) * SM + ar;
-                const bool ok = row && w2 + j < Wv;
-                tp[j] = ok ? sP[at] : 0u;
-                to[j] = ok ? sO[at] : 0u;
-            }
-            transpose32x4(tp);
-            transpose32x4(to);
+            for (int c = 1; c >= 0; --c) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (w2 + j < Wv) {
-                    tabP[(c * W + w2 + j) * 32 + lane] = tp[j];
-                    tabO[(c * W + w2 + j) * 32 + lane] = to[j];
+                for (int r = 15; r >= 0; --r) {
+                    // word 32 lane + d rotated by the lane: 32 lanes hit 32 banks
+                    tab[32 * lane + ((16 * c + r + lane) & 31)] = __byte_perm(x[r], nx, c ? 0x7632 : 0x5410);
+                    if ((rs >> (16 * c + r)) & 1u) nx = x[r];
                 }
+                nx >>= 16;
+            }
+        } else {
+#pragma unroll
+            for (int r = 31; r >= 0; --r) {
+                const int at = 32 * lane + ((r + lane) & 31);
+                tab[at] = x[r];
+                tab[1024 + at] = nx;
+                if ((rs >> r) & 1u) nx = x[r];
+            }
         }
     }
     __syncwarp();
 
-    // ---- phase 1: donors, lane = individual.  Pass A checks every pair's
-    // start candidate (one table lookup) and, when it equals the parent on
-    // F_j, takes the first run start after it (one more); pass B searches
-    // again from the start for the rare individuals whose run start is their
-    // own column (run starts, then the word-parallel scan).  Each word's
-    // flips of a chunk are packed like the patterns into sFM.
-    for (int w2 = 0; w2 < Wv; ++w2) {
-        const int i = 32 * w2 + lane;
-        const bool vi = i < p;
-        for (int c = 0; c < NC; ++c) {
-            const uint32_t xo = tabO[(c * W + w2) * 32 + lane]; // the parents' current patterns
-            const int ne = min(EPW, min(E, k1 - k0) - c * EPW); // elements of this chunk in the item
-            const uint32_t *tc = tabP + c * W * 32;             // chunk c's patterns, by individual
-            const uint16_t *sc = sStart + (c * EPW * W + w2) * 32 + lane;
-            uint32_t fmw = 0, fails = 0;
-#pragma unroll 4
-            for (int el = 0; el < ne; ++el) {
-                const int e2 = c * EPW + el;
-                // the element's field of the packed words: its flips are (donor ^ parent) & field
-                const uint32_t field = fmask << (el * S);
-                // starts exist for individuals < p only (others read candidate 0, and are dropped below)
-                const int st = vi ? sc[el * W * 32] : 0;
-                // every candidate from st up to the next run start d2 has st's pattern; when
-                // that is the parent's, d2 differs from it and is the donor -- unless it is
-                // the parent's own column (pass B); no run start: no donor.  d2 is found
-                // whatever st's pattern (branch-free, all loads issued together)
-                const int x = st + 1 == p ? 0 : st + 1, wx = x >> 5;
-                const uint32_t *rs = sRS + e2 * W;
-                const uint32_t nzm = sNZ[e2];
-                const uint32_t later = nzm & ~((2u << wx) - 1u); // run-start words after wx
-                const uint32_t any = later ? later : nzm;          // else wrap round
-                const int wy = any ? __ffs(any) - 1 : 0;
-                const uint32_t t1 = tc[st], r1 = rs[wx], r2 = rs[wy];
-                const uint32_t m = r1 & (0xFFFFFFFFu << (x & 31));
-                const int d2 = m ? 32 * wx + __ffs(m) - 1 : any ? 32 * wy + __ffs(r2) - 1 : -1;
-                const uint32_t t2 = tc[d2 < 0 ? 0 : d2];
-                const uint32_t f1 = (t1 ^ xo) & field;
-                const uint32_t f2 = d2 >= 0 && d2 != i ? (t2 ^ xo) & field : 0u;
-                fmw |= f1 ? f1 : f2;
-                fails |= !f1 && d2 == i ? 1u << el : 0u;
+    // ---- phase 1: donors.  Call (pair k2, c) covers individuals 32 w2 + 4c ..
+    // + 3; the starts of individuals past p (in the last word's last call)
+    // stay below 32 Wv, inside the element's table
+#pragma unroll 1
+    for (int r = 0; r < 8; ++r) {
+        const int k2 = 4 * r + (lane >> 3), c = lane & 7;
+        const int w2 = k2 & (W - 1), b2 = k2 - w2; // b2: the element's first pair
+        const int j2 = __shfl_sync(kFull, j, k2);
+        if (__shfl_sync(kFull, kv ? 1 : 0, k2)) {
+            const uint4 r4 = philox10_rk(make_uint4((uint32_t)j2, (uint32_t)(8 * w2 + c), g, kTagDonor), P.rk);
+            const int i0 = 32 * w2 + 4 * c;
+            uint32_t en[4], en2[4];
+    #pragma unroll
+            for (int cc = 0; cc < 4; ++cc) {
+                const uint32_t d = (uint32_t)(i0 + cc + 1) + __umulhi(pick(r4, cc), (uint32_t)(p - 1));
+                const uint32_t st = min(d, d - (uint32_t)p); // d < p: d - p wraps above d
+                if constexpr (SB == 8) {
+                    en[cc] = reinterpret_cast<const uint16_t *>(tab)[32 * b2 + st];
+                } else {
+                    const uint32_t k3 = (uint32_t)b2 + (st >> 5), at = 32 * k3 + ((st + k3) & 31);
+                    en[cc] = tab[at];
+                    if constexpr (SB == 32) en2[cc] = tab[1024 + at];
+                }
             }
-            if (!vi) fmw = fails = 0;
-            for (uint32_t f = fails; f; f &= f - 1) { // pass B, divergent
-                const int el = __ffs(f) - 1, off = el * S, e2 = c * EPW + el;
-                const uint32_t xf = (xo >> off) & fmask;
-                const int st = sStart[(e2 * W + w2) * 32 + lane];
-                uint32_t pd = 0;
-                const int d = find_donor_packed(tabP + c * W * 32, off, fmask, sP, sRS + e2 * W, sNZ[e2], SM, e2, W, Wv, p,
-                                                sS[e2], xf, st, st, i, &pd);
-                if (d >= 0) fmw |= (pd ^ xf) << off;
+            if constexpr (SB == 8) {
+                *reinterpret_cast<uint2 *>(res + 16 * k2 + (((c >> 1) ^ ((k2 >> 1) & 3)) << 2) + ((c & 1) << 1)) =
+                    make_uint2(__byte_perm(en[0], en[1], 0x5410), __byte_perm(en[2], en[3], 0x5410));
+            } else {
+                uint32_t *at = res + 32 * k2 + ((c ^ (k2 & 7)) << 2);
+                *reinterpret_cast<uint4 *>(at) = make_uint4(en[0], en[1], en[2], en[3]);
+                if constexpr (SB == 32) *reinterpret_cast<uint4 *>(at + 1024) = make_uint4(en2[0], en2[1], en2[2], en2[3]);
             }
-            sFM[(c * W + w2) * 32 + lane] = fmw;
         }
     }
     __syncwarp();
-    // the flip planes: lane r of the transpose of a word's packed flips gets
-    // variable r mod S of element r / S of the chunk (bit b: individual 32 w2 + b
-    // flips it); four words at a time
-    for (int c = 0; c < NC; ++c) {
-        const int e3 = c * EPW + er;
-        const bool row = er < EPW && e3 < E;
-        for (int w2 = 0; w2 < Wv; w2 += 4) {
-            uint32_t tf[4];
+
+    // the entries back as planes: t1[a] the starts' bits, then t2[a] the
+    // fall-through patterns' bits; f1: the individuals whose start differs
+    uint32_t F[SB];
+    uint32_t f1 = 0, same = kFull; // same: the fall-through pattern is the individual's own in P
+    {
+        uint32_t t2[SB];
+        if constexpr (SB == 8) {
+            const int sw = (lane >> 1) & 3;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) tf[j] = w2 + j < Wv ? sFM[(c * W + w2 + j) * 32 + lane] : 0u;
-            transpose32x4(tf);
+            for (int h = 0; h < 2; ++h) { // chunk i holds individuals 8 i .. 8 i + 7; half h of each
+                uint32_t A[4][2];          // [i][k]: individuals 8 i + 4 h + 2 k, + 1
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (row && w2 + j < Wv) sD[(e3 * W + w2 + j) * SM + ar] = tf[j];
+                for (int i = 0; i < 4; ++i) {
+                    const uint2 v = *reinterpret_cast<const uint2 *>(res + 16 * lane + ((i ^ sw) << 2) + 2 * h);
+                    A[i][0] = v.x;
+                    A[i][1] = v.y;
+                }
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    const int r = 4 * h + 2 * k;
+                    const uint32_t l0 = __byte_perm(A[0][k], A[1][k], 0x5140), h0 = __byte_perm(A[0][k], A[1][k], 0x7362);
+                    const uint32_t l1 = __byte_perm(A[2][k], A[3][k], 0x5140), h1 = __byte_perm(A[2][k], A[3][k], 0x7362);
+                    F[r] = __byte_perm(l0, l1, 0x5410);
+                    t2[r] = __byte_perm(l0, l1, 0x7632);
+                    F[r + 1] = __byte_perm(h0, h1, 0x5410);
+                    t2[r + 1] = __byte_perm(h0, h1, 0x7632);
+                }
+            }
+            transpose_lane<SB>(F);
+            transpose_lane<SB>(t2);
+        } else if constexpr (SB == 16) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { // individuals 4 i .. + 3 and 16 + 4 i .. + 3
+                const uint4 u = *reinterpret_cast<const uint4 *>(res + 32 * lane + ((i ^ (lane & 7)) << 2));
+                const uint4 v = *reinterpret_cast<const uint4 *>(res + 32 * lane + (((i + 4) ^ (lane & 7)) << 2));
+                F[4 * i] = __byte_perm(u.x, v.x, 0x5410);
+                F[4 * i + 1] = __byte_perm(u.y, v.y, 0x5410);
+                F[4 * i + 2] = __byte_perm(u.z, v.z, 0x5410);
+                F[4 * i + 3] = __byte_perm(u.w, v.w, 0x5410);
+                t2[4 * i] = __byte_perm(u.x, v.x, 0x7632);
+                t2[4 * i + 1] = __byte_perm(u.y, v.y, 0x7632);
+                t2[4 * i + 2] = __byte_perm(u.z, v.z, 0x7632);
+                t2[4 * i + 3] = __byte_perm(u.w, v.w, 0x7632);
+            }
+            transpose_lane<SB>(F);
+            transpose_lane<SB>(t2);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint4 u = *reinterpret_cast<const uint4 *>(res + 32 * lane + ((i ^ (lane & 7)) << 2));
+                F[4 * i] = u.x;
+                F[4 * i + 1] = u.y;
+                F[4 * i + 2] = u.z;
+                F[4 * i + 3] = u.w;
+            }
+            transpose_lane<SB>(F);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint4 u = *reinterpret_cast<const uint4 *>(res + 1024 + 32 * lane + ((i ^ (lane & 7)) << 2));
+                t2[4 * i] = u.x;
+                t2[4 * i + 1] = u.y;
+                t2[4 * i + 2] = u.z;
+                t2[4 * i + 3] = u.w;
+            }
+            transpose_lane<SB>(t2);
+        }
+#pragma unroll
+        for (int a = 0; a < SB; ++a)
+            if (a < S) f1 |= F[a] ^ sX[32 * a + lane];
+        if (SB < 32) { // (the widest class keeps no copy of P's rows: more individuals are looked at below)
+#pragma unroll
+            for (int a = 0; a < SB; ++a)
+                if (a < S) same &= ~(t2[a] ^ xp[a]);
+        }
+        // every candidate from the start up to the next run start has the
+        // start's pattern; when that is the parent's, the run start differs
+        // and is the donor, with no run start at all the entry repeats P_d:
+        // no flips, no donor
+#pragma unroll
+        for (int a = 0; a < SB; ++a)
+            if (a < S) F[a] = ((f1 & F[a]) | (~f1 & t2[a])) ^ sX[32 * a + lane];
+    }
+    __syncwarp(); // every lane has read its entries: their slots take the flip planes
+    uint32_t hd = 0; // individuals with a donor
+#pragma unroll
+    for (int a = 0; a < SB; ++a)
+        if (a < S) {
+            const uint32_t Fa = kv ? F[a] & vm : 0u;
+            hd |= Fa;
+            sF[32 * a + lane] = Fa;
+        }
+    // An individual that is itself the run start the search falls through to
+    // is skipped (a donor is another individual).  Only one that changed in
+    // this generation can be: one that did not has the pattern of its run,
+    // and the run before it has another.
+    uint32_t cand = kv ? ~f1 & rs & chg & same : 0u;
+    while (cand) { // divergent, rare
+        const int b = __ffs(cand) - 1, i = 32 * w + b;
+        cand &= cand - 1;
+        uint32_t fl;
+        if (!self_hit<SB>(&fl, tab, sRS + e * W, nz, e * W, j, i, g, p, P.seed)) continue;
+        hd = (hd & ~(1u << b)) | ((fl ? 1u : 0u) << b);
+        for (int a = 0; a < s; ++a) {
+            uint32_t *row = sF + 32 * a + lane;
+            *row = (*row & ~(1u << b)) | (((fl >> a) & 1u) << b);
         }
     }
-    __syncwarp();
+    __syncwarp(); // (the tables are read above)
 
     // ---- phase 2: bit-plane partial evaluation, acceptance, write, lane = pair
     unsigned i_acc = 0, i_dl = 0, i_imp = 0; // this pair's accepted, donor-less and improving trials
     // each item adds less than 2^R to an individual's sum: flush before it could pass 2^kFitPlanes
     if (L.since_flush >= (1 << (kFitPlanes - R))) bs_flush(P, L, s_f);
     if (kv) {
-        const uint32_t *myD = sD + lane * SM, *myO = sO + lane * SM;
+        const uint32_t *myD = sF + lane, *myO = sX + lane; // variable a at word 32 a
         // the delta of every trial, R + 1 planes two's complement: an edge that
         // a trial toggles adds |w| if it was uncut (with its sign folded into
         // the cut bit), -|w| if it was cut (Eq. 1); no partial sum leaves
@@ -467,12 +520,10 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
         uint32_t D[R + 1];
 #pragma unroll
         for (int t = 0; t <= R; ++t) D[t] = 0;
-        uint32_t hd = 0;
         for (int a = 0; a < s; ++a) {
-            const uint32_t Fa = myD[a];
-            hd |= Fa;
+            const uint32_t Fa = myD[32 * a];
             if (!Fa) continue; // no trial flips variable a: none of its edges changes
-            const uint32_t Xa = myO[a];
+            const uint32_t Xa = myO[32 * a];
             const int xb = (int)__ldg(P.seg + f0 + q + a), xe = (int)__ldg(P.seg + f0 + q + a + 1);
             for (int x = xb; x < xe; x += 4) { // four edges' loads issued before their arithmetic
                 int2 ed[4];
@@ -493,9 +544,9 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
         for (int x = n_out; x < n_out + n_in; ++x) {
             const int2 ed = __ldg(P.dep + d0 + x);
             const int a = ed.x & 0xFF, b = ed.x >> 8;
-            const uint32_t tg = myD[a] ^ myD[b];
+            const uint32_t tg = myD[32 * a] ^ myD[32 * b];
             if (!tg) continue; // the edge toggles for no individual
-            const uint32_t cut = myO[a] ^ myO[b] ^ (uint32_t)(ed.y >> 31);
+            const uint32_t cut = myO[32 * a] ^ myO[32 * b] ^ (uint32_t)(ed.y >> 31);
             add_signed<R + 1, kWeightBits>(D, tg & ~cut, tg & cut, (uint32_t)(ed.y < 0 ? -ed.y : ed.y));
         }
         uint32_t nz = 0;
@@ -503,8 +554,6 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
         for (int t = 0; t <= R; ++t) nz |= D[t];
         const uint32_t neg = D[R];
         const uint32_t pos = nz & ~neg;
-        const int lim = p - 32 * w;
-        const uint32_t vm = lim >= 32 ? 0xFFFFFFFFu : ((1u << lim) - 1u);
         const uint32_t eqv = P.eqw[(g & 1) * W + w];
         const uint32_t acc = hd & vm & (pos | (~nz & ~eqv));
         i_acc = __popc(acc);
@@ -516,10 +565,10 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
         if (P.fi.on && acc) atomicOr(&P.fi.accw[w], acc); // Forced Improvement: who had an accepted step
         if (acc) {
             for (int a = 0; a < s; ++a) {
-                const uint32_t m = myD[a] & acc;
+                const uint32_t m = myD[32 * a] & acc;
                 if (m) {
                     const int64_t v = __ldg(P.fv + f0 + a);
-                    P.O[v * W + w] = myO[a] ^ m;
+                    P.O[v * W + w] = myO[32 * a] ^ m;
                 }
             }
             fit_add<R>(L, D, acc); // the accepted deltas (>= 0, below 2^R)
@@ -535,8 +584,8 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
 // elements to run while the learned filter skips elements; warp x takes item
 // x, then items nwarps + the claims it draws from work[t] (P.dyn), one ahead,
 // or x + nwarps, x + 2 nwarps, ... (static stride).
-template <int R, bool LEARN>
-__device__ void phase_mix_bs(const GomParams &P, const VGrid &V, int t, int c, uint32_t g, uint32_t *wsm, BsLane &L,
+template <int SB, int R, bool LEARN>
+__device__ __forceinline__ void phase_mix_bs(const GomParams &P, const VGrid &V, int t, int c, uint32_t g, uint32_t *wsm, BsLane &L,
                              long long *s_f, unsigned long long *s_fc)
 {
     const int lane = threadIdx.x & 31;
@@ -550,7 +599,7 @@ __device__ void phase_mix_bs(const GomParams &P, const VGrid &V, int t, int c, u
     if (P.dyn && lane == 0) claim = atomicAdd(&P.work[t], 1u);
     for (int it = gwarp, next = gwarp + nwarps; it < items;) {
         const int k0 = ka + it * E;
-        bs_item<R, LEARN>(P, qlist, k0, min(k0 + E, kz), g, wsm, L, s_f, s_fc);
+        bs_item<SB, R, LEARN>(P, qlist, k0, min(k0 + E, kz), g, wsm, L, s_f, s_fc);
         if (P.dyn) {
             it = nwarps + (int)__shfl_sync(0xFFFFFFFFu, claim, 0);
             if (it < items && lane == 0) claim = atomicAdd(&P.work[t], 1u);
@@ -580,7 +629,7 @@ __device__ __forceinline__ void bs_finish_generation(const GomParams &P, BsLane 
 // are set up after it); wsm: this warp's region; s_f, s_cnt: the block's
 // fitness accumulators and counters; s_fc: the learned filter's block
 // counters (LEARN only).
-template <int R, bool LEARN>
+template <int SB, int R, bool LEARN>
 __device__ __forceinline__ void bs_generations(const GomParams &P, const VGrid &V, GomBarrier *bar, int G,
                                                int64_t target, unsigned long long *s_keys, uint32_t *wsm,
                                                long long *s_f, unsigned long long *s_cnt, unsigned long long *s_fc)
@@ -613,7 +662,7 @@ __device__ __forceinline__ void bs_generations(const GomParams &P, const VGrid &
         for (int t = 0; t < P.k; ++t) {
             if (t > 0 && !grid_barrier(&bar->count, &P.st->err, nblk, bnext, kBarrierNs)) return;
             if (tr) P.trace[4 + 2 * t] = global_ns();
-            phase_mix_bs<R, LEARN>(P, V, t, P.order[t], g, wsm, L, s_f, s_fc);
+            phase_mix_bs<SB, R, LEARN>(P, V, t, P.order[t], g, wsm, L, s_f, s_fc);
             if (tr) P.trace[5 + 2 * t] = global_ns();
         }
         bs_finish_generation(P, L, s_f, s_cnt);

@@ -210,11 +210,7 @@ struct GomParams {
                         //   regions of warps 0, 1, ... following each other from off_xw
     int32_t learn;      // learned filter: 0 off, 1 history and training log, 2 also skip elements
     GomFI fi;
-    int32_t bs_sm;      // bit-sliced path: words per staged row block of one pair (>= the largest
-                        //   element, odd: a lane-strided row access is free of bank conflicts)
-    int32_t bs_S;       //   field width of one element in a packed pattern (the largest element)
-    int32_t bs_epw;     //   elements per packed pattern word (32 / bs_S)
-    int32_t bs_nc;      //   packed words per individual for one item (ceil(E / bs_epw), E = 32 / W)
+    int32_t bs_S;       // bit-sliced path: variables of the largest element
     int32_t bs_words;   //   shared-memory words of one warp's region
     GomFilter flt;
     uint64_t seed;

@@ -1010,11 +1010,11 @@ __device__ __noinline__ void batch_variant(const GomParams &P, const VGrid V, Go
 // The bit-sliced variant of the batched path: the instance's generations on
 // the bit-sliced phase (gom_bs.cuh), warp w of the block in the w-th region
 // of P.bs_words words after the fitness accumulators.
-template <int R>
+template <int SB, int R>
 __device__ __noinline__ void batch_variant_bs(const GomParams &P, const VGrid V, GomBarrier *bar, int G,
                                               int64_t target, const RunShared &S)
 {
-    bs_generations<R, false>(P, V, bar, G, target, reinterpret_cast<unsigned long long *>(S.dyn),
+    bs_generations<SB, R, false>(P, V, bar, G, target, reinterpret_cast<unsigned long long *>(S.dyn),
                              S.dyn + (threadIdx.x >> 5) * P.bs_words, S.f, S.cnt, nullptr);
 }
 
@@ -1059,10 +1059,17 @@ __global__ void __launch_bounds__(kMixThreads, MINB)
     G = min(G, I.gens);
     if (MINB == 2 && I.variant == kVarBits) { // the bit-sliced phase needs the larger register budget
         if constexpr (MINB == 2) {
-            if (I.bs_r <= 12)
-                batch_variant_bs<12>(sP, V, bar, G, I.target, S);
+            const int cls = bs_class(sP.bs_S);
+            if (cls == 8 && I.bs_r <= 12)
+                batch_variant_bs<8, 12>(sP, V, bar, G, I.target, S);
+            else if (cls == 8)
+                batch_variant_bs<8, 16>(sP, V, bar, G, I.target, S);
+            else if (cls == 16 && I.bs_r <= 12)
+                batch_variant_bs<16, 12>(sP, V, bar, G, I.target, S);
+            else if (cls == 16)
+                batch_variant_bs<16, 16>(sP, V, bar, G, I.target, S);
             else
-                batch_variant_bs<16>(sP, V, bar, G, I.target, S);
+                batch_variant_bs<32, 16>(sP, V, bar, G, I.target, S); // (R = 12 runs in 16 planes as well)
         }
     } else if (I.variant == kVarNarrow || I.variant == kVarBits) {
         if (I.wpi == 4)

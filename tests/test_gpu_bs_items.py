@@ -1,0 +1,50 @@
+"""The bit-sliced mixing against the CPU oracle at the sizes where its donor
+tables can go wrong: largest elements at the edges of the element classes (8,
+16 and 32 variables), population words filled by one individual or all, and
+populations of few distinct rows (long runs of equal patterns, searches that
+fall through to the parent's own column)."""
+import numpy as np
+import pytest
+
+from paper_2203_08680_gb300 import gom
+from paper_2203_08680_gb300 import instances as I
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from test_gpu_parity import _assert_same_state, _assert_same_stats, _gpu_state  # noqa: E402
+
+
+def _windows(n, s):
+    """Singletons and windows of 2 .. s consecutive variables (mixed sizes, overlapping)."""
+    sets = [[v] for v in range(n)]
+    sets += [list(range(v, min(n, v + 1 + (v // s) % s))) for v in range(0, n, s)]
+    sets += [list(range(v, v + s)) for v in range(0, n - s + 1, 2 * s)]
+    return np.cumsum([0] + [len(x) for x in sets]).astype(np.int64), np.concatenate(sets).astype(np.int32)
+
+
+@pytest.mark.parametrize("s,p", [(1, 2), (1, 33), (5, 32), (8, 3), (8, 257), (9, 31), (9, 64), (16, 100), (16, 512),
+                                 (17, 65), (32, 40), (32, 1024)])
+@pytest.mark.parametrize("rows", [0, 3])
+def test_bit_sliced_items(oracle, s, p, rows):
+    """`rows` distinct rows in the population (0: random), six generations, every one compared."""
+    g = I.torus2d(9, seed=s + p, wmin=-20, wmax=100)
+    ep, ev = _windows(g.n, s)
+    P = gom.Population(g, p, 7, fos=gom.gom_fos_create(g.n, ep, ev), bitsliced=True)
+    k, co = oracle.color(g, ep, ev)
+    run = oracle.Run(g, ep, ev, co, k, p, 7)
+    if rows:
+        rng = np.random.default_rng(s * 1000 + p)
+        base = rng.integers(0, 2, (rows, g.n), dtype=np.uint8)
+        pop = base[rng.integers(0, rows, p)]
+        f = np.array([oracle.cut_value(g, x) for x in pop], dtype=np.int64)
+        best = int(f.argmax())
+        P.set_population(torch.from_numpy(pop).cuda(), torch.from_numpy(pop[best]).cuda(), int(f[best]), 0)
+        run.load(pop, f, pop[best], int(f[best]), 0)
+    for gen in range(6):
+        stats, _ = P.generation(1)
+        _assert_same_stats(stats[0], run.generation())
+        _assert_same_state(_gpu_state(P), run.get(), f"generation {gen}")
