@@ -32,7 +32,7 @@ int words_for(int32_t p)
 struct Layout {
     size_t O, P, f, eqw, xe, st, bar, trace, stats, order, work;
     size_t fi_accw, fi_eq, fi_act0, fi_imp, fi_stale, fi_f0;
-    size_t row_ptr, col, wgt, hdr, fv, wout, wabs, seg, dep, cptr;
+    size_t row_ptr, col, wgt, hdr, fv, wout, wabs, seg, dep, bdep, cptr;
     size_t total;
 };
 
@@ -73,6 +73,7 @@ Layout make_layout(int64_t n, int32_t p, int64_t nadj, int64_t m, int64_t total_
     L.wabs = take(sizeof(int32_t) * total_vars);
     L.seg = take(sizeof(uint32_t) * (total_vars + m));
     L.dep = take(sizeof(int32_t) * 2 * ndeps);
+    L.bdep = take(sizeof(int32_t) * 2 * ndeps);
     L.cptr = take(sizeof(int32_t) * (std::max<int32_t>(k, 0) + 1));
     L.total = off;
     return L;
@@ -637,6 +638,7 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
     P.wabs = reinterpret_cast<const int32_t *>(base + L.wabs);
     P.seg = reinterpret_cast<const uint32_t *>(base + L.seg);
     P.dep = reinterpret_cast<const int2 *>(base + L.dep);
+    P.bdep = reinterpret_cast<const int2 *>(base + L.bdep);
     P.cptr = reinterpret_cast<const int32_t *>(base + L.cptr);
 
     // uploads (host vectors outlive the copies: the stream is synchronised below)
@@ -654,6 +656,10 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
     GOM_CUDA(c, upload(base, L.dep, tabs.dep, s));
     GOM_CUDA(c, upload(base, L.cptr, cptr32, s));
 
+    if (c->bs_ok) {
+        k_bs_edges<<<c->grid_io, 256, 0, s>>>(P, reinterpret_cast<int2 *>(base + L.bdep));
+        GOM_CUDA(c, cudaGetLastError());
+    }
     k_init_pop<<<c->grid_io, 256, 0, s>>>(P);
     GOM_CUDA(c, cudaGetLastError());
     k_fitness<<<c->grid_fit, 256, 0, s>>>(P, P.f);

@@ -61,6 +61,54 @@ __device__ __forceinline__ void add_signed(uint32_t (&D)[NP], uint32_t pos, uint
     }
 }
 
+// An edge of the bit-sliced path's lists (GomParams::bdep): x = the far end's
+// word offset v W in O (an edge leaving the element) or its row 32 b (inside);
+// y = the weight's sign in bit 31, |w| from bit kEdgeWeight on and the near
+// end's row 32 a from bit kEdgeRow on.
+constexpr int kEdgeRow = 0;     // 32 a: bits 5 .. 9
+constexpr int kEdgeWeight = 10; // |w|: bits 10 .. 30
+
+// D += the sum over four edges of |w| pos - |w| neg, as add_signed would: the
+// edges in two pairs on UB + 2 planes each, the pairs' sum on UB + 3, and one
+// chain over all NP planes; the four carries of one that complements need
+// (neg) go into the four chains.  148 logic instructions for UB = 8, NP = 13,
+// against 4 x 42 for four chains over all planes.
+template <int NP, int UB>
+__device__ __forceinline__ void add_signed4(uint32_t (&D)[NP], const uint32_t (&pos)[4], const uint32_t (&neg)[4],
+                                            const int2 (&ed)[4])
+{
+    static_assert(NP >= UB + 3, "accumulator narrower than the sum of four edges");
+    uint32_t A[2][UB + 2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t n0 = neg[2 * h], n1 = neg[2 * h + 1];
+        uint32_t carry = n0;
+#pragma unroll
+        for (int t = 0; t < UB + 2; ++t) {
+            const bool w0 = (ed[2 * h].y & (1 << (kEdgeWeight + (t < UB ? t : 0)))) != 0;
+            const bool w1 = (ed[2 * h + 1].y & (1 << (kEdgeWeight + (t < UB ? t : 0)))) != 0;
+            const uint32_t i0 = t < UB && w0 ? pos[2 * h] : n0, i1 = t < UB && w1 ? pos[2 * h + 1] : n1;
+            A[h][t] = i0 ^ i1 ^ carry;
+            carry = (i0 & i1) | (i0 & carry) | (i1 & carry);
+        }
+    }
+    uint32_t S[UB + 3];
+    uint32_t carry = neg[1];
+#pragma unroll
+    for (int t = 0; t < UB + 3; ++t) {
+        const uint32_t a = A[0][t < UB + 2 ? t : UB + 1], b = A[1][t < UB + 2 ? t : UB + 1];
+        S[t] = a ^ b ^ carry;
+        carry = (a & b) | (a & carry) | (b & carry);
+    }
+    carry = neg[3];
+#pragma unroll
+    for (int t = 0; t < NP; ++t) {
+        const uint32_t a = D[t], b = S[t < UB + 3 ? t : UB + 2];
+        D[t] = a ^ b ^ carry;
+        carry = (a & b) | (a & carry) | (b & carry);
+    }
+}
+
 // Per-lane state of the bit-sliced path across the groups of a generation.
 struct BsLane {
     uint32_t fit[kFitPlanes]; // accepted deltas of this lane's 32 individuals (word lane mod W), bit-sliced

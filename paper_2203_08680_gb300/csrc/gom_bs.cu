@@ -76,6 +76,29 @@ __global__ void k_fi_finish(GomParams P)
 
 } // namespace
 
+// One thread per element position: its outside edges, grouped by the near end
+// a (segments of P.seg), then its inside edges.
+__global__ void k_bs_edges(GomParams P, int2 *bdep)
+{
+    for (int64_t q = gthread(); q < P.m; q += gthreads()) {
+        const int4 h0 = P.hdr[2 * q], h1 = P.hdr[2 * q + 1];
+        const int f0 = h0.y, d0 = h0.z, s = h0.w & 0xFF, n_in = h0.w >> 8, n_out = h1.x;
+        const auto pack = [](int a, int w) { // |w| <= 255 where the path is available
+            const uint32_t mag = (uint32_t)(w < 0 ? -w : w);
+            return (int)((uint32_t)(32 * a) << kEdgeRow | mag << kEdgeWeight | (w < 0 ? 0x80000000u : 0u));
+        };
+        for (int a = 0; a < s; ++a)
+            for (uint32_t x = P.seg[f0 + q + a]; x < P.seg[f0 + q + a + 1]; ++x) {
+                const int2 e = P.dep[d0 + x];
+                bdep[d0 + x] = make_int2(e.x * P.W, pack(a, e.y));
+            }
+        for (int x = n_out; x < n_out + n_in; ++x) {
+            const int2 e = P.dep[d0 + x];
+            bdep[d0 + x] = make_int2(32 * (e.x >> 8), pack(e.x & 0xFF, e.y));
+        }
+    }
+}
+
 const void *gom_fi_kernel(int which, int r)
 {
     switch (which) {

@@ -34,8 +34,9 @@
 //            +|w_e| if it was uncut and -|w_e| if it was cut (its cut plane
 //            c_e taken with the weight's sign folded in), so
 //              delta = sum_e |w_e| (t_e & ~c_e) - |w_e| (t_e & c_e),
-//            one signed ripple-carry chain per edge on R + 1 two's-complement
-//            planes (each edge counted once); then the accept plane (Alg. 2:
+//            four edges at a time in signed ripple-carry chains on as many
+//            two's-complement planes as their partial sums need, R + 1 for the
+//            total (each edge counted once); then the accept plane (Alg. 2:
 //            delta > 0, or delta = 0 and not the elitist), counters by
 //            popcount, the accepted flips XORed into the rows, and the
 //            accepted deltas into a bit-sliced per-lane fitness accumulator,
@@ -48,7 +49,9 @@
 // What bounds it: instruction issue and the integer ALU.  Donor tables made and
 // read inside the lane took a generation of the 1000x1000 torus (p = 256) from
 // 2.27 to 1.31 ms against tables of packed patterns transposed across the warp
-// with a run-start search per trial.
+// with a run-start search per trial; one flat edge list per element and chains
+// over four edges took it to 1.10 ms (103 warp instructions per 32 trials, the
+// ALU pipe busy 65 % of the cycles).
 //
 // Elements of one colour group share no variable and no edge (LMIG
 // colouring), so the rows a pair reads and writes belong to it alone during
@@ -254,17 +257,13 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
         s = a.w & 0xFF;
         n_in = a.w >> 8;
         n_out = b.x;
-        // the element's edge list and segment offsets are read in phase 2:
-        // ask for their lines in L2 now (the W lanes of the element take every
-        // W-th line; the arrays start on 256-byte boundaries, so every line
-        // named here holds bytes of the array)
-        const uintptr_t d_at = reinterpret_cast<uintptr_t>(P.dep + d0), d_end = d_at + 8u * (uint32_t)(n_out + n_in);
+        // the element's edge list is read in phase 2: ask for its lines in L2
+        // now (the W lanes of the element take every W-th line; the array
+        // starts on a 256-byte boundary, so every line named here holds bytes
+        // of it)
+        const uintptr_t d_at = reinterpret_cast<uintptr_t>(P.bdep + d0), d_end = d_at + 8u * (uint32_t)(n_out + n_in);
         for (uintptr_t at = (d_at & ~uintptr_t(127)) + 128u * (uint32_t)w; at < d_end; at += 128u * (uint32_t)W)
             prefetch_l2(reinterpret_cast<const void *>(at));
-        if (w == 0) {
-            prefetch_l2(P.seg + f0 + q);
-            prefetch_l2(P.seg + f0 + q + s);
-        }
     }
     uint32_t xp[SB];
     uint32_t chg = 0; // individuals that changed on F_j since the generation start
@@ -520,34 +519,25 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
         uint32_t D[R + 1];
 #pragma unroll
         for (int t = 0; t <= R; ++t) D[t] = 0;
-        for (int a = 0; a < s; ++a) {
-            const uint32_t Fa = myD[32 * a];
-            if (!Fa) continue; // no trial flips variable a: none of its edges changes
-            const uint32_t Xa = myO[32 * a];
-            const int xb = (int)__ldg(P.seg + f0 + q + a), xe = (int)__ldg(P.seg + f0 + q + a + 1);
-            for (int x = xb; x < xe; x += 4) { // four edges' loads issued before their arithmetic
-                int2 ed[4];
-                uint32_t Xv[4];
+        const int ne = n_out + n_in;
+        for (int x = 0; x < ne; x += 4) { // four edges' loads issued before their arithmetic
+            int2 ed[4];
+            uint32_t pos[4], neg[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) ed[u] = x + u < xe ? __ldg(P.dep + d0 + x + u) : make_int2(0, 0);
+            for (int u = 0; u < 4; ++u) ed[u] = x + u < ne ? __ldg(P.bdep + d0 + x + u) : make_int2(0, 0); // weight 0
 #pragma unroll
-                for (int u = 0; u < 4; ++u) Xv[u] = x + u < xe ? P.O[(int64_t)ed[u].x * W + w] : 0u;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    // an outgoing edge toggles wherever a flips
-                    const uint32_t cut = Xa ^ Xv[u] ^ (uint32_t)(ed[u].y >> 31);
-                    if (x + u < xe)
-                        add_signed<R + 1, kWeightBits>(D, Fa & ~cut, Fa & cut, (uint32_t)(ed[u].y < 0 ? -ed[u].y : ed[u].y));
-                }
+            for (int u = 0; u < 4; ++u) { // the far end's word, and whether a trial flips it too
+                neg[u] = x + u < n_out ? P.O[ed[u].x + w] : myO[ed[u].x];
+                pos[u] = x + u < n_out ? 0u : myD[ed[u].x];
             }
-        }
-        for (int x = n_out; x < n_out + n_in; ++x) {
-            const int2 ed = __ldg(P.dep + d0 + x);
-            const int a = ed.x & 0xFF, b = ed.x >> 8;
-            const uint32_t tg = myD[32 * a] ^ myD[32 * b];
-            if (!tg) continue; // the edge toggles for no individual
-            const uint32_t cut = myO[32 * a] ^ myO[32 * b] ^ (uint32_t)(ed.y >> 31);
-            add_signed<R + 1, kWeightBits>(D, tg & ~cut, tg & cut, (uint32_t)(ed.y < 0 ? -ed.y : ed.y));
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int ra = (ed[u].y >> kEdgeRow) & (31 << 5);
+                const uint32_t tg = myD[ra] ^ pos[u], cut = myO[ra] ^ neg[u] ^ (uint32_t)(ed[u].y >> 31);
+                pos[u] = tg & ~cut;
+                neg[u] = tg & cut;
+            }
+            add_signed4<R + 1, kWeightBits>(D, pos, neg, ed);
         }
         uint32_t nz = 0;
 #pragma unroll

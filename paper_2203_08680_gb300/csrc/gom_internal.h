@@ -235,5 +235,6 @@ struct GomParams {
     const int32_t *wabs;     // [total_vars] sum of |w| over each variable's outside edges
     const uint32_t *seg;     // [total_vars + m]
     const int2 *dep;         // outside edges {v, w}, then inside edges {a | b << 8, w}
+    const int2 *bdep;        // the same edges for the bit-sliced path (gom_bitplane.cuh), where it is available
     const int32_t *cptr;     // [k+1] colour -> positions
 };

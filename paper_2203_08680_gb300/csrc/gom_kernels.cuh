@@ -32,6 +32,8 @@ const void *gom_run_kernel(int wpi, int variant, bool learn);
 const void *gom_run_bs_kernel(int s, int r, bool learn);
 const void *gom_mix_bs_kernel(int s, int r, bool learn);
 int gom_bs_warp_words(int s);
+// Packs the dependency lists into the bit-sliced path's edge lists (P.bdep).
+__global__ void k_bs_edges(GomParams P, int2 *bdep);
 // The instances of one element class (8, 16 or 32 variables at most).
 const void *gom_run_bs8(int r, bool learn);
 const void *gom_mix_bs8(int r, bool learn);
