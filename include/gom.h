@@ -88,13 +88,14 @@ extern "C" {
                                works on 32 trials); the donor search stays per individual.
                                Available for elements of at most 32 variables, |w| <= 255 and
                                element weight sums (of |w| over their edges) below 2^16; the
-                               default where available, a variable row has at most 16 words
-                               (p <= 512) and the largest colour group gives at least a quarter
-                               of the resident warps an item (GOM_E_STATE when set to 1 where
-                               unavailable).  Same results either way; the learned filter works
-                               on both.  A batched launch follows the value the caller set for
-                               the context, else the same rule on the warps the instance gets
-                               (bit-sliced instances only with min_blocks 2) */
+                               default where available except for the smallest problems (groups
+                               of a few hundred population words, or one-word populations of
+                               elements above 16 variables that do not fill the GPU)
+                               (GOM_E_STATE when set to 1 where unavailable).  Same results
+                               either way; the learned filter works on both.  A batched launch
+                               follows the value the caller set for the context, else runs
+                               bit-sliced the instances whose largest group gives each of their
+                               warps four (element, word) pairs or more (only with min_blocks 2) */
 
 #define GOM_OPT_FORCED_IMPROVEMENT 5 /* 1: Forced Improvement (Sec. 4, Alg. 1) after each generation's
                                         mixing, in this library's parallel reading (the paper's
@@ -394,7 +395,8 @@ typedef struct gom_batch_config {
     int32_t item_cost;       /* block allocation: a warp's time for one element is taken as
                                 item_cost + (population words) x (variables + edges), so
                                 item_cost is the fixed cost of an item (staging, draws,
-                                memory round trips); 0 means 300 */
+                                memory round trips); 0 means 300.  (On the bit-sliced phase:
+                                per word item_cost / 64 + 0.34 x (variables + edges)) */
 } gom_batch_config_t;
 
 /* Device bytes of a batch of `num` instances (their parameter blocks, the

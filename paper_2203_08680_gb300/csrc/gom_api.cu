@@ -536,9 +536,8 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
             const void *rf = gom_run_bs_kernel(S, R, false), *mf = gom_mix_bs_kernel(S, R, false);
             const void *rfl = gom_run_bs_kernel(S, R, true), *mfl = gom_mix_bs_kernel(S, R, true);
             if (wpb >= 1 && smem <= static_cast<size_t>(kSmemBudget) && rf && mf && rfl && mfl) {
-                const int E = 32 / c->W;
+                const int E = 32 / wv;
                 const int64_t items = (max_group + E - 1) / E;
-                const int64_t need = std::max<int64_t>(1, (items + wpb - 1) / wpb);
                 for (const void *fn : {rf, mf, rfl, mfl}) GOM_CUDA(c, raise_smem_limit(fn, smem));
                 int occ_r = 0, occ_m = 0, occ_rl = 0, occ_ml = 0;
                 GOM_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_r, rf, 32 * wpb, smem));
@@ -554,17 +553,20 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
                     c->mix_bs_fn = mf;
                     c->bs_smem = smem;
                     c->bs_threads = 32 * wpb;
+                    bs_split(wv, max_group, tabs.max_edges, static_cast<int64_t>(c->sms) * occ_r * wpb, wpb,
+                             &c->prm.bs_lsh, &c->prm.bs_nwi);
+                    // a block per tile up to one per SM, then full blocks
+                    const int64_t Et = c->prm.bs_nwi > 1 ? 1 : (32 >> c->prm.bs_lsh) / wv;
+                    const int64_t tiles = std::max<int64_t>(1, (max_group + Et - 1) / Et);
+                    const int64_t need = std::max<int64_t>(std::min<int64_t>(tiles, c->sms),
+                                                           (tiles * c->prm.bs_nwi + wpb - 1) / wpb);
                     c->bs_grid_run = static_cast<int>(std::min<int64_t>(static_cast<int64_t>(c->sms) * occ_r, need));
                     c->bs_grid_mix = static_cast<int>(std::min<int64_t>(
                         std::min<int64_t>(static_cast<int64_t>(c->sms) * occ_m, need), kMaxMixBlocks));
                     c->prm.bs_S = S;
                     c->prm.bs_words = static_cast<int32_t>(ww);
-                    // the default where the largest group gives at least a quarter of the
-                    // resident warps an item, and a variable row has at most 16 words: with
-                    // fewer items the per-lane path's finer items win, and with 32 words
-                    // (one element per item) its scalar trials do (measured on the torus,
-                    // 3D torus and random regular workloads, p = 64 to 1024)
-                    c->bs_on = c->W <= 16 && 4 * items >= static_cast<int64_t>(c->sms) * occ_r * wpb;
+                    c->bs_on = bs_pays(wv, max_group, tabs.max_s, c->prm.stage_all != 0,
+                                       static_cast<int64_t>(c->sms) * occ_r * wpb);
                 }
             }
         }

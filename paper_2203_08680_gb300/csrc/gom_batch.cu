@@ -76,26 +76,44 @@ int64_t max_split_items(const gom_ctx *c)
 }
 
 // Estimated warp time of one generation of an instance: per element, a fixed
-// item cost plus (population words) x (variables + edges).
-double instance_cost(const gom_ctx *c, int item_cost)
+// item cost plus (population words) x (variables + edges); on the bit-sliced
+// phase, per word of an element, item_cost / 64 plus a third per variable and
+// edge (a warp's 32 pairs take 50 + 3.3 e instructions each for elements of e
+// edges, about 9 instructions a unit of the per-lane estimate).
+double instance_cost(const gom_ctx *c, int item_cost, bool bits)
 {
     const int wv = (c->p + 31) / 32;
+    if (bits) return wv * (static_cast<double>(c->m) * item_cost / 64.0 + 0.34 * c->sum_se);
     return static_cast<double>(c->m) * item_cost + static_cast<double>(wv) * c->sum_se;
+}
+
+// Whether an instance on `warps` warps runs the bit-sliced phase (only in the
+// kernel with the larger register budget, min_blocks 2): as the caller set it
+// for the context, else where its largest group gives every warp four pairs or
+// more (48 instances of 200 to 4,000 vertices, one to three a warp: 1.13 ms a
+// generation against 0.94 per lane; 48 of 1,000 to 65,536, five to thirty:
+// 2.1 against 7.2, and 3.1 with those below eight left per lane).
+bool batch_bits(const gom_ctx *c, const gom_batch_config_t &conf, int64_t warps)
+{
+    if (!c->bs_ok || conf.min_blocks != 2) return false;
+    if (c->bs_set >= 0) return c->bs_set == 1;
+    return c->max_group * ((c->p + 31) / 32) >= 4 * warps;
 }
 
 // Blocks per instance: one each, then one at a time to the instance with the
 // largest estimated time per block, up to what its largest colour group can
 // use (one warp per item) or until the device is full.
-std::vector<int32_t> allocate_blocks(const std::vector<gom_ctx *> &ctx, int total_blocks, int warps_per_block,
-                                     int item_cost)
+std::vector<int32_t> allocate_blocks(const std::vector<gom_ctx *> &ctx, int total_blocks, const gom_batch_config_t &conf)
 {
+    const int warps_per_block = conf.warps_per_block, item_cost = conf.item_cost > 0 ? conf.item_cost : 300;
     const size_t B = ctx.size();
     std::vector<int32_t> nb(B, 1);
     std::vector<double> cost(B);
     std::priority_queue<std::pair<double, size_t>> heap;
     std::vector<int64_t> need(B);
     for (size_t b = 0; b < B; ++b) {
-        cost[b] = instance_cost(ctx[b], item_cost);
+        // (as bit-sliced where it can be: what falls back to the per-lane phase is small)
+        cost[b] = instance_cost(ctx[b], item_cost, batch_bits(ctx[b], conf, 0));
         need[b] = (max_split_items(ctx[b]) + warps_per_block - 1) / warps_per_block;
         if (need[b] > 1) heap.push({cost[b], b});
     }
@@ -193,8 +211,7 @@ int gom_batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config
     B->d_inst = reinterpret_cast<GomBatchInst *>(base + L.inst);
     B->d_bars = reinterpret_cast<GomBarrier *>(base + L.bars);
 
-    const std::vector<int32_t> nb =
-        allocate_blocks(cs, total, conf.warps_per_block, conf.item_cost > 0 ? conf.item_cost : 300);
+    const std::vector<int32_t> nb = allocate_blocks(cs, total, conf);
     B->params.resize(num);
     B->inst.resize(num);
     int32_t blk = 0;
@@ -231,6 +248,8 @@ int gom_batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config
         P.learn = 0; // the learned filter is not active inside batched launches
         P.fi.on = 0; // nor Forced Improvement (refused above)
         P.bar = B->d_bars + b; // (P.trace: the context's phase trace, when switched on)
+        // (one-warp tiles: the blocks' named barriers are left to the block-mode instances)
+        if (c->bs_ok) bs_split(wv, c->max_group, c->max_edges, int64_t(nb[b]) * conf.warps_per_block, 1, &P.bs_lsh, &P.bs_nwi);
         B->params[b] = P;
         GomBatchInst &I = B->inst[b];
         I = GomBatchInst{};
@@ -238,14 +257,7 @@ int gom_batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config
         I.nblk = nb[b];
         I.wpi = wpi;
         I.variant = cs[b]->variant;
-        // the bit-sliced phase, as the caller set it for the context, else where
-        // it pays on a single context (at most 16 words per row, items for at
-        // least a quarter of the warps), counted on this instance's warps
-        const int64_t bs_items = (c->max_group + (32 / c->W) - 1) / (32 / c->W);
-        // (only in the kernel with the larger register budget, 2 blocks of 256 threads)
-        const bool use_bs = c->bs_ok && conf.min_blocks == 2 &&
-                            (c->bs_set >= 0 ? c->bs_set == 1
-                                            : c->W <= 16 && 4 * bs_items >= int64_t(nb[b]) * conf.warps_per_block);
+        const bool use_bs = batch_bits(c, conf, int64_t(nb[b]) * conf.warps_per_block);
         if (use_bs) {
             I.variant = kVarBits;
             I.bs_r = c->bs_r;

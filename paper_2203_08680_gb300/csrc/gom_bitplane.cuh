@@ -109,17 +109,35 @@ __device__ __forceinline__ void add_signed4(uint32_t (&D)[NP], const uint32_t (&
     }
 }
 
+// The bit-sliced fitness accumulator of a lane: kFitPlanes planes in
+// registers, or in shared memory (plane t of the warp's lanes at word 32 t; the
+// mixing needs the registers for its tables).
+struct FitRegs {
+    uint32_t v[kFitPlanes];
+    __device__ __forceinline__ uint32_t get(int t) const { return v[t]; }
+    __device__ __forceinline__ void set(int t, uint32_t x) { v[t] = x; }
+};
+struct FitShared {
+    uint32_t *v;
+    __device__ __forceinline__ uint32_t get(int t) const { return v[32 * t]; }
+    __device__ __forceinline__ void set(int t, uint32_t x) { v[32 * t] = x; }
+};
+
 // Per-lane state of the bit-sliced path across the groups of a generation.
+template <class Fit>
 struct BsLane {
-    uint32_t fit[kFitPlanes]; // accepted deltas of this lane's 32 individuals (word lane mod W), bit-sliced
-    int since_flush;          // items added since the last flush (warp-uniform)
+    Fit fit;         // accepted deltas of this lane's 32 individuals (word w), bit-sliced
+    int w;
+    int since_flush; // items added since the last flush (warp-uniform)
     unsigned n_dl, n_acc, n_imp;
 };
 
-__device__ __forceinline__ void bs_lane_zero(BsLane &L)
+template <class Fit>
+__device__ __forceinline__ void bs_lane_zero(BsLane<Fit> &L, int w)
 {
+    L.w = w;
 #pragma unroll
-    for (int t = 0; t < kFitPlanes; ++t) L.fit[t] = 0;
+    for (int t = 0; t < kFitPlanes; ++t) L.fit.set(t, 0);
     L.since_flush = 0;
     L.n_dl = L.n_acc = L.n_imp = 0;
 }
@@ -127,39 +145,48 @@ __device__ __forceinline__ void bs_lane_zero(BsLane &L)
 // Adds the lane's accumulated deltas into the block's fitness accumulators
 // s_f[32 w + b] (one shared atomic per individual with a non-zero sum) and
 // clears them.  Warp-wide call.
-__device__ __forceinline__ void bs_flush(const GomParams &P, BsLane &L, long long *s_f)
+template <class Fit>
+__device__ __forceinline__ void bs_flush(BsLane<Fit> &L, long long *s_f)
 {
-    const int lane = threadIdx.x & 31;
-    const int w = lane & (P.W - 1);
+    const int w = L.w;
     uint32_t any = 0;
 #pragma unroll
-    for (int t = 0; t < kFitPlanes; ++t) any |= L.fit[t];
+    for (int t = 0; t < kFitPlanes; ++t) any |= L.fit.get(t);
     if (any) {
         for (int b = 0; b < 32; ++b) {
             if (!((any >> b) & 1u)) continue;
             unsigned v = 0;
 #pragma unroll
-            for (int t = 0; t < kFitPlanes; ++t) v |= ((L.fit[t] >> b) & 1u) << t;
+            for (int t = 0; t < kFitPlanes; ++t) v |= ((L.fit.get(t) >> b) & 1u) << t;
             atomicAdd(reinterpret_cast<unsigned long long *>(&s_f[32 * w + b]), (unsigned long long)v);
         }
     }
 #pragma unroll
-    for (int t = 0; t < kFitPlanes; ++t) L.fit[t] = 0;
+    for (int t = 0; t < kFitPlanes; ++t) L.fit.set(t, 0);
     L.since_flush = 0;
 }
 
 // Adds the accepted deltas (non-negative and below 2^R: planes 0 .. R - 1 of
 // D, masked by acc) into the lane's fitness accumulator.
-template <int R>
-__device__ __forceinline__ void fit_add(BsLane &L, const uint32_t (&D)[R + 1], uint32_t acc)
+template <int R, class Fit>
+__device__ __forceinline__ void fit_add(BsLane<Fit> &L, const uint32_t (&D)[R + 1], uint32_t acc)
 {
     uint32_t carry = 0;
 #pragma unroll
-    for (int t = 0; t < kFitPlanes; ++t) {
-        const uint32_t in = t < R ? (D[t] & acc) : 0u;
-        const uint32_t a = L.fit[t];
-        L.fit[t] = a ^ in ^ carry;
+    for (int t = 0; t < R; ++t) {
+        const uint32_t in = D[t] & acc, a = L.fit.get(t);
+        L.fit.set(t, a ^ in ^ carry);
         carry = (a & in) | (a & carry) | (in & carry);
+    }
+#pragma unroll
+    for (int t4 = R; t4 < kFitPlanes; t4 += 4) {
+        if (!carry) return;
+#pragma unroll
+        for (int t = t4; t < t4 + 4 && t < kFitPlanes; ++t) {
+            const uint32_t a = L.fit.get(t);
+            L.fit.set(t, a ^ carry);
+            carry &= a;
+        }
     }
 }
 

@@ -51,11 +51,11 @@ __global__ void __launch_bounds__(kMixThreads, 2) k_fi_group(GomParams P, int t)
         s_act[threadIdx.x] = (int)threadIdx.x < P.W ? P.fi.act0[threadIdx.x] & ~done : 0u;
     }
     acc_zero(P, s_f, s_cnt);
-    BsLane L;
-    bs_lane_zero(L);
+    BsLane<FitRegs> L;
+    bs_lane_zero(L, (threadIdx.x & 31) & (P.W - 1));
     unsigned cnt[3] = {0, 0, 0};
     fi_group<R>(P, whole_grid(), t, P.order[t], s_act, L, cnt, s_f);
-    bs_flush(P, L, s_f);
+    bs_flush(L, s_f);
     fi_count_flush(P, cnt);
     acc_flush(P, s_f, s_cnt);
 }

@@ -9,9 +9,13 @@
 // one 32-bit register holds one bit of 32 individuals, so one logic
 // instruction works on 32 trials at once.
 //
-// A warp takes an item of E = 32 / W elements of the colour group (W = words
-// per variable row); lane k owns the pair (element slot k / W, word k mod W),
-// i.e. 32 individuals of one element.  Per item:
+// A tile takes an item of E elements of the colour group.  A pair is one word
+// (32 individuals) of one element; an element has Wv pairs.  Normally a tile
+// is a warp, a lane owns one pair and E = 32 / Wv.  Where a colour group is too
+// small to give every resident warp an item, 2 to 32 lanes share a pair (they
+// repeat phase 0 and split the donor draws and the element's edges), and an
+// element whose lanes pass one warp takes 2 or 4 warps of a block (BsMap).
+// Per item:
 //   phase 0  (lane = pair) the parent's current rows on F_j into shared
 //            memory, the generation-start rows of P on F_j in registers; the
 //            run starts of P's patterns (bit d: pattern d differs from pattern
@@ -124,21 +128,76 @@ __host__ __device__ constexpr int bs_entry_words(int SB) { return 2 * SB; }
 // The class of the largest element S.
 __host__ __device__ constexpr int bs_class(int S) { return S <= 8 ? 8 : S <= 16 ? 16 : 32; }
 
-// Shared-memory words of one warp's region: the donor tables [32 pairs], the
-// trials' entries [32 pairs] (their slots reused for the flip planes
-// [S][32 pairs]), the rows of O on F_j [S][32 pairs] and the run starts [32
-// pairs].  Row arrays are variable-major: lane l reads word 32 a + l, free of
-// bank conflicts for any a.
+// Shared-memory words of one warp's region (a tile of several warps uses its
+// first warp's): the donor tables [32 pairs], the trials' entries [32 pairs]
+// (their slots reused for the flip planes [S][32 pairs]), the rows of O on F_j
+// [S][32 pairs], per pair the run starts, the patterns of the word's last
+// individual and of its first run start, and the warp's fitness planes
+// [kFitPlanes][32 lanes] (every warp of a tile its own).  Row arrays are
+// variable-major: pair slot l reads word 32 a + l, free of bank conflicts for
+// any a.
 __host__ __device__ __forceinline__ int bs_warp_words(int S)
 {
-    return 64 * bs_entry_words(bs_class(S)) + 32 * S + 32;
+    return 64 * bs_entry_words(bs_class(S)) + 32 * S + 96 + 32 * kFitPlanes;
 }
 
-// The dynamic shared memory of the bit-sliced kernels: the block's fitness
-// accumulators (32 W int64, i.e. 64 W words) first, then the warps' regions.
-__device__ __forceinline__ uint32_t *bs_warp_region(const GomParams &P, uint32_t *s_dyn)
+// Blocks per SM the kernels' registers are cut for, by element class: what the
+// regions leave of an SM's shared memory (34, 54 and 90 KB a block).
+constexpr int bs_blocks(int SB) { return SB == 8 ? 6 : SB == 16 ? 4 : 2; }
+
+// This lane's fitness planes; `regions` is the block's first warp region.
+__device__ __forceinline__ uint32_t *bs_fit(const GomParams &P, uint32_t *regions)
 {
-    return s_dyn + 64 * P.W + (threadIdx.x >> 5) * P.bs_words;
+    return regions + ((threadIdx.x >> 5) + 1) * P.bs_words - 32 * kFitPlanes + (threadIdx.x & 31);
+}
+
+// This thread's place in its tile: lanes 2^lsh per pair, nwi warps per tile
+// (more than one only for E = 1), the pair's slot, its element slot e and word
+// w, `sub` the lane's number within the pair; in: the slot holds a pair of the
+// tile's E elements.
+struct BsMap {
+    int lsh, nwi, E;
+    int tile, ntiles; // of the (virtual) grid: consecutive tiles go to different blocks
+    int slot, e, w, sub;
+    bool in;
+    uint32_t *sm;     // the tile's shared region
+};
+
+// The tile's map; `regions` is the block's first warp region.
+template <bool LEARN>
+__device__ __forceinline__ BsMap bs_map(const GomParams &P, const VGrid &V, uint32_t *regions)
+{
+    BsMap M;
+    const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    M.lsh = LEARN ? 0 : P.bs_lsh; // the learned filter's bookkeeping takes one lane per pair
+    M.nwi = LEARN ? 1 : P.bs_nwi;
+    M.E = M.nwi > 1 ? 1 : (32 >> M.lsh) / P.Wv;
+    const int tb = wib / M.nwi, tw = wib - tb * M.nwi;
+    M.tile = tb * V.nblk + V.blk;
+    M.ntiles = (int)(blockDim.x >> 5) / M.nwi * V.nblk;
+    M.slot = (32 * tw + lane) >> M.lsh;
+    M.e = M.slot / P.Wv;
+    M.w = M.slot - M.e * P.Wv;
+    M.sub = lane & ((1 << M.lsh) - 1);
+    M.in = M.e < M.E;
+    M.sm = regions + tb * M.nwi * P.bs_words;
+    return M;
+}
+
+// Waits for the tile's threads (every thread of the tile calls it): a warp, a
+// whole block of four warps, or half of one on a named barrier.  The barrier
+// numbers are constants: a number in a register makes the compiler reserve all
+// 16 of a block, and an SM's 64 then hold four blocks.
+__device__ __forceinline__ void tile_sync(const BsMap &M)
+{
+    if (M.nwi == 1)
+        __syncwarp();
+    else if (M.nwi == kBsThreads / 32)
+        __syncthreads();
+    else if (threadIdx.x < kBsThreads / 2)
+        asm volatile("bar.sync 1, 64;" ::: "memory");
+    else
+        asm volatile("bar.sync 2, 64;" ::: "memory");
 }
 
 // Learned filter bookkeeping after a bit-sliced item (warp-wide): each
@@ -152,14 +211,17 @@ __device__ __noinline__ void bs_record(const GomParams &P, int q, bool ke, bool 
                                        unsigned dl, unsigned imp, unsigned long long *s_fc)
 {
     const int lane = threadIdx.x & 31;
-    const int W = P.W, lw = __ffs(W) - 1, E = 32 >> lw;
-    for (int off = 1; off < W; off <<= 1) {
-        acc += __shfl_xor_sync(kFull, acc, off);
-        dl += __shfl_xor_sync(kFull, dl, off);
-        imp += __shfl_xor_sync(kFull, imp, off);
+    const int Wv = P.Wv, E = 32 / Wv, first = lane - lane % Wv; // the element's first lane (one lane per pair here)
+    unsigned ad = acc | dl << 16, sum_ad = 0, sum_imp = 0; // at most 1,024 each
+    for (int x = 0; x < Wv; ++x) {
+        sum_ad += __shfl_sync(kFull, ad, first + x);
+        sum_imp += __shfl_sync(kFull, imp, first + x);
     }
+    acc = sum_ad & 0xFFFFu;
+    dl = sum_ad >> 16;
+    imp = sum_imp;
     const bool useful = P.flt.label ? imp != 0 : acc != 0;
-    if (ke && (lane & (W - 1)) == 0) {
+    if (ke && lane == first) {
         uint32_t *cur = P.flt.hist + (size_t)(g & 1) * 3 * (size_t)P.m;
         cur[q] = acc;
         cur[P.m + q] = dl;
@@ -170,7 +232,7 @@ __device__ __noinline__ void bs_record(const GomParams &P, int q, bool ke, bool 
         if (audited && useful) atomicAdd(&s_fc[3], 1ull);
     }
     for (int e2 = 0; e2 < E; ++e2) {
-        const int src = e2 << lw;
+        const int src = e2 * Wv;
         const int q2 = __shfl_sync(kFull, q, src);
         const bool ok = __shfl_sync(kFull, ke ? 1 : 0, src) != 0;
         const bool u2 = __shfl_sync(kFull, useful ? 1 : 0, src) != 0;
@@ -219,35 +281,46 @@ __device__ __noinline__ bool self_hit(uint32_t *fl, const uint32_t *tab, const u
     return true;
 }
 
-// One item of colour group c at position t: entries [k0, k1) (at most E) of
-// the group's elements -- positions k0 .. k1 - 1, or with the learned filter
+// An item between its two parts: the lane's element and what the first part
+// found in the generation-start population.
+template <int SB>
+struct BsItem {
+    int q, j, s, f0, d0, n_out, n_in;
+    bool ke, audited;   // the lane's pair exists; the element runs as an audit of the learned filter
+    uint32_t rs, nz;    // run starts of the pair, non-empty run-start words of the element
+    uint32_t xp[SB <= 16 ? SB : 1]; // P's rows (the widest class reads them again)
+};
+
+// First part of an item of a colour group: entries [k0, k1) (at most E) of the
+// group's elements -- positions k0 .. k1 - 1, or with the learned filter
 // skipping, the positions qlist[k0 .. k1) of the compacted list -- with every
-// word, all trials of Alg. 2.
-template <int SB, int R, bool LEARN>
-__device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist, int k0, int k1, uint32_t g,
-                                        uint32_t *wsm, BsLane &L, long long *s_f, unsigned long long *s_fc)
+// word.  Donor tables and the trials' entries: all of it from P, which does
+// not change during a generation, so a tile makes the first item of a group
+// between its arrival at the barrier that opens the group and its wait there.
+template <int SB, bool LEARN>
+__device__ __forceinline__ void bs_prepare(const GomParams &P, const BsMap &M, const int32_t *qlist, int k0, int k1,
+                                           uint32_t g, BsItem<SB> &I)
 {
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, slot = M.slot;
     const int W = P.W, Wv = P.Wv, p = P.p, S = P.bs_S;
-    const int lw = __ffs(W) - 1;
-    const int e = lane >> lw, w = lane & (W - 1);
-    const bool ke = k0 + e < k1; // this lane's element exists
+    const int e = M.e, w = M.w, b2 = e * Wv; // b2: the element's first slot
+    const bool ke = M.in && k0 + e < k1;     // this lane's pair exists
     int q = k0 + e;
-    bool audited = false;
+    I.audited = false;
     if (LEARN && qlist && ke) {
         const int32_t en = qlist[k0 + e];
         q = en & 0x7FFFFFFF;
-        audited = en < 0;
+        I.audited = en < 0;
     }
-    const bool kv = ke && w < Wv; // this lane's pair exists
+    I.q = q;
+    I.ke = ke;
     constexpr int EW = bs_entry_words(SB);
-    uint32_t *tab = wsm, *res = wsm + 32 * EW;
-    uint32_t *sF = res; // flip planes, once every lane has read its entries back
-    uint32_t *sX = wsm + 64 * EW, *sRS = sX + 32 * S;
-    const int lim = p - 32 * w;
-    const uint32_t vm = lim >= 32 ? 0xFFFFFFFFu : lim > 0 ? (1u << lim) - 1u : 0u; // this word's individuals
+    uint32_t *tab = M.sm, *res = M.sm + 32 * EW;
+    uint32_t *sRS = M.sm + 64 * EW + 32 * S, *sLst = sRS + 32, *sFst = sLst + 32;
+    const int lim = p - 32 * w; // >= 1
+    const uint32_t vm = lim >= 32 ? 0xFFFFFFFFu : (1u << lim) - 1u; // this word's individuals
 
-    // ---- phase 0: the pair's rows, run starts, donor table
+    // ---- phase 0: P's rows, run starts, donor table
     int j = 0, s = 0, f0 = 0, d0 = 0, n_in = 0, n_out = 0;
     if (ke) {
         const int4 a = __ldg(P.hdr + 2 * q), b = __ldg(P.hdr + 2 * q + 1);
@@ -258,65 +331,72 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
         n_in = a.w >> 8;
         n_out = b.x;
         // the element's edge list is read in phase 2: ask for its lines in L2
-        // now (the W lanes of the element take every W-th line; the array
+        // now (the Wv words of the element take every Wv-th line; the array
         // starts on a 256-byte boundary, so every line named here holds bytes
         // of it)
         const uintptr_t d_at = reinterpret_cast<uintptr_t>(P.bdep + d0), d_end = d_at + 8u * (uint32_t)(n_out + n_in);
-        for (uintptr_t at = (d_at & ~uintptr_t(127)) + 128u * (uint32_t)w; at < d_end; at += 128u * (uint32_t)W)
+        for (uintptr_t at = (d_at & ~uintptr_t(127)) + 128u * (uint32_t)w; at < d_end; at += 128u * (uint32_t)Wv)
             prefetch_l2(reinterpret_cast<const void *>(at));
     }
+    I.j = j;
+    I.s = s;
+    I.f0 = f0;
+    I.d0 = d0;
+    I.n_in = n_in;
+    I.n_out = n_out;
     uint32_t xp[SB];
-    uint32_t chg = 0; // individuals that changed on F_j since the generation start
 #pragma unroll
     for (int a = 0; a < SB; ++a) xp[a] = 0;
 #pragma unroll
     for (int a8 = 0; a8 < SB; a8 += 8) {
         if (a8 < S) {
             int at[8];
-            uint32_t xo[8];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) at[c] = kv && a8 + c < s ? __ldg(P.fv + f0 + a8 + c) * W + w : -1;
+            for (int c = 0; c < 8; ++c) at[c] = ke && a8 + c < s ? __ldg(P.fv + f0 + a8 + c) * W + w : -1;
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                xo[c] = at[c] >= 0 ? P.O[at[c]] : 0u;
-                xp[a8 + c] = at[c] >= 0 ? P.P[at[c]] : 0u;
-            }
-#pragma unroll
-            for (int c = 0; c < 8; ++c) {
-                chg |= xo[c] ^ xp[a8 + c];
-                if (a8 + c < S) sX[32 * (a8 + c) + lane] = xo[c];
-            }
+            for (int c = 0; c < 8; ++c) xp[a8 + c] = at[c] >= 0 ? P.P[at[c]] : 0u;
         }
     }
-    uint32_t rs = 0, fst = 0, nz;
+    if constexpr (SB <= 16) {
+#pragma unroll
+        for (int a = 0; a < SB; ++a) I.xp[a] = xp[a];
+    }
+    uint32_t rs = 0, nx, nz;
     {   // run starts of the element's patterns in word w: bit b set iff the
         // pattern of individual 32 w + b differs from the one before it
-        // (cyclically: the word before's last individual, by a shuffle of the
-        // packed last bits); fst: the pattern at the word's first run start
-        const int lastb = lim >= 32 ? 31 : lim > 0 ? lim - 1 : 0;
+        // (cyclically: the word before's last individual); the pattern at the
+        // word's first run start
+        const int lastb = lim >= 32 ? 31 : lim - 1;
         uint32_t lst = 0;
 #pragma unroll
         for (int a = 0; a < SB; ++a)
             if (a < S) lst |= ((xp[a] >> lastb) & 1u) << a;
-        const uint32_t prv = __shfl_sync(kFull, lst, e * W + (w == 0 ? Wv - 1 : w - 1));
+        sLst[slot] = lst;
+        tile_sync(M);
+        const uint32_t prv = sLst[M.in ? b2 + (w == 0 ? Wv - 1 : w - 1) : slot];
 #pragma unroll
         for (int a = 0; a < SB; ++a)
             if (a < S) rs |= xp[a] ^ __funnelshift_l(prv << (31 - a), xp[a], 1);
-        rs = kv ? rs & vm : 0u;
-        sRS[lane] = rs;
+        rs = ke ? rs & vm : 0u;
+        sRS[slot] = rs;
         const int fb = rs ? __ffs(rs) - 1 : 0;
+        uint32_t fst = 0;
 #pragma unroll
         for (int a = 0; a < SB; ++a)
             if (a < S) fst |= ((xp[a] >> fb) & 1u) << a;
-        // element e's words with a run start: bits e W .. e W + W - 1 of the ballot
-        const uint32_t nzb = __ballot_sync(kFull, rs != 0);
-        nz = W == 32 ? nzb : (nzb >> (e * W)) & ((1u << W) - 1u);
+        sFst[slot] = fst;
+        tile_sync(M);
+        // the element's words with a run start: bits b2 .. of the ballot over all slots
+        const uint32_t nzb = __ballot_sync(kFull, lane < M.E * Wv && sRS[lane] != 0);
+        nz = Wv == 32 ? nzb : (nzb >> b2) & ((1u << Wv) - 1u);
+        // the first run start after word w (cyclically): its pattern carries into
+        // the word's last individuals; without any run start every pattern is the same
+        const uint32_t later = nz & ~((2u << w) - 1u); // words after w
+        const uint32_t any = later ? later : nz;        // else wrap round
+        nx = any ? sFst[b2 + __ffs(any) - 1] : fst;
+        I.rs = rs;
+        I.nz = nz;
     }
-    // the first run start after word w (cyclically): its pattern carries into
-    // the word's last individuals; without any run start every pattern is the same
-    const uint32_t later = nz & ~((2u << w) - 1u); // words after w
-    const uint32_t any = later ? later : nz;        // else wrap round
-    uint32_t nx = __shfl_sync(kFull, fst, e * W + (any ? __ffs(any) - 1 : w));
     {
         uint32_t x[SB];
 #pragma unroll
@@ -336,15 +416,15 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
                     ent[r / 2] = __byte_perm(lo, hi, 0x5410);
                 }
                 nx >>= 8;
-                *reinterpret_cast<uint4 *>(tab + 16 * lane + 4 * c) = make_uint4(ent[0], ent[1], ent[2], ent[3]);
+                *reinterpret_cast<uint4 *>(tab + 16 * slot + 4 * c) = make_uint4(ent[0], ent[1], ent[2], ent[3]);
             }
         } else if constexpr (SB == 16) {
 #pragma unroll
             for (int c = 1; c >= 0; --c) {
 #pragma unroll
                 for (int r = 15; r >= 0; --r) {
-                    // word 32 lane + d rotated by the lane: 32 lanes hit 32 banks
-                    tab[32 * lane + ((16 * c + r + lane) & 31)] = __byte_perm(x[r], nx, c ? 0x7632 : 0x5410);
+                    // word 32 slot + d rotated by the slot: 32 slots hit 32 banks
+                    tab[32 * slot + ((16 * c + r + slot) & 31)] = __byte_perm(x[r], nx, c ? 0x7632 : 0x5410);
                     if ((rs >> (16 * c + r)) & 1u) nx = x[r];
                 }
                 nx >>= 16;
@@ -352,24 +432,27 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
         } else {
 #pragma unroll
             for (int r = 31; r >= 0; --r) {
-                const int at = 32 * lane + ((r + lane) & 31);
+                const int at = 32 * slot + ((r + slot) & 31);
                 tab[at] = x[r];
                 tab[1024 + at] = nx;
                 if ((rs >> r) & 1u) nx = x[r];
             }
         }
     }
-    __syncwarp();
+    tile_sync(M);
 
-    // ---- phase 1: donors.  Call (pair k2, c) covers individuals 32 w2 + 4c ..
-    // + 3; the starts of individuals past p (in the last word's last call)
-    // stay below 32 Wv, inside the element's table
+    // ---- phase 1: donors, on the warp's own 32 / 2^lsh slots.  Call (slot k2,
+    // c) covers individuals 32 w2 + 4c .. + 3; the starts of individuals past p
+    // (in the last word's last call) stay below 32 Wv, inside the element's table
+    const int own = 32 >> M.lsh, k0w = slot & ~(own - 1); // slots of a warp are aligned to their number
+    const int info = ke ? w | b2 << 8 | 1 << 16 : 0;
 #pragma unroll 1
-    for (int r = 0; r < 8; ++r) {
-        const int k2 = 4 * r + (lane >> 3), c = lane & 7;
-        const int w2 = k2 & (W - 1), b2 = k2 - w2; // b2: the element's first pair
-        const int j2 = __shfl_sync(kFull, j, k2);
-        if (__shfl_sync(kFull, kv ? 1 : 0, k2)) {
+    for (int r = 0; r < own; r += 4) {
+        const int kl = r + (lane >> 3), c = lane & 7;
+        const int src = (kl & (own - 1)) << M.lsh, k2 = k0w + kl;
+        const int j2 = __shfl_sync(kFull, j, src), inf2 = __shfl_sync(kFull, info, src);
+        if (kl < own && inf2) {
+            const int w2 = inf2 & 0xFF, b2 = (inf2 >> 8) & 0xFF; // b2: that element's first slot
             const uint4 r4 = philox10_rk(make_uint4((uint32_t)j2, (uint32_t)(8 * w2 + c), g, kTagDonor), P.rk);
             const int i0 = 32 * w2 + 4 * c;
             uint32_t en[4], en2[4];
@@ -395,7 +478,47 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
             }
         }
     }
-    __syncwarp();
+    __syncwarp(); // (a warp reads its own slots' entries)
+}
+
+// Second part of an item, in its group: the parent's rows, the flip planes,
+// the partial evaluation, acceptance and writes of all its trials (Alg. 2).
+template <int SB, int R, bool LEARN>
+__device__ __forceinline__ void bs_item(const GomParams &P, const BsMap &M, const BsItem<SB> &I, uint32_t g,
+                                        BsLane<FitShared> &L, long long *s_f, unsigned long long *s_fc)
+{
+    const int slot = M.slot;
+    const int W = P.W, p = P.p, S = P.bs_S;
+    const int w = M.w, b2 = M.e * P.Wv, s = I.s;
+    const bool ke = I.ke;
+    constexpr int EW = bs_entry_words(SB);
+    const uint32_t *tab = M.sm;
+    uint32_t *res = M.sm + 32 * EW;
+    uint32_t *sF = res; // flip planes, once every lane has read its entries back
+    uint32_t *sX = M.sm + 64 * EW, *sRS = sX + 32 * S;
+    const int lim = p - 32 * w; // >= 1
+    const uint32_t vm = lim >= 32 ? 0xFFFFFFFFu : (1u << lim) - 1u; // this word's individuals
+
+    uint32_t chg = kFull; // individuals that changed on F_j since the generation start
+#pragma unroll
+    for (int a8 = 0; a8 < SB; a8 += 8) {
+        if (a8 < S) {
+            int at[8];
+            uint32_t xo[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) at[c] = ke && a8 + c < s ? __ldg(P.fv + I.f0 + a8 + c) * W + w : -1;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) xo[c] = at[c] >= 0 ? P.O[at[c]] : 0u;
+            if constexpr (SB > 16) {
+                if (a8 == 0) chg = 0;
+#pragma unroll
+                for (int c = 0; c < 8; ++c) chg |= at[c] >= 0 ? xo[c] ^ P.P[at[c]] : 0u;
+            }
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                if (a8 + c < S) sX[32 * (a8 + c) + slot] = xo[c];
+        }
+    }
 
     // the entries back as planes: t1[a] the starts' bits, then t2[a] the
     // fall-through patterns' bits; f1: the individuals whose start differs
@@ -404,13 +527,13 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
     {
         uint32_t t2[SB];
         if constexpr (SB == 8) {
-            const int sw = (lane >> 1) & 3;
+            const int sw = (slot >> 1) & 3;
 #pragma unroll
             for (int h = 0; h < 2; ++h) { // chunk i holds individuals 8 i .. 8 i + 7; half h of each
                 uint32_t A[4][2];          // [i][k]: individuals 8 i + 4 h + 2 k, + 1
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    const uint2 v = *reinterpret_cast<const uint2 *>(res + 16 * lane + ((i ^ sw) << 2) + 2 * h);
+                    const uint2 v = *reinterpret_cast<const uint2 *>(res + 16 * slot + ((i ^ sw) << 2) + 2 * h);
                     A[i][0] = v.x;
                     A[i][1] = v.y;
                 }
@@ -430,8 +553,8 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
         } else if constexpr (SB == 16) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) { // individuals 4 i .. + 3 and 16 + 4 i .. + 3
-                const uint4 u = *reinterpret_cast<const uint4 *>(res + 32 * lane + ((i ^ (lane & 7)) << 2));
-                const uint4 v = *reinterpret_cast<const uint4 *>(res + 32 * lane + (((i + 4) ^ (lane & 7)) << 2));
+                const uint4 u = *reinterpret_cast<const uint4 *>(res + 32 * slot + ((i ^ (slot & 7)) << 2));
+                const uint4 v = *reinterpret_cast<const uint4 *>(res + 32 * slot + (((i + 4) ^ (slot & 7)) << 2));
                 F[4 * i] = __byte_perm(u.x, v.x, 0x5410);
                 F[4 * i + 1] = __byte_perm(u.y, v.y, 0x5410);
                 F[4 * i + 2] = __byte_perm(u.z, v.z, 0x5410);
@@ -446,7 +569,7 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
         } else {
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                const uint4 u = *reinterpret_cast<const uint4 *>(res + 32 * lane + ((i ^ (lane & 7)) << 2));
+                const uint4 u = *reinterpret_cast<const uint4 *>(res + 32 * slot + ((i ^ (slot & 7)) << 2));
                 F[4 * i] = u.x;
                 F[4 * i + 1] = u.y;
                 F[4 * i + 2] = u.z;
@@ -455,7 +578,7 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
             transpose_lane<SB>(F);
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                const uint4 u = *reinterpret_cast<const uint4 *>(res + 1024 + 32 * lane + ((i ^ (lane & 7)) << 2));
+                const uint4 u = *reinterpret_cast<const uint4 *>(res + 1024 + 32 * slot + ((i ^ (slot & 7)) << 2));
                 t2[4 * i] = u.x;
                 t2[4 * i + 1] = u.y;
                 t2[4 * i + 2] = u.z;
@@ -465,11 +588,11 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
         }
 #pragma unroll
         for (int a = 0; a < SB; ++a)
-            if (a < S) f1 |= F[a] ^ sX[32 * a + lane];
-        if (SB < 32) { // (the widest class keeps no copy of P's rows: more individuals are looked at below)
+            if (a < S) f1 |= F[a] ^ sX[32 * a + slot];
+        if constexpr (SB <= 16) {
 #pragma unroll
             for (int a = 0; a < SB; ++a)
-                if (a < S) same &= ~(t2[a] ^ xp[a]);
+                if (a < S) same &= ~(t2[a] ^ I.xp[a]);
         }
         // every candidate from the start up to the next run start has the
         // start's pattern; when that is the parent's, the run start differs
@@ -477,41 +600,43 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
         // no flips, no donor
 #pragma unroll
         for (int a = 0; a < SB; ++a)
-            if (a < S) F[a] = ((f1 & F[a]) | (~f1 & t2[a])) ^ sX[32 * a + lane];
+            if (a < S) F[a] = ((f1 & F[a]) | (~f1 & t2[a])) ^ sX[32 * a + slot];
     }
-    __syncwarp(); // every lane has read its entries: their slots take the flip planes
+    tile_sync(M); // every lane has read its entries: their slots take the flip planes
     uint32_t hd = 0; // individuals with a donor
 #pragma unroll
     for (int a = 0; a < SB; ++a)
         if (a < S) {
-            const uint32_t Fa = kv ? F[a] & vm : 0u;
+            const uint32_t Fa = ke ? F[a] & vm : 0u;
             hd |= Fa;
-            sF[32 * a + lane] = Fa;
+            sF[32 * a + slot] = Fa;
         }
     // An individual that is itself the run start the search falls through to
-    // is skipped (a donor is another individual).  Only one that changed in
-    // this generation can be: one that did not has the pattern of its run,
-    // and the run before it has another.
-    uint32_t cand = kv ? ~f1 & rs & chg & same : 0u;
+    // is skipped (a donor is another individual).  Its start equals the parent
+    // and the fall-through is its own pattern in P, another one: only an
+    // individual that changed in this generation can be (for the widest
+    // class that is all that is checked here).
+    uint32_t cand = ke ? ~f1 & I.rs & chg & same : 0u;
     while (cand) { // divergent, rare
         const int b = __ffs(cand) - 1, i = 32 * w + b;
         cand &= cand - 1;
         uint32_t fl;
-        if (!self_hit<SB>(&fl, tab, sRS + e * W, nz, e * W, j, i, g, p, P.seed)) continue;
+        if (!self_hit<SB>(&fl, tab, sRS + b2, I.nz, b2, I.j, i, g, p, P.seed)) continue;
         hd = (hd & ~(1u << b)) | ((fl ? 1u : 0u) << b);
-        for (int a = 0; a < s; ++a) {
-            uint32_t *row = sF + 32 * a + lane;
-            *row = (*row & ~(1u << b)) | (((fl >> a) & 1u) << b);
-        }
+        if (M.sub == 0)
+            for (int a = 0; a < s; ++a) {
+                uint32_t *row = sF + 32 * a + slot;
+                *row = (*row & ~(1u << b)) | (((fl >> a) & 1u) << b);
+            }
     }
-    __syncwarp(); // (the tables are read above)
+    __syncwarp();
 
-    // ---- phase 2: bit-plane partial evaluation, acceptance, write, lane = pair
+    // ---- phase 2: bit-plane partial evaluation, acceptance, write
     unsigned i_acc = 0, i_dl = 0, i_imp = 0; // this pair's accepted, donor-less and improving trials
     // each item adds less than 2^R to an individual's sum: flush before it could pass 2^kFitPlanes
-    if (L.since_flush >= (1 << (kFitPlanes - R))) bs_flush(P, L, s_f);
-    if (kv) {
-        const uint32_t *myD = sF + lane, *myO = sX + lane; // variable a at word 32 a
+    if (L.since_flush >= (1 << (kFitPlanes - R))) bs_flush(L, s_f);
+    {
+        const uint32_t *myD = sF + slot, *myO = sX + slot; // variable a at word 32 a
         // the delta of every trial, R + 1 planes two's complement: an edge that
         // a trial toggles adds |w| if it was uncut (with its sign folded into
         // the cut bit), -|w| if it was cut (Eq. 1); no partial sum leaves
@@ -519,16 +644,16 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
         uint32_t D[R + 1];
 #pragma unroll
         for (int t = 0; t <= R; ++t) D[t] = 0;
-        const int ne = n_out + n_in;
-        for (int x = 0; x < ne; x += 4) { // four edges' loads issued before their arithmetic
+        const int ne = ke ? I.n_out + I.n_in : 0;
+        for (int x = 4 * M.sub; x < ne; x += 4 << M.lsh) { // four edges' loads issued before their arithmetic
             int2 ed[4];
             uint32_t pos[4], neg[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) ed[u] = x + u < ne ? __ldg(P.bdep + d0 + x + u) : make_int2(0, 0); // weight 0
+            for (int u = 0; u < 4; ++u) ed[u] = x + u < ne ? __ldg(P.bdep + I.d0 + x + u) : make_int2(0, 0); // weight 0
 #pragma unroll
             for (int u = 0; u < 4; ++u) { // the far end's word, and whether a trial flips it too
-                neg[u] = x + u < n_out ? P.O[ed[u].x + w] : myO[ed[u].x];
-                pos[u] = x + u < n_out ? 0u : myD[ed[u].x];
+                neg[u] = x + u < I.n_out ? P.O[ed[u].x + w] : myO[ed[u].x];
+                pos[u] = x + u < I.n_out ? 0u : myD[ed[u].x];
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -539,89 +664,115 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const int32_t *qlist
             }
             add_signed4<R + 1, kWeightBits>(D, pos, neg, ed);
         }
-        uint32_t nz = 0;
+        for (int off = 1; off < 1 << M.lsh; off <<= 1) { // the sums of the pair's lanes
+            uint32_t carry = 0;
 #pragma unroll
-        for (int t = 0; t <= R; ++t) nz |= D[t];
+            for (int t = 0; t <= R; ++t) {
+                const uint32_t a = D[t], b = __shfl_xor_sync(kFull, a, off);
+                D[t] = a ^ b ^ carry;
+                carry = (a & b) | (a & carry) | (b & carry);
+            }
+        }
+        uint32_t nzd = 0;
+#pragma unroll
+        for (int t = 0; t <= R; ++t) nzd |= D[t];
         const uint32_t neg = D[R];
-        const uint32_t pos = nz & ~neg;
+        const uint32_t pos = nzd & ~neg;
         const uint32_t eqv = P.eqw[(g & 1) * W + w];
-        const uint32_t acc = hd & vm & (pos | (~nz & ~eqv));
-        i_acc = __popc(acc);
-        i_imp = __popc(acc & pos);
-        i_dl = __popc(vm & ~hd);
-        L.n_acc += i_acc;
-        L.n_imp += i_imp;
-        L.n_dl += i_dl;
-        if (P.fi.on && acc) atomicOr(&P.fi.accw[w], acc); // Forced Improvement: who had an accepted step
+        const uint32_t acc = hd & (pos | (~nzd & ~eqv));
+        if (ke && M.sub == 0) {
+            i_acc = __popc(acc);
+            i_imp = __popc(acc & pos);
+            i_dl = __popc(vm & ~hd);
+            L.n_acc += i_acc;
+            L.n_imp += i_imp;
+            L.n_dl += i_dl;
+            if (P.fi.on && acc) atomicOr(&P.fi.accw[w], acc); // Forced Improvement: who had an accepted step
+        }
         if (acc) {
-            for (int a = 0; a < s; ++a) {
+            for (int a = M.sub; a < s; a += 1 << M.lsh) {
                 const uint32_t m = myD[32 * a] & acc;
                 if (m) {
-                    const int64_t v = __ldg(P.fv + f0 + a);
+                    const int64_t v = __ldg(P.fv + I.f0 + a);
                     P.O[v * W + w] = myO[32 * a] ^ m;
                 }
             }
-            fit_add<R>(L, D, acc); // the accepted deltas (>= 0, below 2^R)
+            if (M.sub == 0) fit_add<R>(L, D, acc); // the accepted deltas (>= 0, below 2^R)
         }
     }
     ++L.since_flush;
-    __syncwarp();
-    if (LEARN && P.learn) bs_record(P, q, ke, audited, g, i_acc, i_dl, i_imp, s_fc);
+    tile_sync(M); // the region may be rewritten
+    if (LEARN && P.learn) bs_record(P, I.q, ke, I.audited, g, i_acc, i_dl, i_imp, s_fc);
 }
 
-// One colour group (position t, colour c) on the bit-sliced path: items of
-// E = 32 / W consecutive elements of the group -- of the compacted list of the
-// elements to run while the learned filter skips elements; warp x takes item
-// x, then items nwarps + the claims it draws from work[t] (P.dyn), one ahead,
-// or x + nwarps, x + 2 nwarps, ... (static stride).
-template <int SB, int R, bool LEARN>
-__device__ __forceinline__ void phase_mix_bs(const GomParams &P, const VGrid &V, int t, int c, uint32_t g, uint32_t *wsm, BsLane &L,
-                             long long *s_f, unsigned long long *s_fc)
+// The elements of colour c that run: positions, or with the learned filter
+// skipping, entries of the compacted list.
+struct BsGroup {
+    const int32_t *qlist;
+    int ka, kz, items;
+};
+
+template <bool LEARN>
+__device__ __forceinline__ BsGroup bs_group(const GomParams &P, const BsMap &M, int c)
+{
+    const bool cl = LEARN && P.learn == 2 && P.flt.compact;
+    BsGroup G;
+    G.qlist = cl ? P.flt.act : nullptr;
+    G.ka = cl ? P.flt.act_ptr[c] : P.cptr[c];
+    G.kz = cl ? P.flt.act_ptr[c + 1] : P.cptr[c + 1];
+    G.items = (G.kz - G.ka + M.E - 1) / M.E;
+    return G;
+}
+
+// One colour group (position t) on the bit-sliced path: items of E consecutive
+// elements; tile x takes item x first -- prepared before `open`, the barrier
+// that opens the group (false: it gave up) --, then items ntiles + the claims
+// it draws from work[t] (P.dyn, one-warp tiles), one ahead, or x + ntiles, x +
+// 2 ntiles, ... (static stride).
+template <int SB, int R, bool LEARN, class Open>
+__device__ __forceinline__ bool phase_mix_bs(const GomParams &P, const BsMap &M, int t, int c, uint32_t g, Open open,
+                                             BsLane<FitShared> &L, long long *s_f, unsigned long long *s_fc)
 {
     const int lane = threadIdx.x & 31;
-    const int gwarp = (int)(V.thread() >> 5), nwarps = (int)(V.threads() >> 5);
-    const int E = 32 / P.W;
-    const bool cl = LEARN && P.learn == 2 && P.flt.compact;
-    const int32_t *qlist = cl ? P.flt.act : nullptr;
-    const int ka = cl ? P.flt.act_ptr[c] : P.cptr[c], kz = cl ? P.flt.act_ptr[c + 1] : P.cptr[c + 1];
-    const int items = (kz - ka + E - 1) / E;
+    const BsGroup G = bs_group<LEARN>(P, M, c);
+    const bool dyn = P.dyn && M.nwi == 1;
     unsigned claim = 0;
-    if (P.dyn && lane == 0) claim = atomicAdd(&P.work[t], 1u);
-    for (int it = gwarp, next = gwarp + nwarps; it < items;) {
-        const int k0 = ka + it * E;
-        bs_item<SB, R, LEARN>(P, qlist, k0, min(k0 + E, kz), g, wsm, L, s_f, s_fc);
-        if (P.dyn) {
-            it = nwarps + (int)__shfl_sync(0xFFFFFFFFu, claim, 0);
-            if (it < items && lane == 0) claim = atomicAdd(&P.work[t], 1u);
-        } else {
-            it = next;
-            next += nwarps;
-        }
+    BsItem<SB> I;
+    for (int it = M.tile, next = M.tile + M.ntiles, first = 1;; first = 0) { // (one call site of either part)
+        const int k0 = G.ka + it * M.E;
+        if (it < G.items) bs_prepare<SB, LEARN>(P, M, G.qlist, k0, min(k0 + M.E, G.kz), g, I);
+        if (first && !open()) return false;
+        if (it >= G.items) return true;
+        if (dyn && lane == 0) claim = atomicAdd(&P.work[t], 1u);
+        bs_item<SB, R, LEARN>(P, M, I, g, L, s_f, s_fc);
+        it = dyn ? M.ntiles + (int)__shfl_sync(kFull, claim, 0) : next;
+        next += M.ntiles;
     }
 }
 
 // Adds the warp's counters and the lanes' fitness sums into the block's
 // accumulators.
-__device__ __forceinline__ void bs_finish_generation(const GomParams &P, BsLane &L, long long *s_f,
+__device__ __forceinline__ void bs_finish_generation(const GomParams &P, BsLane<FitShared> &L, long long *s_f,
                                                      unsigned long long *s_cnt)
 {
-    bs_flush(P, L, s_f);
+    bs_flush(L, s_f);
     count_flush(s_cnt, L.n_dl, L.n_acc, L.n_imp);
     L.n_dl = L.n_acc = L.n_imp = 0;
 }
 
 // Up to G generations of one context on the bit-sliced phase, on the blocks
 // of the (virtual) grid V, the phases separated by grid barriers on `bar`:
-// [generation start + group order] | group 0 | ... | group k-1 | and again;
+// [generation start + group order] | group 0 | ... | group k-1 | and again,
+// each tile preparing its first item of a group ahead of the group's barrier;
 // every block computes a generation's end from the fitness array after the
 // barrier that closes its last group (block 0 of V records it).  s_keys: room
-// for the k group keys of the order phase (it may overlay wsm and s_f, which
-// are set up after it); wsm: this warp's region; s_f, s_cnt: the block's
+// for the k group keys of the order phase (it may overlay the regions and s_f, which
+// are set up after it); regions: the block's first warp region; s_f, s_cnt: the block's
 // fitness accumulators and counters; s_fc: the learned filter's block
 // counters (LEARN only).
 template <int SB, int R, bool LEARN>
 __device__ __forceinline__ void bs_generations(const GomParams &P, const VGrid &V, GomBarrier *bar, int G,
-                                               int64_t target, unsigned long long *s_keys, uint32_t *wsm,
+                                               int64_t target, unsigned long long *s_keys, uint32_t *regions,
                                                long long *s_f, unsigned long long *s_cnt, unsigned long long *s_fc)
 {
     const unsigned nblk = (unsigned)V.nblk;
@@ -635,8 +786,9 @@ __device__ __forceinline__ void bs_generations(const GomParams &P, const VGrid &
         P.st->target = target;
     }
     const bool tr = P.trace != nullptr && lead && threadIdx.x == 0;
-    BsLane L;
-    bs_lane_zero(L);
+    const BsMap M = bs_map<LEARN>(P, V, regions);
+    BsLane<FitShared> L;
+    L.fit.v = bs_fit(P, regions);
     for (int qg = 0; qg < G; ++qg) {
         if (qg > 0 && phase_gen_end(P, target, g - 1, e, lead)) return;
         if (tr) P.trace[0] = global_ns();
@@ -644,16 +796,21 @@ __device__ __forceinline__ void bs_generations(const GomParams &P, const VGrid &
         phase_order(P, V, s_keys, g);
         if (LEARN) fc_zero(s_fc);
         acc_zero(P, s_f, s_cnt);
+        bs_lane_zero(L, M.w); // (the order phase's keys overlay the planes)
         if (tr) P.trace[1] = P.trace[2] = global_ns();
         if (!grid_barrier(&bar->count, &P.st->err, nblk, bnext, kBarrierNs)) return;
         if (LEARN && P.learn && !phase_filter_select(P, V, g, &bar->count, nblk, bnext, P.learn == 2 && P.flt.compact))
             return;
         if (tr) P.trace[3] = global_ns();
         for (int t = 0; t < P.k; ++t) {
-            if (t > 0 && !grid_barrier(&bar->count, &P.st->err, nblk, bnext, kBarrierNs)) return;
-            if (tr) P.trace[4 + 2 * t] = global_ns();
-            phase_mix_bs<SB, R, LEARN>(P, V, t, P.order[t], g, wsm, L, s_f, s_fc);
+            const auto open = [&] {
+                if (t > 0 && !grid_wait(&bar->count, &P.st->err, nblk, bnext, kBarrierNs)) return false;
+                if (tr) P.trace[4 + 2 * t] = global_ns();
+                return true;
+            };
+            if (!phase_mix_bs<SB, R, LEARN>(P, M, t, P.order[t], g, open, L, s_f, s_fc)) return;
             if (tr) P.trace[5 + 2 * t] = global_ns();
+            if (t + 1 < P.k) grid_arrive(&bar->count);
         }
         bs_finish_generation(P, L, s_f, s_cnt);
         acc_flush(P, s_f, s_cnt);

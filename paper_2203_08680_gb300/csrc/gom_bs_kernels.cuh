@@ -16,18 +16,18 @@ namespace {
 // memory holds the block's fitness accumulators, then the warps' regions (the
 // k group keys of the order phase overlay them).
 template <int SB, int R, bool LEARN>
-__global__ void __launch_bounds__(kBsThreads, 5) k_run_bs(GomParams P, int G, int64_t target)
+__global__ void __launch_bounds__(kBsThreads, bs_blocks(SB)) k_run_bs(GomParams P, int G, int64_t target)
 {
     extern __shared__ __align__(16) uint32_t s_dyn[];
     __shared__ unsigned long long s_cnt[4], s_fc[4];
     bs_generations<SB, R, LEARN>(P, whole_grid(), P.bar, G, target, reinterpret_cast<unsigned long long *>(s_dyn),
-                             bs_warp_region(P, s_dyn), reinterpret_cast<long long *>(s_dyn), s_cnt, s_fc);
+                             s_dyn + 64 * P.W, reinterpret_cast<long long *>(s_dyn), s_cnt, s_fc);
 }
 
 // Per-launch path: the mixing of the group at position t (one launch per
 // group in the per-generation CUDA graph).
 template <int SB, int R, bool LEARN>
-__global__ void __launch_bounds__(kBsThreads, 5) k_mix_bs(GomParams P, int t)
+__global__ void __launch_bounds__(kBsThreads, bs_blocks(SB)) k_mix_bs(GomParams P, int t)
 {
     extern __shared__ __align__(16) uint32_t s_dyn[];
     __shared__ unsigned long long s_cnt[4], s_fc[4];
@@ -35,10 +35,11 @@ __global__ void __launch_bounds__(kBsThreads, 5) k_mix_bs(GomParams P, int t)
     if (P.st->done) return;
     fc_zero(s_fc);
     acc_zero(P, s_f, s_cnt);
-    BsLane L;
-    bs_lane_zero(L);
-    uint32_t *wsm = bs_warp_region(P, s_dyn);
-    phase_mix_bs<SB, R, LEARN>(P, whole_grid(), t, P.order[t], P.st->g, wsm, L, s_f, s_fc);
+    const BsMap M = bs_map<LEARN>(P, whole_grid(), s_dyn + 64 * P.W);
+    BsLane<FitShared> L;
+    L.fit.v = bs_fit(P, s_dyn + 64 * P.W);
+    bs_lane_zero(L, M.w);
+    phase_mix_bs<SB, R, LEARN>(P, M, t, P.order[t], P.st->g, [] { return true; }, L, s_f, s_fc);
     bs_finish_generation(P, L, s_f, s_cnt);
     acc_flush(P, s_f, s_cnt);
     if (LEARN) fc_flush(P, s_fc);

@@ -128,6 +128,42 @@ inline void item_split(int W, int32_t p, int64_t max_group, int64_t warps, int32
     }
 }
 
+// Lanes per pair (2^lsh) and warps per tile of the bit-sliced path for a
+// largest colour group of `max_group` elements of `wv` words on `warps` warps
+// in blocks of `wpb`: the most lanes for which the group's tiles still fit the
+// warps at once and every lane has four edges to add.  A group of few elements
+// is bound by the latency of one item, and that is mostly its serial edges.
+inline void bs_split(int wv, int64_t max_group, int64_t max_edges, int64_t warps, int wpb, int *lsh, int *nwi)
+{
+    *lsh = 0;
+    *nwi = 1;
+    for (int l = 1; l <= 5 && (int64_t(4) << (l - 1)) < max_edges; ++l) {
+        int nw = 1;
+        while (32 * nw < wv << l) nw *= 2;
+        if (nw > wpb || wpb % nw) return;
+        const int64_t E = nw > 1 ? 1 : (32 >> l) / wv;
+        if ((max_group + E - 1) / E * nw > warps) return;
+        *lsh = l;
+        *nwi = nw;
+    }
+}
+
+// Whether the bit-sliced path is the faster one where both are available, for
+// a largest colour group of `max_group` elements of wv words, the largest of
+// max_s variables, on `warps` resident bit-sliced warps.  Microseconds per
+// generation, per-lane / bit-sliced (late generations): 2D torus 100 p = 256
+// 111 / 70, p = 64 56 / 51; 3D torus 50 p = 128 1046 / 312; random 12-regular
+// 60,000 p = 512 5459 / 3372; 2D torus 300 p = 1,024 also 6 times faster.  The
+// per-lane path wins where it stages every group at once and a group is no
+// more than a few hundred words (2D torus 10 p = 16 50 / 58, 50 p = 64 58 / 62),
+// and for one-word populations of large elements that do not fill the warps
+// (linkage tree of bound 30, 100x100 torus, p = 32: 142 / 239; p = 100: 267 / 259).
+inline bool bs_pays(int wv, int64_t max_group, int64_t max_s, bool stage_all, int64_t warps)
+{
+    if (stage_all && (wv == 1 || max_group * wv <= 1024)) return false;
+    return !(wv == 1 && max_s > 16 && max_group <= 4 * warps);
+}
+
 // Raises a kernel's dynamic shared memory limit to at least `bytes`, never
 // lowers it: kernel instances are shared by every context (and batch), and a
 // limit lowered below what an existing context launches with would make its

@@ -162,28 +162,49 @@ __device__ __forceinline__ unsigned long long barrier_first(const unsigned long 
     return ld_acquire_u64(count) / nblk * nblk + nblk;
 }
 
+__device__ __forceinline__ bool barrier_poll(unsigned long long *count, int *err, unsigned nblk,
+                                             unsigned long long &next, unsigned long long limit_ns)
+{
+    volatile int *verr = err;
+    const unsigned long long target = next;
+    next += nblk;
+    const unsigned long long t0 = global_ns();
+    while (ld_acquire_u64(count) < target) {
+        if (*verr || global_ns() - t0 > limit_ns) {
+            atomicExch(err, 1);
+            return false;
+        }
+        __nanosleep(32);
+    }
+    return true;
+}
+
 __device__ bool grid_barrier(unsigned long long *count, int *err, unsigned nblk, unsigned long long &next,
                              unsigned long long limit_ns)
 {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        volatile int *verr = err;
         red_add_release_u64(count, 1ull);
-        const unsigned long long target = next;
-        next += nblk;
-        int ok = 1;
-        const unsigned long long t0 = global_ns();
-        while (ld_acquire_u64(count) < target) {
-            if (*verr || global_ns() - t0 > limit_ns) {
-                ok = 0;
-                atomicExch(err, 1);
-                break;
-            }
-            __nanosleep(32);
-        }
-        s_ok = ok;
+        s_ok = barrier_poll(count, err, nblk, next, limit_ns);
     }
+    __syncthreads();
+    return s_ok;
+}
+
+// The barrier in two halves: what a block does between them overlaps the other
+// blocks' arrival.  Both are called by every thread of the block.
+__device__ __forceinline__ void grid_arrive(unsigned long long *count)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) red_add_release_u64(count, 1ull);
+}
+
+__device__ bool grid_wait(unsigned long long *count, int *err, unsigned nblk, unsigned long long &next,
+                          unsigned long long limit_ns)
+{
+    __shared__ int s_ok;
+    if (threadIdx.x == 0) s_ok = barrier_poll(count, err, nblk, next, limit_ns);
     __syncthreads();
     return s_ok;
 }

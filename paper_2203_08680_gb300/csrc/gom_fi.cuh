@@ -93,7 +93,7 @@ __device__ void fi_start(const GomParams &P, const VGrid &V, bool newel, int aw,
 // The FI steps of one item: elements [q0, q1) of the group at position t,
 // lane = (element slot, word); s_act[w] the individuals of word w still in FI.
 template <int R>
-__device__ __forceinline__ void fi_item(const GomParams &P, int t, int q0, int q1, const uint32_t *s_act, BsLane &L,
+__device__ __forceinline__ void fi_item(const GomParams &P, int t, int q0, int q1, const uint32_t *s_act, BsLane<FitRegs> &L,
                                         unsigned (&cnt)[3], long long *s_f)
 {
     const int lane = threadIdx.x & 31;
@@ -101,7 +101,7 @@ __device__ __forceinline__ void fi_item(const GomParams &P, int t, int q0, int q
     const int lw = __ffs(W) - 1;
     const int e = lane >> lw, w = lane & (W - 1);
     const int q = q0 + e;
-    if (L.since_flush >= (1 << (kFitPlanes - R))) bs_flush(P, L, s_f);
+    if (L.since_flush >= (1 << (kFitPlanes - R))) bs_flush(L, s_f);
     ++L.since_flush;
     if (q >= q1 || w >= Wv) return;
     const uint32_t act = s_act[w];
@@ -161,7 +161,7 @@ __device__ __forceinline__ void fi_item(const GomParams &P, int t, int q0, int q
 // consecutive elements, warp x takes items x, x + nwarps, ...  The fitness
 // deltas go to the lanes' accumulators L, the counters to cnt.
 template <int R>
-__device__ void fi_group(const GomParams &P, const VGrid &V, int t, int c, const uint32_t *s_act, BsLane &L,
+__device__ void fi_group(const GomParams &P, const VGrid &V, int t, int c, const uint32_t *s_act, BsLane<FitRegs> &L,
                          unsigned (&cnt)[3], long long *s_f)
 {
     const int gwarp = (int)(V.thread() >> 5), nwarps = (int)(V.threads() >> 5);
@@ -248,8 +248,8 @@ __device__ __noinline__ bool fi_generation(const GomParams &P, const VGrid V, un
     }
     __syncthreads();
     __shared__ uint32_t s_act[32];
-    BsLane L;
-    bs_lane_zero(L);
+    BsLane<FitRegs> L;
+    bs_lane_zero(L, (threadIdx.x & 31) & (P.W - 1));
     unsigned cnt[3] = {0, 0, 0};
     for (int t = 0; t < P.k; ++t) {
         if (t > 0) {
@@ -262,7 +262,7 @@ __device__ __noinline__ bool fi_generation(const GomParams &P, const VGrid V, un
         fi_group<R>(P, V, t, order[t], s_act, L, cnt, s_f);
         __syncthreads(); // every warp has read s_act
     }
-    bs_flush(P, L, s_f);
+    bs_flush(L, s_f);
     fi_count_flush(P, cnt);
     acc_flush(P, s_f, s_cnt);
     if (!grid_barrier(bar_count, &P.st->err, nblk, bnext, kBarrierNs)) return false;

@@ -211,6 +211,8 @@ struct GomParams {
     int32_t learn;      // learned filter: 0 off, 1 history and training log, 2 also skip elements
     GomFI fi;
     int32_t bs_S;       // bit-sliced path: variables of the largest element
+    int32_t bs_lsh;     //   2^bs_lsh lanes per pair, bs_nwi warps per tile (gom_bs.cuh)
+    int32_t bs_nwi;
     int32_t bs_words;   //   shared-memory words of one warp's region
     GomFilter flt;
     uint64_t seed;

@@ -1008,14 +1008,14 @@ __device__ __noinline__ void batch_variant(const GomParams &P, const VGrid V, Go
 }
 
 // The bit-sliced variant of the batched path: the instance's generations on
-// the bit-sliced phase (gom_bs.cuh), warp w of the block in the w-th region
-// of P.bs_words words after the fitness accumulators.
+// the bit-sliced phase (gom_bs.cuh), its warps' regions of P.bs_words words
+// after the fitness accumulators.
 template <int SB, int R>
 __device__ __noinline__ void batch_variant_bs(const GomParams &P, const VGrid V, GomBarrier *bar, int G,
                                               int64_t target, const RunShared &S)
 {
     bs_generations<SB, R, false>(P, V, bar, G, target, reinterpret_cast<unsigned long long *>(S.dyn),
-                             S.dyn + (threadIdx.x >> 5) * P.bs_words, S.f, S.cnt, nullptr);
+                             S.dyn, S.f, S.cnt, nullptr);
 }
 
 // Batched path: many independent instances in one cooperative launch.  Each
