@@ -13,6 +13,7 @@
 #include "gom_ctx.h"
 #include "gom_internal.h"
 #include "gom_kernels.cuh"
+#include "gom_rows.cuh"
 
 namespace {
 
@@ -574,10 +575,9 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
     // dynamic item claims: faster warps take more items (in stage-all mode
     // every warp has at most one item per group and the schedule is moot)
     c->prm.dyn = 1;
-    const int blk_mult = std::max(1, c->W / 8);
-    c->grid_fit = std::max(blk_mult, c->sms * 4 / blk_mult * blk_mult);
+    c->grid_fit = cut_grid(c->n, c->p, 256, c->sms * 2);
     c->grid_start = c->sms * 4;
-    c->grid_io = c->sms * 4;
+    c->grid_io = c->sms * 8;
     c->grid_order = (c->k + 255) / 256;
     c->order_smem = sizeof(unsigned long long) * std::max(c->k, 1);
     if (c->order_smem > 48 * 1024)
@@ -748,7 +748,7 @@ int gom_get_population(gom_ctx_t *ctx, uint8_t *d_pop, int64_t *d_fit, int64_t *
 {
     if (!ctx) return GOM_E_ARG;
     if (d_pop) {
-        k_export_pop<<<ctx->grid_io, 256, 0, ctx->stream>>>(ctx->prm, d_pop);
+        k_export_pop<<<ctx->grid_io, kRowThreads, 0, ctx->stream>>>(ctx->prm, d_pop);
         GOM_CUDA(ctx, cudaGetLastError());
     }
     if (d_fit)
@@ -777,12 +777,9 @@ int gom_set_population(gom_ctx_t *ctx, const uint8_t *d_pop, const uint8_t *d_el
                        int64_t generation)
 {
     if (!ctx || !d_pop || !d_elite || generation < 0 || generation > UINT32_MAX) return GOM_E_ARG;
-    k_import_pop<<<ctx->grid_io, 256, 0, ctx->stream>>>(ctx->prm, d_pop, d_elite);
+    k_import_pop<<<ctx->grid_io, kRowThreads, 0, ctx->stream>>>(ctx->prm, d_pop, d_elite, elite_f, generation);
     GOM_CUDA(ctx, cudaGetLastError());
-    GOM_CUDA(ctx, cudaMemsetAsync(ctx->prm.f, 0, sizeof(int64_t) * 32 * ctx->W, ctx->stream));
     k_fitness<<<ctx->grid_fit, 256, 0, ctx->stream>>>(ctx->prm, ctx->prm.f);
-    GOM_CUDA(ctx, cudaGetLastError());
-    k_set_state<<<1, 256, 0, ctx->stream>>>(ctx->prm, elite_f, generation);
     GOM_CUDA(ctx, cudaGetLastError());
     return GOM_OK;
 }

@@ -26,6 +26,7 @@
 #include "gom_filter_dev.cuh"
 #include "gom_internal.h"
 #include "gom_kernels.cuh"
+#include "gom_rows.cuh"
 
 
 // ----------------------------------------------------------------------------
@@ -60,29 +61,11 @@ __global__ void k_init_pop(GomParams P)
     }
 }
 
-// Full evaluation (Sec. 6.2): f[i] = sum over edges {u<v} of w_uv [x_u != x_v].
-// A warp takes chunks of 32 vertices for one word; lane = individual.
-// The number of warps in the grid is a multiple of W.
-__global__ void k_fitness(GomParams P, int64_t *out)
+// Full evaluation (Sec. 6.2) of the population, added into out[p].
+__global__ void __launch_bounds__(256, 2) k_fitness(GomParams P, int64_t *out)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = gthread() >> 5, nwarps = gthreads() >> 5;
-    const int w = (int)(warp & (P.W - 1));
-    if (w >= P.Wv) return;
-    const int64_t nchunks = (P.n + 31) / 32;
-    long long acc = 0;
-    for (int64_t ch = warp / P.W; ch < nchunks; ch += nwarps / P.W) {
-        const int64_t uend = min((int64_t)P.n, 32 * ch + 32);
-        for (int64_t u = 32 * ch; u < uend; ++u) {
-            const uint32_t xu = P.O[u * P.W + w];
-            for (int64_t e = P.row_ptr[u]; e < P.row_ptr[u + 1]; ++e) {
-                const int64_t v = P.col[e];
-                if (v > u && (((xu ^ P.O[v * P.W + w]) >> lane) & 1u)) acc += P.wgt[e];
-            }
-        }
-    }
-    const int i = 32 * w + lane;
-    if (i < P.p && acc) atomicAdd((unsigned long long *)&out[i], (unsigned long long)acc);
+    __shared__ long long s_f[1024], s_const;
+    cut_sums(P.O, P.n, P.p, P.W, P.row_ptr, P.col, P.wgt, s_f, &s_const, out);
 }
 
 // Elitist of a fresh population: lowest index of maximal fitness.
@@ -97,21 +80,6 @@ __global__ void k_elite_init(GomParams P)
         P.st->argmax = arg;
         P.st->improved = 1;
         P.st->done = 0;
-    }
-    for (int w = threadIdx.x; w < 2 * P.W; w += blockDim.x) P.eqw[w] = kFull;
-}
-
-// State after an import: given elitist fitness and generation counter.
-__global__ void k_set_state(GomParams P, int64_t fe, int64_t g)
-{
-    if (threadIdx.x == 0) {
-        P.st->fe = fe;
-        P.st->best = fe;
-        P.st->argmax = 0;
-        P.st->improved = 0;
-        P.st->done = 0;
-        P.st->g = (uint32_t)g;
-        P.st->cnt[0] = P.st->cnt[1] = P.st->cnt[2] = P.st->cnt[3] = 0;
     }
     for (int w = threadIdx.x; w < 2 * P.W; w += blockDim.x) P.eqw[w] = kFull;
 }
@@ -1163,13 +1131,10 @@ const void *gom_run_kernel(int wpi, int variant, bool learn)
 
 // ----------------------------------------------------------------------------
 // uint8 rows out[i*n + v] of the population.
-__global__ void k_export_pop(GomParams P, uint8_t *out)
+__global__ void __launch_bounds__(kRowThreads) k_export_pop(GomParams P, uint8_t *out)
 {
-    const int64_t total = (int64_t)P.p * P.n;
-    for (int64_t idx = gthread(); idx < total; idx += gthreads()) {
-        const int64_t i = idx / P.n, v = idx - i * P.n;
-        out[idx] = (uint8_t)((P.O[v * P.W + (i >> 5)] >> (i & 31)) & 1u);
-    }
+    __shared__ __align__(16) uint32_t sm[row_words(32)];
+    unpack_rows(P.O, P.n, P.p, P.W, out, sm);
 }
 
 __global__ void k_export_elite(GomParams P, uint8_t *out)
@@ -1180,19 +1145,25 @@ __global__ void k_export_elite(GomParams P, uint8_t *out)
         out[v] = improved ? (uint8_t)((P.O[v * P.W + aw] >> ab) & 1u) : P.xe[v];
 }
 
-// Packs uint8 rows in[i*n + v] into the bit-sliced O and copies the elitist.
-__global__ void k_import_pop(GomParams P, const uint8_t *in, const uint8_t *elite)
+// Packs uint8 rows in[i*n + v] into the bit-sliced O, copies the elitist, and
+// sets the state of an import: the given elitist fitness and generation
+// counter, the fitness array zeroed for the evaluation that follows.
+__global__ void __launch_bounds__(kRowThreads) k_import_pop(GomParams P, const uint8_t *in, const uint8_t *elite,
+                                                            int64_t fe, int64_t g)
 {
-    const int64_t total = (int64_t)P.n * P.W;
-    for (int64_t idx = gthread(); idx < total; idx += gthreads()) {
-        const int64_t v = idx / P.W;
-        const int w = (int)(idx - v * P.W);
-        uint32_t word = 0;
-        for (int b = 0; b < 32; ++b) {
-            const int64_t i = 32 * w + b;
-            if (i < P.p && in[i * P.n + v]) word |= 1u << b;
-        }
-        P.O[idx] = word;
-        if (w == 0) P.xe[v] = elite[v] ? 1 : 0;
+    __shared__ __align__(16) uint32_t sm[row_words(32)];
+    pack_rows(in, P.n, P.p, P.W, P.O, sm);
+    for (int64_t v = gthread(); v < P.n; v += gthreads()) P.xe[v] = elite[v] ? 1 : 0;
+    if (blockIdx.x > 0) return;
+    if (threadIdx.x == 0) {
+        P.st->fe = fe;
+        P.st->best = fe;
+        P.st->argmax = 0;
+        P.st->improved = 0;
+        P.st->done = 0;
+        P.st->g = (uint32_t)g;
+        P.st->cnt[0] = P.st->cnt[1] = P.st->cnt[2] = P.st->cnt[3] = 0;
     }
+    for (int w = threadIdx.x; w < 2 * P.W; w += blockDim.x) P.eqw[w] = kFull;
+    for (int i = threadIdx.x; i < 32 * P.W; i += blockDim.x) P.f[i] = 0;
 }

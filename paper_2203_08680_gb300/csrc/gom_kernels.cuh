@@ -9,7 +9,6 @@
 __global__ void k_init_pop(GomParams P);
 __global__ void k_fitness(GomParams P, int64_t *out);
 __global__ void k_elite_init(GomParams P);
-__global__ void k_set_state(GomParams P, int64_t fe, int64_t g);
 __global__ void k_begin_call(GomParams P, int64_t target);
 __global__ void k_gen_start(GomParams P);
 __global__ void k_order(GomParams P);
@@ -61,4 +60,4 @@ __global__ void k_filter_scan(GomParams P, int nwarps);
 __global__ void k_filter_compact(GomParams P);
 __global__ void k_export_pop(GomParams P, uint8_t *out);
 __global__ void k_export_elite(GomParams P, uint8_t *out);
-__global__ void k_import_pop(GomParams P, const uint8_t *in, const uint8_t *elite);
+__global__ void k_import_pop(GomParams P, const uint8_t *in, const uint8_t *elite, int64_t fe, int64_t g);

@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/gom.h"
+#include "gom_rows.cuh"
 
 namespace {
 
@@ -87,53 +88,21 @@ cudaError_t scratch_address(uint32_t **out)
     return cudaSuccess;
 }
 
-// Packs pop[i*n + v] (uint8 {0,1}) into words[v*W + w], bit b = individual
-// 32w + b; bits of individuals >= p are zero, so every word is rewritten.  A
-// warp takes 32 variables of one word: lane l owns variable v0 + l, and for
-// each of the 32 individuals the warp reads 32 consecutive bytes of its row.
-__global__ void k_noalloc_pack(const uint8_t *pop, int32_t n, int32_t p, int32_t W, uint32_t *words)
+__global__ void __launch_bounds__(kRowThreads)
+    k_noalloc_pack(const uint8_t *pop, int32_t n, int32_t p, int32_t W, uint32_t *words, int64_t *fit)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
-    const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-    const int64_t nchunks = (n + 31) / 32;
-    for (int64_t it = warp; it < nchunks * W; it += nwarps) {
-        const int64_t v = 32 * (it / W) + lane;
-        const int w = static_cast<int>(it % W);
-        uint32_t word = 0;
-        if (v < n) {
-            const int bmax = p - 32 * w < 32 ? p - 32 * w : 32;
-            for (int b = 0; b < bmax; ++b)
-                if (pop[(32 * static_cast<int64_t>(w) + b) * n + v]) word |= 1u << b;
-            words[v * W + w] = word;
-        }
-    }
+    __shared__ __align__(16) uint32_t sm[row_words(32)];
+    pack_rows(pop, n, p, W, words, sm);
+    if (blockIdx.x == 0)
+        for (int i = threadIdx.x; i < p; i += blockDim.x) fit[i] = 0; // for the sums that follow
 }
 
-// fit[i] += sum over edges {u < v} of w_uv [x_u != x_v] (the cut weight):
-// warps take 32-vertex chunks of one word, lane = individual.  The warp
-// count of the grid is a multiple of W.
-__global__ void k_noalloc_cut(const uint32_t *words, int32_t n, int32_t p, int32_t W, const int64_t *row_ptr,
-                              const int32_t *col, const int32_t *wgt, int64_t *fit)
+__global__ void __launch_bounds__(256, 2)
+    k_noalloc_cut(const uint32_t *words, int32_t n, int32_t p, int32_t W, const int64_t *row_ptr, const int32_t *col,
+                  const int32_t *wgt, int64_t *fit)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
-    const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-    const int w = static_cast<int>(warp % W);
-    const int64_t nchunks = (n + 31) / 32;
-    long long acc = 0;
-    for (int64_t ch = warp / W; ch < nchunks; ch += nwarps / W) {
-        const int64_t uend = ch * 32 + 32 < n ? ch * 32 + 32 : n;
-        for (int64_t u = 32 * ch; u < uend; ++u) {
-            const uint32_t xu = words[u * W + w];
-            for (int64_t e = row_ptr[u]; e < row_ptr[u + 1]; ++e) {
-                const int64_t v = col[e];
-                if (v > u && (((xu ^ words[v * W + w]) >> lane) & 1u)) acc += wgt[e];
-            }
-        }
-    }
-    const int64_t i = 32 * static_cast<int64_t>(w) + lane;
-    if (i < p && acc) atomicAdd(reinterpret_cast<unsigned long long *>(&fit[i]), static_cast<unsigned long long>(acc));
+    __shared__ long long s_f[1024], s_const;
+    cut_sums(words, n, p, W, row_ptr, col, wgt, s_f, &s_const, fit);
 }
 
 } // namespace
@@ -151,18 +120,13 @@ extern "C" int gom_fitness_noalloc(const int64_t *d_row_ptr, const int32_t *d_co
     uint32_t *scratch = nullptr;
     if (scratch_address(&scratch) != cudaSuccess) return GOM_E_CUDA;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    if (cudaMemsetAsync(d_fitness_out, 0, sizeof(int64_t) * pop, s) != cudaSuccess) return GOM_E_CUDA;
-    const int64_t pack_warps = (num_vertices + 31) / 32 * W;
-    const int pack_grid = static_cast<int>((pack_warps + 7) / 8 < 4096 ? (pack_warps + 7) / 8 : 4096);
-    k_noalloc_pack<<<pack_grid, 256, 0, s>>>(d_pop, num_vertices, pop, W, scratch);
+    // eight (four) resident blocks a SM cover a GB300; fewer where the problem is small
+    const int64_t tiles = (num_vertices + kRowVars - 1) / kRowVars / row_tiles(W) + 1;
+    k_noalloc_pack<<<static_cast<int>(tiles < 1216 ? tiles : 1216), kRowThreads, 0, s>>>(d_pop, num_vertices, pop, W, scratch,
+                                                                                      d_fitness_out);
     if (cudaGetLastError() != cudaSuccess) return GOM_E_CUDA;
-    // 8 warps per block; the block count is a multiple of W / 8 so the warp count is a multiple of W
-    const int mult = W > 8 ? W / 8 : 1;
-    int cut_grid = static_cast<int>(((num_vertices + 31) / 32 * W + 7) / 8);
-    cut_grid = cut_grid < 1024 ? cut_grid : 1024;
-    cut_grid = (cut_grid + mult - 1) / mult * mult;
-    k_noalloc_cut<<<cut_grid, 256, 0, s>>>(scratch, num_vertices, pop, W, d_row_ptr, d_col, d_weight,
-                                           d_fitness_out);
+    k_noalloc_cut<<<cut_grid(num_vertices, pop, 256, 304), 256, 0, s>>>(scratch, num_vertices, pop, W, d_row_ptr, d_col,
+                                                                        d_weight, d_fitness_out);
     if (cudaGetLastError() != cudaSuccess) return GOM_E_CUDA;
     return GOM_OK;
 }
