@@ -95,7 +95,10 @@ extern "C" {
                                either way; the learned filter works on both.  A batched launch
                                follows the value the caller set for the context, else runs
                                bit-sliced the instances whose largest group gives each of their
-                               warps four (element, word) pairs or more (only with min_blocks 2) */
+                               warps four (element, word) pairs or more (only with min_blocks 2).
+                               Weights up to 65,535 with element sums below 2^20 run on bit-planes
+                               by default as well; there the option reads 0 and can only be set
+                               to 0 (the per-lane mixing) */
 
 #define GOM_OPT_FORCED_IMPROVEMENT 5 /* 1: Forced Improvement (Sec. 4, Alg. 1) after each generation's
                                         mixing, in this library's parallel reading (the paper's

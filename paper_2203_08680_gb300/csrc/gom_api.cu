@@ -512,9 +512,8 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
         const int32_t *h = tabs.hdr.data() + 8 * q;
         c->sum_se += (h[3] & 0xFF) + (h[3] >> 8) + h[4];
     }
-    // the bit-sliced path: elements of <= 32 variables, |w| <= 255, element
-    // sums of |w| below 2^16 (R-bit plane accumulators, R = 12 or 16); an item
-    // is E = 32 / W elements, one pair (element, word) per lane
+    // the bit-sliced path: elements of <= 32 variables, weights and element
+    // sums of |w| within its instances' planes (bs_planes)
     int64_t max_w = 0;
     for (int64_t x = 0; x < g->num_adj; ++x) max_w = std::max<int64_t>(max_w, std::llabs(g->weight[x]));
     // Forced Improvement works on bit-planes too: |w| <= 255 and element sums of |w| below 2^16
@@ -526,30 +525,35 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
         c->fi_grid = std::max(1, c->sms * std::max(occ_f, 1));
     }
     {
-        const int R = tabs.max_abs_w < (int64_t(1) << 12) ? 12 : 16;
-        if (coop && variant == kVarNarrow && max_w <= 255 && tabs.max_abs_w < (int64_t(1) << 16)) {
+        int R = 0, UB = 0;
+        if (coop && variant == kVarNarrow && bs_planes(max_w, tabs.max_abs_w, &R, &UB)) {
             const int S = static_cast<int>(std::max<int64_t>(tabs.max_s, 1));
             const int64_t ww = gom_bs_warp_words(S);
             const int wpb = static_cast<int>(std::min<int64_t>(kBsThreads / 32, kSmemBudget / (ww * 4)));
             // the block's fitness accumulators (32 W int64), then the warps' regions
             const size_t smem = std::max(static_cast<size_t>(256 * c->W + ww * 4 * wpb), keys_smem);
             // the kernels without the learned filter's code, and with it (same grids)
-            const void *rf = gom_run_bs_kernel(S, R, false), *mf = gom_mix_bs_kernel(S, R, false);
-            const void *rfl = gom_run_bs_kernel(S, R, true), *mfl = gom_mix_bs_kernel(S, R, true);
-            if (wpb >= 1 && smem <= static_cast<size_t>(kSmemBudget) && rf && mf && rfl && mfl) {
+            const void *rf = gom_run_bs_kernel(S, R, UB, false), *mf = gom_mix_bs_kernel(S, R, UB, false);
+            const void *rfl = gom_run_bs_kernel(S, R, UB, true), *mfl = gom_mix_bs_kernel(S, R, UB, true);
+            if (wpb >= 1 && smem <= static_cast<size_t>(kSmemBudget)) {
                 const int E = 32 / wv;
                 const int64_t items = (max_group + E - 1) / E;
-                for (const void *fn : {rf, mf, rfl, mfl}) GOM_CUDA(c, raise_smem_limit(fn, smem));
+                for (const void *fn : {rf, mf, rfl, mfl})
+                    if (fn) GOM_CUDA(c, raise_smem_limit(fn, smem));
                 int occ_r = 0, occ_m = 0, occ_rl = 0, occ_ml = 0;
                 GOM_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_r, rf, 32 * wpb, smem));
                 GOM_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_m, mf, 32 * wpb, smem));
-                GOM_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_rl, rfl, 32 * wpb, smem));
-                GOM_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_ml, mfl, 32 * wpb, smem));
-                occ_r = std::min(occ_r, occ_rl);
-                occ_m = std::min(occ_m, occ_ml);
+                if (rfl && mfl) { // (8-bit weights)
+                    GOM_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_rl, rfl, 32 * wpb, smem));
+                    GOM_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_ml, mfl, 32 * wpb, smem));
+                    occ_r = std::min(occ_r, occ_rl);
+                    occ_m = std::min(occ_m, occ_ml);
+                }
                 if (occ_r > 0 && occ_m > 0) {
                     c->bs_r = R;
-                    c->bs_ok = true;
+                    c->bs_ub = UB;
+                    c->bs_can = true;
+                    c->bs_ok = UB == 8;
                     c->run_bs_fn = rf;
                     c->mix_bs_fn = mf;
                     c->bs_smem = smem;
@@ -658,7 +662,7 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
     GOM_CUDA(c, upload(base, L.dep, tabs.dep, s));
     GOM_CUDA(c, upload(base, L.cptr, cptr32, s));
 
-    if (c->bs_ok) {
+    if (c->bs_can) {
         k_bs_edges<<<c->grid_io, 256, 0, s>>>(P, reinterpret_cast<int2 *>(base + L.bdep));
         GOM_CUDA(c, cudaGetLastError());
     }
@@ -901,7 +905,7 @@ int gom_get_option(gom_ctx_t *ctx, int32_t option, int64_t *value)
         return GOM_OK;
     }
     if (option == GOM_OPT_BITSLICED) {
-        *value = ctx->bs_on ? 1 : 0;
+        *value = ctx->bs_on && ctx->bs_ok ? 1 : 0;
         return GOM_OK;
     }
     if (option == GOM_OPT_FORCED_IMPROVEMENT) {

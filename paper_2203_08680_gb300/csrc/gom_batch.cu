@@ -95,7 +95,7 @@ double instance_cost(const gom_ctx *c, int item_cost, bool bits)
 // 2.1 against 7.2, and 3.1 with those below eight left per lane).
 bool batch_bits(const gom_ctx *c, const gom_batch_config_t &conf, int64_t warps)
 {
-    if (!c->bs_ok || conf.min_blocks != 2) return false;
+    if (!c->bs_can || conf.min_blocks != 2) return false;
     if (c->bs_set >= 0) return c->bs_set == 1;
     return c->max_group * ((c->p + 31) / 32) >= 4 * warps;
 }
@@ -178,7 +178,7 @@ int gom_batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config
                 slice_layout(c->max_s, c->max_edges, c->W, wpi, c->variant, split != 0, (wv + wpi - 1) / wpi);
             max_warp_words = std::max<int64_t>(max_warp_words, SL.base_words);
         }
-        if (c->bs_ok && conf.min_blocks == 2) // a bit-sliced warp region
+        if (c->bs_can && conf.min_blocks == 2) // a bit-sliced warp region
             max_warp_words = std::max<int64_t>(max_warp_words, c->prm.bs_words);
     }
     const int32_t f_words = 2 * 32 * maxW;
@@ -249,7 +249,7 @@ int gom_batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config
         P.fi.on = 0; // nor Forced Improvement (refused above)
         P.bar = B->d_bars + b; // (P.trace: the context's phase trace, when switched on)
         // (one-warp tiles: the blocks' named barriers are left to the block-mode instances)
-        if (c->bs_ok) bs_split(wv, c->max_group, c->max_edges, int64_t(nb[b]) * conf.warps_per_block, 1, &P.bs_lsh, &P.bs_nwi);
+        if (c->bs_can) bs_split(wv, c->max_group, c->max_edges, int64_t(nb[b]) * conf.warps_per_block, 1, &P.bs_lsh, &P.bs_nwi);
         B->params[b] = P;
         GomBatchInst &I = B->inst[b];
         I = GomBatchInst{};
@@ -261,6 +261,7 @@ int gom_batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config
         if (use_bs) {
             I.variant = kVarBits;
             I.bs_r = c->bs_r;
+            I.bs_ub = c->bs_ub;
         }
         I.target = INT64_MAX;
         blk += nb[b];

@@ -14,7 +14,29 @@
 namespace {
 
 constexpr int kFitPlanes = 24;  // bits of the per-lane bit-sliced fitness accumulator
-constexpr int kWeightBits = 8;  // |w| < 2^8 on this path
+constexpr int kWeightBits = 8;  // |w| < 2^8 in Forced Improvement
+
+// Transposes the NR x NR bit blocks of NR registers inside the lane (NR = 8:
+// four blocks, one per byte column; 16: two; 32: one): bit NR c + r of x[a]
+// on entry is bit NR c + a of x[r] on return.  log2(NR) steps; step j swaps
+// the off-diagonal j x j blocks of each 2j x 2j block.  3 * 4 * 4 = 48
+// instructions transpose 8 variables of 32 individuals in each of 32 lanes,
+// where shuffle transposes across the warp took 15 for one word of 32
+// individuals, used 20 of 32 rows, and kept the shuffle unit busy.
+template <int NR, int J = NR / 2>
+__device__ __forceinline__ void transpose_lane(uint32_t (&x)[NR])
+{
+    constexpr uint32_t m = J == 16 ? 0x0000FFFFu : J == 8 ? 0x00FF00FFu : J == 4 ? 0x0F0F0F0Fu : J == 2 ? 0x33333333u
+                                                                                                    : 0x55555555u;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        if (r & J) continue;
+        const uint32_t a = x[r], b = x[r + J];
+        x[r] = (a & m) | ((b << J) & ~m);
+        x[r + J] = ((a >> J) & m) | (b & ~m);
+    }
+    if constexpr (J > 1) transpose_lane<NR, J / 2>(x); // (a loop over J would stay a loop, with x in local memory)
+}
 
 // x & (bit t of u ? ~0 : 0), for a per-lane weight u.
 __device__ __forceinline__ uint32_t bit_mask(uint32_t x, uint32_t u, int t) { return ((u >> t) & 1u) ? x : 0u; }
@@ -142,27 +164,42 @@ __device__ __forceinline__ void bs_lane_zero(BsLane<Fit> &L, int w)
     L.n_dl = L.n_acc = L.n_imp = 0;
 }
 
+// The 32 numbers whose planes x[0 .. kFitPlanes) are, each added into f[b].
+__device__ __forceinline__ void planes_add(uint32_t (&x)[32], long long *f)
+{
+    transpose_lane<32>(x);
+#pragma unroll
+    for (int b = 0; b < 32; ++b)
+        if (x[b]) atomicAdd(reinterpret_cast<unsigned long long *>(&f[b]), (unsigned long long)x[b]);
+}
+
 // Adds the lane's accumulated deltas into the block's fitness accumulators
 // s_f[32 w + b] (one shared atomic per individual with a non-zero sum) and
-// clears them.  Warp-wide call.
-template <class Fit>
-__device__ __forceinline__ void bs_flush(BsLane<Fit> &L, long long *s_f)
+// clears them.
+__device__ __forceinline__ void bs_flush(BsLane<FitRegs> &L, long long *s_f)
 {
-    const int w = L.w;
-    uint32_t any = 0;
+    uint32_t x[32];
 #pragma unroll
-    for (int t = 0; t < kFitPlanes; ++t) any |= L.fit.get(t);
-    if (any) {
-        for (int b = 0; b < 32; ++b) {
-            if (!((any >> b) & 1u)) continue;
-            unsigned v = 0;
+    for (int t = 0; t < 32; ++t) x[t] = t < kFitPlanes ? L.fit.v[t < kFitPlanes ? t : 0] : 0u;
+    planes_add(x, s_f + 32 * L.w);
 #pragma unroll
-            for (int t = 0; t < kFitPlanes; ++t) v |= ((L.fit.get(t) >> b) & 1u) << t;
-            atomicAdd(reinterpret_cast<unsigned long long *>(&s_f[32 * w + b]), (unsigned long long)v);
-        }
-    }
+    for (int t = 0; t < kFitPlanes; ++t) L.fit.v[t] = 0;
+    L.since_flush = 0;
+}
+
+__device__ __noinline__ void bs_flush_shared(uint32_t *v, long long *f)
+{
+    uint32_t x[32];
 #pragma unroll
-    for (int t = 0; t < kFitPlanes; ++t) L.fit.set(t, 0);
+    for (int t = 0; t < 32; ++t) x[t] = t < kFitPlanes ? v[32 * t] : 0u;
+    planes_add(x, f);
+#pragma unroll
+    for (int t = 0; t < kFitPlanes; ++t) v[32 * t] = 0;
+}
+
+__device__ __forceinline__ void bs_flush(BsLane<FitShared> &L, long long *s_f)
+{
+    bs_flush_shared(L.fit.v, s_f + 32 * L.w);
     L.since_flush = 0;
 }
 

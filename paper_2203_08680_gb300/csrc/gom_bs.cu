@@ -83,7 +83,7 @@ __global__ void k_bs_edges(GomParams P, int2 *bdep)
     for (int64_t q = gthread(); q < P.m; q += gthreads()) {
         const int4 h0 = P.hdr[2 * q], h1 = P.hdr[2 * q + 1];
         const int f0 = h0.y, d0 = h0.z, s = h0.w & 0xFF, n_in = h0.w >> 8, n_out = h1.x;
-        const auto pack = [](int a, int w) { // |w| <= 255 where the path is available
+        const auto pack = [](int a, int w) { // |w| < 2^16 where the path is available
             const uint32_t mag = (uint32_t)(w < 0 ? -w : w);
             return (int)((uint32_t)(32 * a) << kEdgeRow | mag << kEdgeWeight | (w < 0 ? 0x80000000u : 0u));
         };
@@ -109,14 +109,16 @@ const void *gom_fi_kernel(int which, int r)
     }
 }
 
-const void *gom_run_bs_kernel(int s, int r, bool learn)
+const void *gom_run_bs_kernel(int s, int r, int ub, bool learn)
 {
-    return bs_class(s) == 8 ? gom_run_bs8(r, learn) : bs_class(s) == 16 ? gom_run_bs16(r, learn) : gom_run_bs32(r, learn);
+    const int c = bs_class(s);
+    return c == 8 ? gom_run_bs8(r, ub, learn) : c == 16 ? gom_run_bs16(r, ub, learn) : gom_run_bs32(r, ub, learn);
 }
 
-const void *gom_mix_bs_kernel(int s, int r, bool learn)
+const void *gom_mix_bs_kernel(int s, int r, int ub, bool learn)
 {
-    return bs_class(s) == 8 ? gom_mix_bs8(r, learn) : bs_class(s) == 16 ? gom_mix_bs16(r, learn) : gom_mix_bs32(r, learn);
+    const int c = bs_class(s);
+    return c == 8 ? gom_mix_bs8(r, ub, learn) : c == 16 ? gom_mix_bs16(r, ub, learn) : gom_mix_bs32(r, ub, learn);
 }
 
 int gom_bs_warp_words(int s) { return bs_warp_words(s); }

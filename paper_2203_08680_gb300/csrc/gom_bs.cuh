@@ -61,9 +61,11 @@
 // colouring), so the rows a pair reads and writes belong to it alone during
 // the group.
 //
-// The path takes elements of at most 32 variables, |w| <= 255, and elements
-// whose sum of |w| over their edges is below 2^R (R = 12 or 16, the width of
-// the bit-plane accumulators); the host selects it only then.
+// The path takes elements of at most 32 variables, |w| < 2^UB, and elements
+// whose sum of |w| over their edges is below 2^R, the width of the bit-plane
+// accumulators: (R, UB) = (12, 8), (16, 8), (16, 12) or (20, 16); the host
+// selects it only then.  (The last two took a generation of the 317x317 torus
+// with weights in [-1000, 1000], p = 100, from 700 us per lane to 182 us.)
 #pragma once
 
 #include <climits>
@@ -76,28 +78,6 @@
 #include "gom_internal.h"
 
 namespace {
-
-// Transposes the NR x NR bit blocks of NR registers inside the lane (NR = 8:
-// four blocks, one per byte column; 16: two; 32: one): bit NR c + r of x[a]
-// on entry is bit NR c + a of x[r] on return.  log2(NR) steps; step j swaps
-// the off-diagonal j x j blocks of each 2j x 2j block.  3 * 4 * 4 = 48
-// instructions transpose 8 variables of 32 individuals in each of 32 lanes,
-// where shuffle transposes across the warp took 15 for one word of 32
-// individuals, used 20 of 32 rows, and kept the shuffle unit busy.
-template <int NR, int J = NR / 2>
-__device__ __forceinline__ void transpose_lane(uint32_t (&x)[NR])
-{
-    constexpr uint32_t m = J == 16 ? 0x0000FFFFu : J == 8 ? 0x00FF00FFu : J == 4 ? 0x0F0F0F0Fu : J == 2 ? 0x33333333u
-                                                                                                    : 0x55555555u;
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-        if (r & J) continue;
-        const uint32_t a = x[r], b = x[r + J];
-        x[r] = (a & m) | ((b << J) & ~m);
-        x[r + J] = ((a >> J) & m) | (b & ~m);
-    }
-    if constexpr (J > 1) transpose_lane<NR, J / 2>(x); // (a loop over J would stay a loop, with x in local memory)
-}
 
 // Brings the 128-byte line holding *ptr into L2 (a hint: no data returned).
 __device__ __forceinline__ void prefetch_l2(const void *ptr)
@@ -483,7 +463,7 @@ __device__ __forceinline__ void bs_prepare(const GomParams &P, const BsMap &M, c
 
 // Second part of an item, in its group: the parent's rows, the flip planes,
 // the partial evaluation, acceptance and writes of all its trials (Alg. 2).
-template <int SB, int R, bool LEARN>
+template <int SB, int R, int UB, bool LEARN>
 __device__ __forceinline__ void bs_item(const GomParams &P, const BsMap &M, const BsItem<SB> &I, uint32_t g,
                                         BsLane<FitShared> &L, long long *s_f, unsigned long long *s_fc)
 {
@@ -662,7 +642,7 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const BsMap &M, cons
                 pos[u] = tg & ~cut;
                 neg[u] = tg & cut;
             }
-            add_signed4<R + 1, kWeightBits>(D, pos, neg, ed);
+            add_signed4<R + 1, UB>(D, pos, neg, ed);
         }
         for (int off = 1; off < 1 << M.lsh; off <<= 1) { // the sums of the pair's lanes
             uint32_t carry = 0;
@@ -729,7 +709,7 @@ __device__ __forceinline__ BsGroup bs_group(const GomParams &P, const BsMap &M, 
 // that opens the group (false: it gave up) --, then items ntiles + the claims
 // it draws from work[t] (P.dyn, one-warp tiles), one ahead, or x + ntiles, x +
 // 2 ntiles, ... (static stride).
-template <int SB, int R, bool LEARN, class Open>
+template <int SB, int R, int UB, bool LEARN, class Open>
 __device__ __forceinline__ bool phase_mix_bs(const GomParams &P, const BsMap &M, int t, int c, uint32_t g, Open open,
                                              BsLane<FitShared> &L, long long *s_f, unsigned long long *s_fc)
 {
@@ -744,7 +724,7 @@ __device__ __forceinline__ bool phase_mix_bs(const GomParams &P, const BsMap &M,
         if (first && !open()) return false;
         if (it >= G.items) return true;
         if (dyn && lane == 0) claim = atomicAdd(&P.work[t], 1u);
-        bs_item<SB, R, LEARN>(P, M, I, g, L, s_f, s_fc);
+        bs_item<SB, R, UB, LEARN>(P, M, I, g, L, s_f, s_fc);
         it = dyn ? M.ntiles + (int)__shfl_sync(kFull, claim, 0) : next;
         next += M.ntiles;
     }
@@ -770,7 +750,7 @@ __device__ __forceinline__ void bs_finish_generation(const GomParams &P, BsLane<
 // are set up after it); regions: the block's first warp region; s_f, s_cnt: the block's
 // fitness accumulators and counters; s_fc: the learned filter's block
 // counters (LEARN only).
-template <int SB, int R, bool LEARN>
+template <int SB, int R, int UB, bool LEARN>
 __device__ __forceinline__ void bs_generations(const GomParams &P, const VGrid &V, GomBarrier *bar, int G,
                                                int64_t target, unsigned long long *s_keys, uint32_t *regions,
                                                long long *s_f, unsigned long long *s_cnt, unsigned long long *s_fc)
@@ -808,7 +788,7 @@ __device__ __forceinline__ void bs_generations(const GomParams &P, const VGrid &
                 if (tr) P.trace[4 + 2 * t] = global_ns();
                 return true;
             };
-            if (!phase_mix_bs<SB, R, LEARN>(P, M, t, P.order[t], g, open, L, s_f, s_fc)) return;
+            if (!phase_mix_bs<SB, R, UB, LEARN>(P, M, t, P.order[t], g, open, L, s_f, s_fc)) return;
             if (tr) P.trace[5 + 2 * t] = global_ns();
             if (t + 1 < P.k) grid_arrive(&bar->count);
         }
@@ -816,7 +796,7 @@ __device__ __forceinline__ void bs_generations(const GomParams &P, const VGrid &
         acc_flush(P, s_f, s_cnt);
         if (LEARN) fc_flush(P, s_fc);
         if (!grid_barrier(&bar->count, &P.st->err, nblk, bnext, kBarrierNs)) return;
-        if (P.fi.on && !fi_generation<R>(P, V, &bar->count, nblk, bnext, e, P.order, s_f, s_cnt)) return;
+        if (P.fi.on && !fi_generation<(R <= 12 ? 12 : 16)>(P, V, &bar->count, nblk, bnext, e, P.order, s_f, s_cnt)) return;
         if (tr) P.trace[4 + 2 * P.k] = global_ns();
         ++g;
     }

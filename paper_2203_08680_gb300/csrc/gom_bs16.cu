@@ -2,5 +2,5 @@
 #include "gom_bs_kernels.cuh"
 #include "gom_kernels.cuh"
 
-const void *gom_run_bs16(int r, bool learn) { return learn ? run_bs_kernel<16, true>(r) : run_bs_kernel<16, false>(r); }
-const void *gom_mix_bs16(int r, bool learn) { return learn ? mix_bs_kernel<16, true>(r) : mix_bs_kernel<16, false>(r); }
+const void *gom_run_bs16(int r, int ub, bool learn) { return run_bs_kernel<16>(r, ub, learn); }
+const void *gom_mix_bs16(int r, int ub, bool learn) { return mix_bs_kernel<16>(r, ub, learn); }

@@ -24,12 +24,14 @@ struct gom_ctx {
     bool can_persist = false;     // cooperative launch available and the sizes fit
     bool persistent = false;      // current path: k_run (true) or the per-generation graph
     // the bit-sliced mixing path (gom_bs.cu), where the FOS and weights allow it
-    bool bs_ok = false;           // available for this context
+    bool bs_can = false;          // available for this context
+    bool bs_ok = false;           // and within the option's limits (8-bit weights): the caller may switch it on, and
+                                  //   the learned filter runs on it
     bool bs_on = false;           // selected (GOM_OPT_BITSLICED)
     int bs_set = -1;              // GOM_OPT_BITSLICED as the caller set it (-1: never set; batched launches
                                   //   then choose by the instance's share of warps)
     const void *run_bs_fn = nullptr, *mix_bs_fn = nullptr; // the instances for the learned filter's mode
-    int bs_r = 0;                 // their accumulator width R
+    int bs_r = 0, bs_ub = 0;      // their accumulator and weight widths
     size_t bs_smem = 0;           // dynamic shared memory of both (warp regions, group keys)
     int bs_threads = 0;           // their block size
     int bs_grid_run = 0, bs_grid_mix = 0;
@@ -65,9 +67,23 @@ struct gom_ctx {
 };
 
 
-// The bit-sliced path runs the context's generations (selected and
-// available; the learned filter works on either path).
-inline bool use_bs(const gom_ctx *ctx) { return ctx->bs_on; }
+// The bit-sliced path runs the context's generations: selected, and with the
+// learned filter on within its instances' limits.
+inline bool use_bs(const gom_ctx *ctx) { return ctx->bs_on && (ctx->bs_ok || !ctx->prm.learn); }
+
+// Weight and sum widths of the bit-sliced instances for |w| <= max_w and
+// element sums of |w| <= max_abs_w; false where there is none.
+inline bool bs_planes(int64_t max_w, int64_t max_abs_w, int *r, int *ub)
+{
+    static constexpr int kPlanes[4][2] = {{12, 8}, {16, 8}, {16, 12}, {20, 16}};
+    for (const auto &c : kPlanes)
+        if (max_abs_w < (int64_t(1) << c[0]) && max_w < (int64_t(1) << c[1])) {
+            *r = c[0];
+            *ub = c[1];
+            return true;
+        }
+    return false;
+}
 
 inline int cuda_fail(gom_ctx *ctx, cudaError_t e)
 {

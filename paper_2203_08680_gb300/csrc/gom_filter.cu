@@ -280,8 +280,8 @@ int gom_filter_set_mode(gom_ctx_t *ctx, int32_t mode)
     ctx->mix_fn = mix;
     ctx->run_fn = run;
     if (ctx->bs_ok) { // the bit-sliced instances with (or without) the filter's select phase and bookkeeping
-        ctx->run_bs_fn = gom_run_bs_kernel(ctx->prm.bs_S, ctx->bs_r, learn);
-        ctx->mix_bs_fn = gom_mix_bs_kernel(ctx->prm.bs_S, ctx->bs_r, learn);
+        ctx->run_bs_fn = gom_run_bs_kernel(ctx->prm.bs_S, ctx->bs_r, ctx->bs_ub, learn);
+        ctx->mix_bs_fn = gom_mix_bs_kernel(ctx->prm.bs_S, ctx->bs_r, ctx->bs_ub, learn);
     }
     ctx->prm.learn = mode;
     return rebuild_graphs(ctx);

@@ -107,9 +107,11 @@ struct GomBatchInst {
     int32_t variant;    // kernel variant (kVarNarrow, kVarWide, kVarHuge; kVarBits: the bit-sliced phase)
     int64_t target;     // target fitness of the current call
     int32_t gens;       // generations of the current call for this instance
-    int32_t bs_r;       // kVarBits: the width R of its plane accumulators (12 or 16)
+    int32_t bs_r;       // kVarBits: the width R of its plane accumulators
     int32_t gens_run;   // generations run by the last call
     int32_t err;        // the instance's device error word after the last call
+    int32_t bs_ub;      // kVarBits: bits of its weights
+    int32_t pad_;
 };
 
 // Learned trial filter (gom_filter_*): a 16 -> 64 -> 1 MLP with bf16 weights

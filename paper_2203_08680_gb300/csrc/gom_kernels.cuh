@@ -23,23 +23,24 @@ const void *gom_mix_kernel(int wpi, int variant, bool learn);
 // int G, int64_t target), with the same instances (null where none).
 const void *gom_run_kernel(int wpi, int variant, bool learn);
 // The bit-sliced path (gom_bs.cu): the persistent generation kernel
-// k_run_bs<class, R, learn>(GomParams, int G, int64_t target) and the
-// per-group mixing kernel k_mix_bs<class, R, learn>(GomParams, int t) for
-// elements of at most s <= 32 variables and bit-plane accumulators of R bits
-// (12 or 16; null beyond), with or without the learned filter's select phase
-// and bookkeeping, and the shared-memory words of one warp's region.
-const void *gom_run_bs_kernel(int s, int r, bool learn);
-const void *gom_mix_bs_kernel(int s, int r, bool learn);
+// k_run_bs<class, R, UB, learn>(GomParams, int G, int64_t target) and the
+// per-group mixing kernel k_mix_bs<class, R, UB, learn>(GomParams, int t) for
+// elements of at most s <= 32 variables, weights of UB bits and sums of R bits
+// (BsPlanes), with or without the learned filter's select phase and
+// bookkeeping (8-bit weights only, else null), and the shared-memory words of
+// one warp's region.
+const void *gom_run_bs_kernel(int s, int r, int ub, bool learn);
+const void *gom_mix_bs_kernel(int s, int r, int ub, bool learn);
 int gom_bs_warp_words(int s);
 // Packs the dependency lists into the bit-sliced path's edge lists (P.bdep).
 __global__ void k_bs_edges(GomParams P, int2 *bdep);
 // The instances of one element class (8, 16 or 32 variables at most).
-const void *gom_run_bs8(int r, bool learn);
-const void *gom_mix_bs8(int r, bool learn);
-const void *gom_run_bs16(int r, bool learn);
-const void *gom_mix_bs16(int r, bool learn);
-const void *gom_run_bs32(int r, bool learn);
-const void *gom_mix_bs32(int r, bool learn);
+const void *gom_run_bs8(int r, int ub, bool learn);
+const void *gom_mix_bs8(int r, int ub, bool learn);
+const void *gom_run_bs16(int r, int ub, bool learn);
+const void *gom_mix_bs16(int r, int ub, bool learn);
+const void *gom_run_bs32(int r, int ub, bool learn);
+const void *gom_mix_bs32(int r, int ub, bool learn);
 // Forced Improvement on the per-launch path: which = 0 k_fi_elite(GomParams)
 // (one block of 1024), 1 k_fi_start(GomParams), 2 k_fi_group<R>(GomParams,
 // int t) (256 threads), 3 k_fi_finish(GomParams).

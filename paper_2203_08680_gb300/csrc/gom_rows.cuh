@@ -203,22 +203,6 @@ __device__ __forceinline__ void add_bytes4(uint32_t (&acc)[kCutPlanes], const ui
     }
 }
 
-// 32 x 32 bit transpose of 32 registers inside the lane.
-template <int J = 16>
-__device__ __forceinline__ void transpose_planes(uint32_t (&x)[32])
-{
-    constexpr uint32_t m = J == 16 ? 0x0000FFFFu : J == 8 ? 0x00FF00FFu : J == 4 ? 0x0F0F0F0Fu : J == 2 ? 0x33333333u
-                                                                                                    : 0x55555555u;
-#pragma unroll
-    for (int r = 0; r < 32; ++r) {
-        if (r & J) continue;
-        const uint32_t a = x[r], b = x[r + J];
-        x[r] = (a & m) | ((b << J) & ~m);
-        x[r + J] = ((a >> J) & m) | (b & ~m);
-    }
-    if constexpr (J > 1) transpose_planes<J / 2>(x);
-}
-
 // Adds a warp's planes (lane = slot Wv + word) into s_f[32 word + b], times
 // 2^shift, and clears them: the slots' planes added in a tree, then the sums
 // of slot 0's lanes turned into numbers.  Warp-wide.
@@ -243,7 +227,7 @@ __device__ __forceinline__ void cut_flush(uint32_t (&acc)[kCutPlanes], int Wv, i
         uint32_t x[32];
 #pragma unroll
         for (int t = 0; t < 32; ++t) x[t] = t < kCutPlanes ? acc[t] : 0u;
-        transpose_planes(x);
+        transpose_lane<32>(x);
 #pragma unroll
         for (int b = 0; b < 32; ++b)
             if (x[b])

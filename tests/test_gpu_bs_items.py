@@ -48,3 +48,28 @@ def test_bit_sliced_items(oracle, s, p, rows):
         stats, _ = P.generation(1)
         _assert_same_stats(stats[0], run.generation())
         _assert_same_state(_gpu_state(P), run.get(), f"generation {gen}")
+
+
+@pytest.mark.parametrize("wmax,degree", [(255, 4), (256, 4), (4095, 4), (4096, 6), (65535, 4), (65535, 9)])
+@pytest.mark.parametrize("path", ["persistent", "graph", "batch"])
+def test_wide_weights(oracle, wmax, degree, path):
+    """Weights up to every plane width's bound, of either sign (65,535 on 90-edge elements: sums past the widest
+    planes, the per-lane path)."""
+    g = I.random_regular(600, degree, seed=wmax % 97, wmin=-wmax, wmax=wmax)
+    g.weight[:] = np.where(np.abs(g.weight) > wmax * 9 // 10, np.sign(g.weight) * wmax, g.weight)
+    P = gom.Population(g, 70, 5, persistent=path != "graph")
+    ep, ev = oracle.build_fos(g)
+    k, co = oracle.color(g, ep, ev)
+    run = oracle.Run(g, ep, ev, co, k, 70, 5)
+    if path == "batch":
+        ws = torch.empty(gom.gom_batch_workspace_bytes(1) + 256, dtype=torch.uint8, device="cuda")
+        batch = gom.gom_batch_create([P.ctx], (4, 2, 8, 300), ws[(-ws.data_ptr()) % 256:])
+    for gen in range(5):
+        if path == "batch":
+            gom.gom_batch_generation(batch, 1)
+            stats = gom.gom_batch_stats(batch, 0, 1)
+        else:
+            stats, _ = P.generation(1)
+        _assert_same_stats(stats[0], run.generation())
+        _assert_same_state(_gpu_state(P), run.get(), f"generation {gen}")
+    assert np.array_equal(P.fitness().cpu().numpy(), run.get()["f"])
