@@ -33,7 +33,7 @@ int words_for(int32_t p)
 struct Layout {
     size_t O, P, f, eqw, xe, st, bar, trace, stats, order, work;
     size_t fi_accw, fi_eq, fi_act0, fi_imp, fi_stale, fi_f0;
-    size_t row_ptr, col, wgt, hdr, fv, wout, wabs, seg, dep, bdep, cptr;
+    size_t row_ptr, col, wgt, hdr, fv, wout, wabs, seg, dep, bdep, cptr, ms_list, ms_ptr;
     size_t total;
 };
 
@@ -76,6 +76,8 @@ Layout make_layout(int64_t n, int32_t p, int64_t nadj, int64_t m, int64_t total_
     L.dep = take(sizeof(int32_t) * 2 * ndeps);
     L.bdep = take(sizeof(int32_t) * 2 * ndeps);
     L.cptr = take(sizeof(int32_t) * (std::max<int32_t>(k, 0) + 1));
+    L.ms_list = take(sizeof(int32_t) * m);
+    L.ms_ptr = take(sizeof(int32_t) * 5 * std::max<int32_t>(k, 1));
     L.total = off;
     return L;
 }
@@ -151,7 +153,7 @@ int build_graph(gom_ctx *ctx, bool timed, cudaGraph_t *out_graph, cudaGraphExec_
         }
         ts[t] = t;
         void *args2[] = {&prm, &ts[t]};
-        if (use_bs(ctx))
+        if (use_bs(ctx) && ctx->mix_bs_fn)
             e = add_kernel(g, &node, last, ctx->mix_bs_fn, ctx->bs_grid_mix, ctx->bs_threads, ctx->bs_smem, args2);
         else
             e = add_kernel(g, &node, last, ctx->mix_fn, ctx->grid_mix, ctx->mix_threads, ctx->mix_smem, args2);
@@ -216,9 +218,10 @@ int accumulate_timing(gom_ctx *ctx)
 int rebuild_graphs(gom_ctx *ctx)
 {
     // the learned filter's counting unit and list mode follow the mixing path in use
-    ctx->prm.flt.compact = use_bs(ctx) ? 1 : 0;
+    const bool bs = use_bs(ctx) && ctx->mix_bs_fn;
+    ctx->prm.flt.compact = bs ? 1 : 0;
     ctx->prm.flt.items_per_elem =
-        use_bs(ctx) || !ctx->prm.split ? 1 : (ctx->prm.Wv + ctx->wpi - 1) / std::max(ctx->wpi, 1);
+        bs || !ctx->prm.split ? 1 : (ctx->prm.Wv + ctx->wpi - 1) / std::max(ctx->wpi, 1);
     GOM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     const bool had_timed = ctx->texec != nullptr;
     if (ctx->exec) cudaGraphExecDestroy(ctx->exec);
@@ -576,6 +579,74 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
             }
         }
     }
+    // the bit-sliced path by element classes: models with elements above 32
+    // variables, or above 16 with at least half of the elements in a smaller
+    // class (each class then pays for its own tables only; up to 16 variables
+    // one class with more resident warps is the faster: 237 against 256 us a
+    // generation for the 200x200 torus' tree of bound 10, p = 300)
+    std::vector<int32_t> ms_list, ms_ptr;
+    int ms_ub = 0;
+    if (max_w < 256 && tabs.max_abs_w < (int64_t(1) << 16))
+        ms_ub = 8;
+    else if (max_w < 65536 && tabs.max_abs_w < (int64_t(1) << 20))
+        ms_ub = 16;
+    if (coop && ms_ub && tabs.max_s > 16 && (c->bs_can || tabs.max_s > 32)) {
+        const auto cls = [&](int64_t q) {
+            const int s = tabs.hdr[8 * q + 3] & 0xFF;
+            return s > 32 ? 0 : s > 16 ? 1 : s > 8 ? 2 : 3;
+        };
+        const int top = tabs.max_s > 32 ? 0 : 1;
+        int64_t below = 0, most_pairs = 0, small_edges = 0, large_edges = 0, most_units = 1;
+        ms_list.reserve(static_cast<size_t>(c->m));
+        for (int32_t col = 0; col < c->k; ++col) {
+            int64_t count[4] = {0, 0, 0, 0};
+            for (int h = 0; h < 4; ++h) {
+                ms_ptr.push_back(static_cast<int32_t>(ms_list.size()));
+                for (int64_t q = fos->cptr[col]; q < fos->cptr[col + 1]; ++q)
+                    if (cls(q) == h) {
+                        ms_list.push_back(static_cast<int32_t>(q));
+                        ++count[h];
+                        const int32_t *e = tabs.hdr.data() + 8 * q;
+                        int64_t &most = h > 0 ? small_edges : large_edges;
+                        most = std::max<int64_t>(most, (e[3] >> 8) + e[4]);
+                    }
+            }
+            ms_ptr.push_back(static_cast<int32_t>(ms_list.size()));
+            for (int h = top + 1; h < 4; ++h) below += count[h];
+            most_pairs = std::max(most_pairs, count[1] + count[2] + count[3]);
+            most_units = std::max(most_units, count[0] + (count[1] + count[2] + count[3]));
+        }
+        const int wpb = kBsThreads / 32;
+        const size_t smem = std::max(static_cast<size_t>(256 * c->W) +
+                                         sizeof(uint32_t) * gom_bs_multi_words(static_cast<int>(tabs.max_s), wv, wpb,
+                                                                               static_cast<int>(large_edges)),
+                                     keys_smem);
+        const void *fn = gom_run_multi_kernel(ms_ub);
+        int occ_s = 0;
+        if ((top == 0 || 2 * below >= c->m) && smem <= static_cast<size_t>(kSmemBudget)) {
+            GOM_CUDA(c, raise_smem_limit(fn, smem));
+            GOM_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_s, fn, kBsThreads, smem));
+        }
+        if (occ_s > 0) {
+            c->run_ms_fn = fn;
+            c->ms_smem = smem;
+            c->ms_ub = ms_ub;
+            c->ms_edges = small_edges;
+            c->prm.ms_edges = static_cast<int32_t>(large_edges);
+            const int64_t warps = static_cast<int64_t>(c->sms) * occ_s * wpb;
+            bs_split(wv, std::max<int64_t>(most_pairs, 1), small_edges, warps, wpb, &c->prm.bs_lsh, &c->prm.bs_nwi);
+            // a block for every large element and small element of a group up to one per SM, then four tiles a block
+            c->ms_grid = static_cast<int>(std::min<int64_t>(
+                static_cast<int64_t>(c->sms) * occ_s,
+                std::max<int64_t>(std::min<int64_t>(most_units, c->sms), (most_units * c->prm.bs_nwi + wpb - 1) / wpb)));
+            c->prm.bs_S = static_cast<int32_t>(std::min<int64_t>(tabs.max_s, 32));
+            c->prm.bs_words = gom_bs_warp_words(c->prm.bs_S);
+            if (!c->bs_can) {
+                c->bs_can = true;
+                c->bs_on = bs_pays(wv, max_group, tabs.max_s, c->prm.stage_all != 0, warps);
+            }
+        }
+    }
     // dynamic item claims: faster warps take more items (in stage-all mode
     // every warp has at most one item per group and the schedule is moot)
     c->prm.dyn = 1;
@@ -646,6 +717,8 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
     P.dep = reinterpret_cast<const int2 *>(base + L.dep);
     P.bdep = reinterpret_cast<const int2 *>(base + L.bdep);
     P.cptr = reinterpret_cast<const int32_t *>(base + L.cptr);
+    P.ms_list = reinterpret_cast<const int32_t *>(base + L.ms_list);
+    P.ms_ptr = reinterpret_cast<const int32_t *>(base + L.ms_ptr);
 
     // uploads (host vectors outlive the copies: the stream is synchronised below)
     std::vector<int32_t> cptr32(fos->cptr.begin(), fos->cptr.end());
@@ -661,6 +734,10 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
     GOM_CUDA(c, upload(base, L.seg, tabs.seg, s));
     GOM_CUDA(c, upload(base, L.dep, tabs.dep, s));
     GOM_CUDA(c, upload(base, L.cptr, cptr32, s));
+    if (c->run_ms_fn) {
+        GOM_CUDA(c, upload(base, L.ms_list, ms_list, s));
+        GOM_CUDA(c, upload(base, L.ms_ptr, ms_ptr, s));
+    }
 
     if (c->bs_can) {
         k_bs_edges<<<c->grid_io, 256, 0, s>>>(P, reinterpret_cast<int2 *>(base + L.bdep));
@@ -701,7 +778,10 @@ int gom_generation(gom_ctx_t *ctx, int32_t num_generations, int64_t target_fitne
             int gens = chunk;
             int64_t target = target_fitness;
             void *args[] = {&prm, &gens, &target};
-            if (use_bs(ctx))
+            if (use_bs(ctx) && ctx->run_ms_fn && !ctx->prm.learn)
+                GOM_CUDA(ctx, cudaLaunchCooperativeKernel(ctx->run_ms_fn, dim3(ctx->ms_grid), dim3(kBsThreads), args,
+                                                          ctx->ms_smem, ctx->stream));
+            else if (use_bs(ctx))
                 GOM_CUDA(ctx, cudaLaunchCooperativeKernel(ctx->run_bs_fn, dim3(ctx->bs_grid_run), dim3(ctx->bs_threads),
                                                           args, ctx->bs_smem, ctx->stream));
             else

@@ -87,15 +87,24 @@ double instance_cost(const gom_ctx *c, int item_cost, bool bits)
     return static_cast<double>(c->m) * item_cost + static_cast<double>(wv) * c->sum_se;
 }
 
+// The bit-sliced phase by element classes, where the instance has it (a large
+// element takes four warps of a block or more).  level: 0 every phase, 1
+// without this one, 2 per lane only -- a batch whose shared memory or
+// co-resident blocks do not reach for all takes the next level.
+bool batch_multi(const gom_ctx *c, const gom_batch_config_t &conf, int level)
+{
+    return level == 0 && c->run_ms_fn && conf.min_blocks == 2 && conf.warps_per_block >= 4;
+}
+
 // Whether an instance on `warps` warps runs the bit-sliced phase (only in the
 // kernel with the larger register budget, min_blocks 2): as the caller set it
 // for the context, else where its largest group gives every warp four pairs or
 // more (48 instances of 200 to 4,000 vertices, one to three a warp: 1.13 ms a
 // generation against 0.94 per lane; 48 of 1,000 to 65,536, five to thirty:
 // 2.1 against 7.2, and 3.1 with those below eight left per lane).
-bool batch_bits(const gom_ctx *c, const gom_batch_config_t &conf, int64_t warps)
+bool batch_bits(const gom_ctx *c, const gom_batch_config_t &conf, int level, int64_t warps)
 {
-    if (!c->bs_can || conf.min_blocks != 2) return false;
+    if (conf.min_blocks != 2 || level == 2 || !(c->bs_r || batch_multi(c, conf, level))) return false;
     if (c->bs_set >= 0) return c->bs_set == 1;
     return c->max_group * ((c->p + 31) / 32) >= 4 * warps;
 }
@@ -103,7 +112,8 @@ bool batch_bits(const gom_ctx *c, const gom_batch_config_t &conf, int64_t warps)
 // Blocks per instance: one each, then one at a time to the instance with the
 // largest estimated time per block, up to what its largest colour group can
 // use (one warp per item) or until the device is full.
-std::vector<int32_t> allocate_blocks(const std::vector<gom_ctx *> &ctx, int total_blocks, const gom_batch_config_t &conf)
+std::vector<int32_t> allocate_blocks(const std::vector<gom_ctx *> &ctx, int total_blocks, const gom_batch_config_t &conf,
+                                     int level, const double *weights)
 {
     const int warps_per_block = conf.warps_per_block, item_cost = conf.item_cost > 0 ? conf.item_cost : 300;
     const size_t B = ctx.size();
@@ -113,7 +123,8 @@ std::vector<int32_t> allocate_blocks(const std::vector<gom_ctx *> &ctx, int tota
     std::vector<int64_t> need(B);
     for (size_t b = 0; b < B; ++b) {
         // (as bit-sliced where it can be: what falls back to the per-lane phase is small)
-        cost[b] = instance_cost(ctx[b], item_cost, batch_bits(ctx[b], conf, 0));
+        cost[b] = instance_cost(ctx[b], item_cost, batch_bits(ctx[b], conf, level, 0));
+        if (weights) cost[b] *= weights[b];
         need[b] = (max_split_items(ctx[b]) + warps_per_block - 1) / warps_per_block;
         if (need[b] > 1) heap.push({cost[b], b});
     }
@@ -136,6 +147,14 @@ size_t gom_batch_workspace_bytes(int32_t num) { return num < 1 ? 0 : batch_layou
 
 int gom_batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config_t *cfg, void *d_workspace,
                      size_t ws_bytes, void *cuda_stream, gom_batch_t **out)
+{
+    return batch_create(ctxs, num, cfg, nullptr, d_workspace, ws_bytes, cuda_stream, out);
+}
+
+} // extern "C"
+
+int batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config_t *cfg, const double *weights,
+                 void *d_workspace, size_t ws_bytes, void *cuda_stream, gom_batch_t **out)
 {
     if (!ctxs || num < 1 || !out) return GOM_E_ARG;
     const gom_batch_config_t conf = cfg ? *cfg : gom_batch_config_t{4, 3, 0, 0};
@@ -165,35 +184,47 @@ int gom_batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config
     // int64), then one staging slice per warp (the largest slice of any
     // instance, whichever item split its allocation gets), or the colour-group
     // keys of the instance with most colours
-    int maxW = 1, maxk = 1;
-    int64_t max_warp_words = 8;
-    for (gom_ctx *c : cs) {
-        maxW = std::max(maxW, c->W);
-        maxk = std::max(maxk, c->k);
-        const int wv = (c->p + 31) / 32;
-        for (int64_t warps : {int64_t(1), INT64_MAX / 8}) {
-            int wpi = 1, split = 0;
-            item_split(c->W, c->p, c->max_group, warps, c->variant, &wpi, &split);
-            const SliceLayout SL =
-                slice_layout(c->max_s, c->max_edges, c->W, wpi, c->variant, split != 0, (wv + wpi - 1) / wpi);
-            max_warp_words = std::max<int64_t>(max_warp_words, SL.base_words);
-        }
-        if (c->bs_can && conf.min_blocks == 2) // a bit-sliced warp region
-            max_warp_words = std::max<int64_t>(max_warp_words, c->prm.bs_words);
-    }
-    const int32_t f_words = 2 * 32 * maxW;
-    const int64_t slices = std::max<int64_t>(int64_t(8) * maxk,
-                                             int64_t(4) * max_warp_words * conf.warps_per_block);
-    const int64_t smem = int64_t(4) * f_words + slices;
-    if (smem > kBatchSmemBudget) return GOM_E_LIMIT;
-
     const void *fn = gom_batch_kernel(conf.min_blocks);
     const int threads = 32 * conf.warps_per_block;
-    GOM_CUDA(nullptr, raise_smem_limit(fn, static_cast<size_t>(smem)));
-    int occ = 0;
-    GOM_CUDA(nullptr, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, static_cast<size_t>(smem)));
-    const int total = conf.max_blocks > 0 ? std::min(sms * occ, conf.max_blocks) : sms * occ;
-    if (total < num) return GOM_E_LIMIT;
+    int32_t f_words = 0;
+    int64_t smem = 0;
+    int total = 0, level = 0;
+    for (;; ++level) {
+        int maxW = 1, maxk = 1;
+        int64_t max_warp_words = 8;
+        for (gom_ctx *c : cs) {
+            maxW = std::max(maxW, c->W);
+            maxk = std::max(maxk, c->k);
+            const int wv = (c->p + 31) / 32;
+            for (int64_t warps : {int64_t(1), INT64_MAX / 8}) {
+                int wpi = 1, split = 0;
+                item_split(c->W, c->p, c->max_group, warps, c->variant, &wpi, &split);
+                const SliceLayout SL =
+                    slice_layout(c->max_s, c->max_edges, c->W, wpi, c->variant, split != 0, (wv + wpi - 1) / wpi);
+                max_warp_words = std::max<int64_t>(max_warp_words, SL.base_words);
+            }
+            if (!batch_bits(c, conf, level, 0)) continue;
+            // a block of the bit-sliced phase by element classes, or a bit-sliced warp region
+            if (batch_multi(c, conf, level))
+                max_warp_words = std::max<int64_t>(
+                    max_warp_words, (gom_bs_multi_words(static_cast<int>(c->max_s), wv, conf.warps_per_block, c->prm.ms_edges) +
+                                     conf.warps_per_block - 1) / conf.warps_per_block);
+            else
+                max_warp_words = std::max<int64_t>(max_warp_words, c->prm.bs_words);
+        }
+        f_words = 2 * 32 * maxW;
+        const int64_t slices = std::max<int64_t>(int64_t(8) * maxk, int64_t(4) * max_warp_words * conf.warps_per_block);
+        smem = int64_t(4) * f_words + slices;
+        total = 0;
+        if (smem <= kBatchSmemBudget) {
+            GOM_CUDA(nullptr, raise_smem_limit(fn, static_cast<size_t>(smem)));
+            int occ = 0;
+            GOM_CUDA(nullptr, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, static_cast<size_t>(smem)));
+            total = conf.max_blocks > 0 ? std::min(sms * occ, conf.max_blocks) : sms * occ;
+        }
+        if (total >= num) break;
+        if (level == 2) return GOM_E_LIMIT;
+    }
 
     std::unique_ptr<gom_batch> bt(new (std::nothrow) gom_batch());
     if (!bt) return GOM_E_ARG;
@@ -211,7 +242,7 @@ int gom_batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config
     B->d_inst = reinterpret_cast<GomBatchInst *>(base + L.inst);
     B->d_bars = reinterpret_cast<GomBarrier *>(base + L.bars);
 
-    const std::vector<int32_t> nb = allocate_blocks(cs, total, conf);
+    const std::vector<int32_t> nb = allocate_blocks(cs, total, conf, level, weights);
     B->params.resize(num);
     B->inst.resize(num);
     int32_t blk = 0;
@@ -249,7 +280,7 @@ int gom_batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config
         P.fi.on = 0; // nor Forced Improvement (refused above)
         P.bar = B->d_bars + b; // (P.trace: the context's phase trace, when switched on)
         // (one-warp tiles: the blocks' named barriers are left to the block-mode instances)
-        if (c->bs_can) bs_split(wv, c->max_group, c->max_edges, int64_t(nb[b]) * conf.warps_per_block, 1, &P.bs_lsh, &P.bs_nwi);
+        if (c->bs_can) bs_split(wv, c->max_group, c->run_ms_fn ? c->ms_edges : c->max_edges, int64_t(nb[b]) * conf.warps_per_block, 1, &P.bs_lsh, &P.bs_nwi);
         B->params[b] = P;
         GomBatchInst &I = B->inst[b];
         I = GomBatchInst{};
@@ -257,11 +288,12 @@ int gom_batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config
         I.nblk = nb[b];
         I.wpi = wpi;
         I.variant = cs[b]->variant;
-        const bool use_bs = batch_bits(c, conf, int64_t(nb[b]) * conf.warps_per_block);
+        const bool use_bs = batch_bits(c, conf, level, int64_t(nb[b]) * conf.warps_per_block);
         if (use_bs) {
-            I.variant = kVarBits;
+            const bool multi = batch_multi(c, conf, level);
+            I.variant = multi ? kVarMulti : kVarBits;
             I.bs_r = c->bs_r;
-            I.bs_ub = c->bs_ub;
+            I.bs_ub = multi ? c->ms_ub : c->bs_ub;
         }
         I.target = INT64_MAX;
         blk += nb[b];
@@ -276,6 +308,8 @@ int gom_batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config
     *out = bt.release();
     return GOM_OK;
 }
+
+extern "C" {
 
 namespace {
 

@@ -86,9 +86,9 @@ __device__ __forceinline__ void add_signed(uint32_t (&D)[NP], uint32_t pos, uint
 // An edge of the bit-sliced path's lists (GomParams::bdep): x = the far end's
 // word offset v W in O (an edge leaving the element) or its row 32 b (inside);
 // y = the weight's sign in bit 31, |w| from bit kEdgeWeight on and the near
-// end's row 32 a from bit kEdgeRow on.
-constexpr int kEdgeRow = 0;     // 32 a: bits 5 .. 9
-constexpr int kEdgeWeight = 10; // |w|: bits 10 .. 30
+// end's row 32 a in the bits of kEdgeRowMask.
+constexpr int kEdgeRowMask = 127 << 5; // a <= 127
+constexpr int kEdgeWeight = 12;        // |w|: bits 12 .. 27
 
 // D += the sum over four edges of |w| pos - |w| neg, as add_signed would: the
 // edges in two pairs on UB + 2 planes each, the pairs' sum on UB + 3, and one

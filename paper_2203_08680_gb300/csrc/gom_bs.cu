@@ -85,7 +85,7 @@ __global__ void k_bs_edges(GomParams P, int2 *bdep)
         const int f0 = h0.y, d0 = h0.z, s = h0.w & 0xFF, n_in = h0.w >> 8, n_out = h1.x;
         const auto pack = [](int a, int w) { // |w| < 2^16 where the path is available
             const uint32_t mag = (uint32_t)(w < 0 ? -w : w);
-            return (int)((uint32_t)(32 * a) << kEdgeRow | mag << kEdgeWeight | (w < 0 ? 0x80000000u : 0u));
+            return (int)((uint32_t)(32 * a) | mag << kEdgeWeight | (w < 0 ? 0x80000000u : 0u));
         };
         for (int a = 0; a < s; ++a)
             for (uint32_t x = P.seg[f0 + q + a]; x < P.seg[f0 + q + a + 1]; ++x) {

@@ -263,34 +263,32 @@ __device__ __noinline__ bool self_hit(uint32_t *fl, const uint32_t *tab, const u
 
 // An item between its two parts: the lane's element and what the first part
 // found in the generation-start population.
-template <int SB>
 struct BsItem {
     int q, j, s, f0, d0, n_out, n_in;
     bool ke, audited;   // the lane's pair exists; the element runs as an audit of the learned filter
     uint32_t rs, nz;    // run starts of the pair, non-empty run-start words of the element
-    uint32_t xp[SB <= 16 ? SB : 1]; // P's rows (the widest class reads them again)
+    uint32_t xp[16];    // P's rows (the widest class reads them again)
 };
 
 // First part of an item of a colour group: entries [k0, k1) (at most E) of the
-// group's elements -- positions k0 .. k1 - 1, or with the learned filter
-// skipping, the positions qlist[k0 .. k1) of the compacted list -- with every
-// word.  Donor tables and the trials' entries: all of it from P, which does
+// group's elements -- positions k0 .. k1 - 1, or the positions qlist[k0 .. k1)
+// of a list (the learned filter's, or an element class's) -- with every word.  Donor tables and the trials' entries: all of it from P, which does
 // not change during a generation, so a tile makes the first item of a group
 // between its arrival at the barrier that opens the group and its wait there.
 template <int SB, bool LEARN>
 __device__ __forceinline__ void bs_prepare(const GomParams &P, const BsMap &M, const int32_t *qlist, int k0, int k1,
-                                           uint32_t g, BsItem<SB> &I)
+                                           uint32_t g, BsItem &I)
 {
     const int lane = threadIdx.x & 31, slot = M.slot;
-    const int W = P.W, Wv = P.Wv, p = P.p, S = P.bs_S;
+    const int W = P.W, Wv = P.Wv, p = P.p, S = min(P.bs_S, SB);
     const int e = M.e, w = M.w, b2 = e * Wv; // b2: the element's first slot
     const bool ke = M.in && k0 + e < k1;     // this lane's pair exists
     int q = k0 + e;
     I.audited = false;
-    if (LEARN && qlist && ke) {
+    if (qlist && ke) {
         const int32_t en = qlist[k0 + e];
         q = en & 0x7FFFFFFF;
-        I.audited = en < 0;
+        I.audited = LEARN && en < 0;
     }
     I.q = q;
     I.ke = ke;
@@ -461,14 +459,44 @@ __device__ __forceinline__ void bs_prepare(const GomParams &P, const BsMap &M, c
     __syncwarp(); // (a warp reads its own slots' entries)
 }
 
+// Adds the toggled edges of an element's trials in word w (32 individuals)
+// into D: part `part` of `parts` of the first `ne` of its edges list(x), four at
+// a time.  myD, myO: the flip planes and the parent's rows of the word,
+// variable a at 32 a.
+template <int R, int UB, class List>
+__device__ __forceinline__ void bs_edges_add(const GomParams &P, const BsItem &I, List list, int ne, int part,
+                                             int parts, int w, const uint32_t *myD, const uint32_t *myO,
+                                             uint32_t (&D)[R + 1])
+{
+    for (int x = 4 * part; x < ne; x += 4 * parts) { // four edges' loads issued before their arithmetic
+        int2 ed[4];
+        uint32_t pos[4], neg[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) ed[u] = x + u < ne ? list(x + u) : make_int2(0, 0); // weight 0
+#pragma unroll
+        for (int u = 0; u < 4; ++u) { // the far end's word, and whether a trial flips it too
+            neg[u] = x + u < I.n_out ? P.O[ed[u].x + w] : myO[ed[u].x];
+            pos[u] = x + u < I.n_out ? 0u : myD[ed[u].x];
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int ra = ed[u].y & kEdgeRowMask;
+            const uint32_t tg = myD[ra] ^ pos[u], cut = myO[ra] ^ neg[u] ^ (uint32_t)(ed[u].y >> 31);
+            pos[u] = tg & ~cut;
+            neg[u] = tg & cut;
+        }
+        add_signed4<R + 1, UB>(D, pos, neg, ed);
+    }
+}
+
 // Second part of an item, in its group: the parent's rows, the flip planes,
 // the partial evaluation, acceptance and writes of all its trials (Alg. 2).
 template <int SB, int R, int UB, bool LEARN>
-__device__ __forceinline__ void bs_item(const GomParams &P, const BsMap &M, const BsItem<SB> &I, uint32_t g,
+__device__ __forceinline__ void bs_item(const GomParams &P, const BsMap &M, const BsItem &I, uint32_t g,
                                         BsLane<FitShared> &L, long long *s_f, unsigned long long *s_fc)
 {
     const int slot = M.slot;
-    const int W = P.W, p = P.p, S = P.bs_S;
+    const int W = P.W, p = P.p, S = min(P.bs_S, SB);
     const int w = M.w, b2 = M.e * P.Wv, s = I.s;
     const bool ke = I.ke;
     constexpr int EW = bs_entry_words(SB);
@@ -624,26 +652,7 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const BsMap &M, cons
         uint32_t D[R + 1];
 #pragma unroll
         for (int t = 0; t <= R; ++t) D[t] = 0;
-        const int ne = ke ? I.n_out + I.n_in : 0;
-        for (int x = 4 * M.sub; x < ne; x += 4 << M.lsh) { // four edges' loads issued before their arithmetic
-            int2 ed[4];
-            uint32_t pos[4], neg[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) ed[u] = x + u < ne ? __ldg(P.bdep + I.d0 + x + u) : make_int2(0, 0); // weight 0
-#pragma unroll
-            for (int u = 0; u < 4; ++u) { // the far end's word, and whether a trial flips it too
-                neg[u] = x + u < I.n_out ? P.O[ed[u].x + w] : myO[ed[u].x];
-                pos[u] = x + u < I.n_out ? 0u : myD[ed[u].x];
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int ra = (ed[u].y >> kEdgeRow) & (31 << 5);
-                const uint32_t tg = myD[ra] ^ pos[u], cut = myO[ra] ^ neg[u] ^ (uint32_t)(ed[u].y >> 31);
-                pos[u] = tg & ~cut;
-                neg[u] = tg & cut;
-            }
-            add_signed4<R + 1, UB>(D, pos, neg, ed);
-        }
+        bs_edges_add<R, UB>(P, I, [&](int x) { return __ldg(P.bdep + I.d0 + x); }, ke ? I.n_out + I.n_in : 0, M.sub, 1 << M.lsh, w, myD, myO, D);
         for (int off = 1; off < 1 << M.lsh; off <<= 1) { // the sums of the pair's lanes
             uint32_t carry = 0;
 #pragma unroll
@@ -717,7 +726,7 @@ __device__ __forceinline__ bool phase_mix_bs(const GomParams &P, const BsMap &M,
     const BsGroup G = bs_group<LEARN>(P, M, c);
     const bool dyn = P.dyn && M.nwi == 1;
     unsigned claim = 0;
-    BsItem<SB> I;
+    BsItem I;
     for (int it = M.tile, next = M.tile + M.ntiles, first = 1;; first = 0) { // (one call site of either part)
         const int k0 = G.ka + it * M.E;
         if (it < G.items) bs_prepare<SB, LEARN>(P, M, G.qlist, k0, min(k0 + M.E, G.kz), g, I);
@@ -743,17 +752,20 @@ __device__ __forceinline__ void bs_finish_generation(const GomParams &P, BsLane<
 // Up to G generations of one context on the bit-sliced phase, on the blocks
 // of the (virtual) grid V, the phases separated by grid barriers on `bar`:
 // [generation start + group order] | group 0 | ... | group k-1 | and again,
-// each tile preparing its first item of a group ahead of the group's barrier;
+// each tile preparing its first item of a group before its wait at the group's barrier;
 // every block computes a generation's end from the fitness array after the
 // barrier that closes its last group (block 0 of V records it).  s_keys: room
 // for the k group keys of the order phase (it may overlay the regions and s_f, which
-// are set up after it); regions: the block's first warp region; s_f, s_cnt: the block's
+// are set up after it); fit, w: the lane's fitness planes and their word; s_f, s_cnt: the block's
 // fitness accumulators and counters; s_fc: the learned filter's block
 // counters (LEARN only).
-template <int SB, int R, int UB, bool LEARN>
-__device__ __forceinline__ void bs_generations(const GomParams &P, const VGrid &V, GomBarrier *bar, int G,
-                                               int64_t target, unsigned long long *s_keys, uint32_t *regions,
-                                               long long *s_f, unsigned long long *s_cnt, unsigned long long *s_fc)
+// mix(t, c, g, open, L) mixes the group at position t, colour c, calling open()
+// -- the wait at the barrier that opens the group -- once in every thread, and
+// is false when that gave up.
+template <int R, bool LEARN, class Mix>
+__device__ __forceinline__ void bs_run(const GomParams &P, const VGrid &V, GomBarrier *bar, int G, int64_t target,
+                                       unsigned long long *s_keys, uint32_t *fit, int w, long long *s_f,
+                                       unsigned long long *s_cnt, unsigned long long *s_fc, Mix mix)
 {
     const unsigned nblk = (unsigned)V.nblk;
     const bool lead = V.blk == 0;
@@ -766,9 +778,8 @@ __device__ __forceinline__ void bs_generations(const GomParams &P, const VGrid &
         P.st->target = target;
     }
     const bool tr = P.trace != nullptr && lead && threadIdx.x == 0;
-    const BsMap M = bs_map<LEARN>(P, V, regions);
     BsLane<FitShared> L;
-    L.fit.v = bs_fit(P, regions);
+    L.fit.v = fit;
     for (int qg = 0; qg < G; ++qg) {
         if (qg > 0 && phase_gen_end(P, target, g - 1, e, lead)) return;
         if (tr) P.trace[0] = global_ns();
@@ -776,7 +787,7 @@ __device__ __forceinline__ void bs_generations(const GomParams &P, const VGrid &
         phase_order(P, V, s_keys, g);
         if (LEARN) fc_zero(s_fc);
         acc_zero(P, s_f, s_cnt);
-        bs_lane_zero(L, M.w); // (the order phase's keys overlay the planes)
+        bs_lane_zero(L, w); // (the order phase's keys overlay the planes)
         if (tr) P.trace[1] = P.trace[2] = global_ns();
         if (!grid_barrier(&bar->count, &P.st->err, nblk, bnext, kBarrierNs)) return;
         if (LEARN && P.learn && !phase_filter_select(P, V, g, &bar->count, nblk, bnext, P.learn == 2 && P.flt.compact))
@@ -788,7 +799,7 @@ __device__ __forceinline__ void bs_generations(const GomParams &P, const VGrid &
                 if (tr) P.trace[4 + 2 * t] = global_ns();
                 return true;
             };
-            if (!phase_mix_bs<SB, R, UB, LEARN>(P, M, t, P.order[t], g, open, L, s_f, s_fc)) return;
+            if (!mix(t, P.order[t], g, open, L)) return;
             if (tr) P.trace[5 + 2 * t] = global_ns();
             if (t + 1 < P.k) grid_arrive(&bar->count);
         }
@@ -801,6 +812,18 @@ __device__ __forceinline__ void bs_generations(const GomParams &P, const VGrid &
         ++g;
     }
     if (G > 0 && lead) phase_gen_end(P, target, g - 1, e, true);
+}
+
+template <int SB, int R, int UB, bool LEARN>
+__device__ __forceinline__ void bs_generations(const GomParams &P, const VGrid &V, GomBarrier *bar, int G,
+                                               int64_t target, unsigned long long *s_keys, uint32_t *regions,
+                                               long long *s_f, unsigned long long *s_cnt, unsigned long long *s_fc)
+{
+    const BsMap M = bs_map<LEARN>(P, V, regions);
+    bs_run<R, LEARN>(P, V, bar, G, target, s_keys, bs_fit(P, regions), M.w, s_f, s_cnt, s_fc,
+                     [&](int t, int c, uint32_t g, auto &open, BsLane<FitShared> &L) {
+                         return phase_mix_bs<SB, R, UB, LEARN>(P, M, t, c, g, open, L, s_f, s_fc);
+                     });
 }
 
 } // namespace

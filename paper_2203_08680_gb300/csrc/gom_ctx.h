@@ -31,10 +31,16 @@ struct gom_ctx {
     int bs_set = -1;              // GOM_OPT_BITSLICED as the caller set it (-1: never set; batched launches
                                   //   then choose by the instance's share of warps)
     const void *run_bs_fn = nullptr, *mix_bs_fn = nullptr; // the instances for the learned filter's mode
-    int bs_r = 0, bs_ub = 0;      // their accumulator and weight widths
+    int bs_r = 0, bs_ub = 0;      // their accumulator and weight widths (elements above 32 variables have none)
     size_t bs_smem = 0;           // dynamic shared memory of both (warp regions, group keys)
     int bs_threads = 0;           // their block size
     int bs_grid_run = 0, bs_grid_mix = 0;
+    // the bit-sliced path by element classes (gom_bs_multi.cu): linkage models of mixed sizes, elements above 32
+    // variables included, where run_ms_fn is set; persistent path only, without the learned filter
+    const void *run_ms_fn = nullptr;
+    size_t ms_smem = 0;
+    int ms_grid = 0, ms_ub = 0;
+    int64_t ms_edges = 0;        // most edges of an element of at most 32 variables
     // Forced Improvement (GOM_OPT_FORCED_IMPROVEMENT)
     bool fi_ok = false;           // available: |w| <= 255, element sums of |w| below 2^16
     int fi_r = 16;                // bit-plane width of its accumulators
@@ -172,12 +178,15 @@ inline void bs_split(int wv, int64_t max_group, int64_t max_edges, int64_t warps
 // 60,000 p = 512 5459 / 3372; 2D torus 300 p = 1,024 also 6 times faster.  The
 // per-lane path wins where it stages every group at once and a group is no
 // more than a few hundred words (2D torus 10 p = 16 50 / 58, 50 p = 64 58 / 62),
-// and for one-word populations of large elements that do not fill the warps
-// (linkage tree of bound 30, 100x100 torus, p = 32: 142 / 239; p = 100: 267 / 259).
+// and for models with elements of 17 to 64 variables where the population has
+// one word and does not fill the warps (linkage tree of bound 30, 100x100 torus,
+// p = 32: 142 / 239) or a group has a few hundred words (20x20 torus, p = 100,
+// bound 30 147 / 193, bound 64 208 / 304; p = 512 253 / 194 and 416 / 315).
 inline bool bs_pays(int wv, int64_t max_group, int64_t max_s, bool stage_all, int64_t warps)
 {
     if (stage_all && (wv == 1 || max_group * wv <= 1024)) return false;
-    return !(wv == 1 && max_s > 16 && max_group <= 4 * warps);
+    if (max_s <= 16 || max_s > 64) return true;
+    return !(wv == 1 && max_group <= 4 * warps) && max_group * wv > 256;
 }
 
 // Raises a kernel's dynamic shared memory limit to at least `bytes`, never
@@ -203,6 +212,11 @@ inline cudaError_t raise_smem_limit(const void *fn, size_t bytes)
 // host_stats[0..num) (may be null) and their number (*run_out).  Waits for
 // the stream.  GOM_E_TIMEOUT if the context's device error word is set.
 int ctx_read_stats(gom_ctx *ctx, int32_t num, gom_gen_stats_t *host_stats, int32_t *run_out);
+
+// gom_batch_create with the generations each instance makes for one of the
+// others' (weights, or null: the same number), for the block shares.
+int batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config_t *cfg, const double *weights,
+                 void *d_workspace, size_t ws_bytes, void *cuda_stream, gom_batch_t **out);
 
 // Rebuilds the per-generation graphs after a change of the parameters they
 // copy (the timed variant only if it exists).  Waits for the stream.

@@ -69,8 +69,8 @@ int build_elem_tables(const gom_graph_t *g, const gom_fos &fos, ElemTables *out)
 // masks and deltas), wide = <= 64 variables (64-bit masks and deltas), huge =
 // 65 to GOM_MAX_ELEMENT variables (128-bit masks, 64-bit deltas; at most two
 // population words per item, no learned filter).
-enum : int32_t { kVarNarrow = 0, kVarWide = 1, kVarHuge = 2, kVarBits = 3 }; // kVarBits: batched instances on
-                                                                          // the bit-sliced phase
+enum : int32_t { kVarNarrow = 0, kVarWide = 1, kVarHuge = 2, kVarBits = 3, kVarMulti = 4 }; // the last two:
+    // batched instances on the bit-sliced phase, the whole model in one class or by element classes
 inline int32_t kernel_variant(int64_t max_s, int64_t max_abs_w)
 {
     if (max_s <= 32 && max_abs_w < (int64_t(1) << 30)) return kVarNarrow;
@@ -104,13 +104,13 @@ struct GomBarrier { // grid barrier of the persistent kernel: monotonic arrival 
 struct GomBatchInst {
     int32_t blk0, nblk; // its blocks [blk0, blk0 + nblk) of the launch
     int32_t wpi;        // words per item of its mixing (1, 2, 4)
-    int32_t variant;    // kernel variant (kVarNarrow, kVarWide, kVarHuge; kVarBits: the bit-sliced phase)
+    int32_t variant;    // kernel variant (kVarNarrow, ...)
     int64_t target;     // target fitness of the current call
     int32_t gens;       // generations of the current call for this instance
     int32_t bs_r;       // kVarBits: the width R of its plane accumulators
     int32_t gens_run;   // generations run by the last call
     int32_t err;        // the instance's device error word after the last call
-    int32_t bs_ub;      // kVarBits: bits of its weights
+    int32_t bs_ub;      // kVarBits, kVarMulti: bits of its weights
     int32_t pad_;
 };
 
@@ -212,9 +212,10 @@ struct GomParams {
                         //   regions of warps 0, 1, ... following each other from off_xw
     int32_t learn;      // learned filter: 0 off, 1 history and training log, 2 also skip elements
     GomFI fi;
-    int32_t bs_S;       // bit-sliced path: variables of the largest element
+    int32_t bs_S;       // bit-sliced path: variables of the largest element (at most 32)
     int32_t bs_lsh;     //   2^bs_lsh lanes per pair, bs_nwi warps per tile (gom_bs.cuh)
     int32_t bs_nwi;
+    int32_t ms_edges;   //   most edges of an element above 32 variables
     int32_t bs_words;   //   shared-memory words of one warp's region
     GomFilter flt;
     uint64_t seed;
@@ -241,4 +242,7 @@ struct GomParams {
     const int2 *dep;         // outside edges {v, w}, then inside edges {a | b << 8, w}
     const int2 *bdep;        // the same edges for the bit-sliced path (gom_bitplane.cuh), where it is available
     const int32_t *cptr;     // [k+1] colour -> positions
+    const int32_t *ms_list;  // [m] positions by colour, inside a colour by element class (gom_bs_multi.cuh)
+    const int32_t *ms_ptr;   // [5k] colour c's classes in ms_list: 33 to 128 variables, 17 to 32, 9 to 16, at most 8,
+                             //   and the end
 };

@@ -32,6 +32,13 @@ const void *gom_run_kernel(int wpi, int variant, bool learn);
 const void *gom_run_bs_kernel(int s, int r, int ub, bool learn);
 const void *gom_mix_bs_kernel(int s, int r, int ub, bool learn);
 int gom_bs_warp_words(int s);
+// The bit-sliced path by element classes (gom_bs_multi.cu): its persistent
+// kernel for elements of at most max_s <= 128 variables and weights of ub = 8
+// (sums below 2^16) or 16 bits (2^20), and a block's dynamic shared-memory
+// words after the fitness accumulators (edges: the most of an element above 32
+// variables).
+const void *gom_run_multi_kernel(int ub);
+int gom_bs_multi_words(int max_s, int wv, int warps, int edges);
 // Packs the dependency lists into the bit-sliced path's edge lists (P.bdep).
 __global__ void k_bs_edges(GomParams P, int2 *bdep);
 // The instances of one element class (8, 16 or 32 variables at most).

@@ -73,3 +73,35 @@ def test_wide_weights(oracle, wmax, degree, path):
         _assert_same_stats(stats[0], run.generation())
         _assert_same_state(_gpu_state(P), run.get(), f"generation {gen}")
     assert np.array_equal(P.fitness().cpu().numpy(), run.get()["f"])
+
+
+@pytest.mark.parametrize("bound,p", [(10, 300), (16, 33), (17, 64), (40, 65), (64, 512), (100, 70), (128, 1024), (128, 32)])
+@pytest.mark.parametrize("path", ["persistent", "batch", "wide"])
+def test_linkage_trees_by_class(oracle, bound, p, path):
+    """Elements of 1 to `bound` variables in one model: the small classes' items and the blocks' large elements
+    (33 to 128 variables) on the default path, batched, and with 16-bit weights; a few distinct rows at first, so
+    that long runs and self-hits occur."""
+    wmax = 30000 if path == "wide" else 100
+    g = I.torus2d(22, seed=bound + p, wmin=-wmax // 3, wmax=wmax)
+    ep, ev = oracle.build_bflt(g, bound)
+    P = gom.Population(g, p, 9, fos=gom.gom_build_fos(g, gom.GOM_FOS_BFLT, bound))
+    k, co = oracle.color(g, ep, ev)
+    run = oracle.Run(g, ep, ev, co, k, p, 9)
+    rng = np.random.default_rng(bound * 7 + p)
+    base = rng.integers(0, 2, (5, g.n), dtype=np.uint8)
+    pop = base[rng.integers(0, 5, p)]
+    f = np.array([oracle.cut_value(g, x) for x in pop], dtype=np.int64)
+    best = int(f.argmax())
+    P.set_population(torch.from_numpy(pop).cuda(), torch.from_numpy(pop[best]).cuda(), int(f[best]), 0)
+    run.load(pop, f, pop[best], int(f[best]), 0)
+    if path == "batch":
+        ws = torch.empty(gom.gom_batch_workspace_bytes(1) + 256, dtype=torch.uint8, device="cuda")
+        batch = gom.gom_batch_create([P.ctx], (4, 2, 2, 300), ws[(-ws.data_ptr()) % 256:])
+    for gen in range(4):
+        if path == "batch":
+            gom.gom_batch_generation(batch, 1)
+            stats = gom.gom_batch_stats(batch, 0, 1)
+        else:
+            stats, _ = P.generation(1)
+        _assert_same_stats(stats[0], run.generation())
+        _assert_same_state(_gpu_state(P), run.get(), f"generation {gen}")
