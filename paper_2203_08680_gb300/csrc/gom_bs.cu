@@ -1,6 +1,5 @@
 // gom_bs.cu -- the bit-sliced mixing path's kernels by element class (their
-// instances are in gom_bs8.cu, gom_bs16.cu and gom_bs32.cu, so that they
-// compile in parallel) and the Forced Improvement kernels of the
+// instances are in gom_bs5.cu to gom_bs32.cu, so that they compile in parallel) and the Forced Improvement kernels of the
 // per-generation graph.
 #include <climits>
 #include <cuda_runtime.h>
@@ -111,14 +110,24 @@ const void *gom_fi_kernel(int which, int r)
 
 const void *gom_run_bs_kernel(int s, int r, int ub, bool learn)
 {
-    const int c = bs_class(s);
-    return c == 8 ? gom_run_bs8(r, ub, learn) : c == 16 ? gom_run_bs16(r, ub, learn) : gom_run_bs32(r, ub, learn);
+    switch (bs_class(s)) {
+    case 5: return gom_run_bs5(r, ub, learn);
+    case 7: return gom_run_bs7(r, ub, learn);
+    case 8: return gom_run_bs8(r, ub, learn);
+    case 16: return gom_run_bs16(r, ub, learn);
+    default: return gom_run_bs32(r, ub, learn);
+    }
 }
 
 const void *gom_mix_bs_kernel(int s, int r, int ub, bool learn)
 {
-    const int c = bs_class(s);
-    return c == 8 ? gom_mix_bs8(r, ub, learn) : c == 16 ? gom_mix_bs16(r, ub, learn) : gom_mix_bs32(r, ub, learn);
+    switch (bs_class(s)) {
+    case 5: return gom_mix_bs5(r, ub, learn);
+    case 7: return gom_mix_bs7(r, ub, learn);
+    case 8: return gom_mix_bs8(r, ub, learn);
+    case 16: return gom_mix_bs16(r, ub, learn);
+    default: return gom_mix_bs32(r, ub, learn);
+    }
 }
 
 int gom_bs_warp_words(int s) { return bs_warp_words(s); }

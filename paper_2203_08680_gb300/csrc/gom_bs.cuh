@@ -100,13 +100,21 @@ __device__ __forceinline__ int next_run_start(const uint32_t *rs, uint32_t nz, i
     return 32 * w2 + __ffs(rs[w2]) - 1;
 }
 
-// Shared-memory words of one pair's table entries, by the class SB of the
-// largest element (8, 16 or 32 variables): 32 entries of 2 bytes (P_d in the
-// low byte, N_d in the high one), 4 bytes (halves) or 8 bytes (P_d, N_d).
-__host__ __device__ constexpr int bs_entry_words(int SB) { return 2 * SB; }
+// The kernels' element classes: instances for elements of at most SB = 5, 7, 8,
+// 16 or 32 variables (5 and 7: the neighbourhoods of degree 4 and 6; with the
+// rows known at compile time a generation of torus1000, p = 256, takes 9 %
+// less than in the class of 8).
+__host__ __device__ constexpr int bs_class(int S) { return S <= 5 ? 5 : S <= 7 ? 7 : S <= 8 ? 8 : S <= 16 ? 16 : 32; }
 
-// The class of the largest element S.
-__host__ __device__ constexpr int bs_class(int S) { return S <= 8 ? 8 : S <= 16 ? 16 : 32; }
+// Rows of a class's shared arrays: the class's in the small ones, else those of
+// the model's largest element.
+__host__ __device__ constexpr int bs_rows(int S) { return S <= 8 ? bs_class(S) : S; }
+
+// Variables of a pattern in the class's tables: entries of 2 bytes (P_d in the
+// low byte, N_d in the high one), 4 bytes (halves) or 8 bytes (P_d, N_d) for
+// 8, 16 or 32; a pair's 32 entries take twice as many words.
+__host__ __device__ constexpr int bs_table(int S) { return S <= 8 ? 8 : S <= 16 ? 16 : 32; }
+__host__ __device__ constexpr int bs_entry_words(int S) { return 2 * bs_table(S); }
 
 // Shared-memory words of one warp's region (a tile of several warps uses its
 // first warp's): the donor tables [32 pairs], the trials' entries [32 pairs]
@@ -118,12 +126,12 @@ __host__ __device__ constexpr int bs_class(int S) { return S <= 8 ? 8 : S <= 16 
 // any a.
 __host__ __device__ __forceinline__ int bs_warp_words(int S)
 {
-    return 64 * bs_entry_words(bs_class(S)) + 32 * S + 96 + 32 * kFitPlanes;
+    return 64 * bs_entry_words(S) + 32 * bs_rows(S) + 96 + 32 * kFitPlanes;
 }
 
 // Blocks per SM the kernels' registers are cut for, by element class: what the
 // regions leave of an SM's shared memory (34, 54 and 90 KB a block).
-constexpr int bs_blocks(int SB) { return SB == 8 ? 6 : SB == 16 ? 4 : 2; }
+constexpr int bs_blocks(int SB) { return SB <= 8 ? 6 : SB <= 16 ? 4 : 2; }
 
 // This lane's fitness planes; `regions` is the block's first warp region.
 __device__ __forceinline__ uint32_t *bs_fit(const GomParams &P, uint32_t *regions)
@@ -243,14 +251,14 @@ __device__ __noinline__ bool self_hit(uint32_t *fl, const uint32_t *tab, const u
     const int st = (int)min(d, d - (uint32_t)p);
     if (next_run_start(rs, nz, st + 1 == p ? 0 : st + 1) != i) return false;
     const auto entry = [&](int x, uint32_t *next) -> uint32_t {
-        if constexpr (SB == 8) {
+        if constexpr (bs_table(SB) == 8) {
             const uint32_t en = reinterpret_cast<const uint16_t *>(tab)[32 * b2 + x];
             *next = en >> 8;
             return en & 0xFFu;
         } else {
             const int k3 = b2 + (x >> 5), at = 32 * k3 + ((x + k3) & 31);
-            *next = SB == 16 ? tab[at] >> 16 : tab[1024 + at];
-            return SB == 16 ? tab[at] & 0xFFFFu : tab[at];
+            *next = bs_table(SB) == 16 ? tab[at] >> 16 : tab[1024 + at];
+            return bs_table(SB) == 16 ? tab[at] & 0xFFFFu : tab[at];
         }
     };
     uint32_t unused, nn;
@@ -280,7 +288,7 @@ __device__ __forceinline__ void bs_prepare(const GomParams &P, const BsMap &M, c
                                            uint32_t g, BsItem &I)
 {
     const int lane = threadIdx.x & 31, slot = M.slot;
-    const int W = P.W, Wv = P.Wv, p = P.p, S = min(P.bs_S, SB);
+    const int W = P.W, Wv = P.Wv, p = P.p, S = SB < 8 ? SB : min(P.bs_S, SB);
     const int e = M.e, w = M.w, b2 = e * Wv; // b2: the element's first slot
     const bool ke = M.in && k0 + e < k1;     // this lane's pair exists
     int q = k0 + e;
@@ -292,7 +300,7 @@ __device__ __forceinline__ void bs_prepare(const GomParams &P, const BsMap &M, c
     }
     I.q = q;
     I.ke = ke;
-    constexpr int EW = bs_entry_words(SB);
+    constexpr int EW = bs_entry_words(SB), TB = bs_table(SB);
     uint32_t *tab = M.sm, *res = M.sm + 32 * EW;
     uint32_t *sRS = M.sm + 64 * EW + 32 * S, *sLst = sRS + 32, *sFst = sLst + 32;
     const int lim = p - 32 * w; // >= 1
@@ -328,11 +336,12 @@ __device__ __forceinline__ void bs_prepare(const GomParams &P, const BsMap &M, c
 #pragma unroll
     for (int a8 = 0; a8 < SB; a8 += 8) {
         if (a8 < S) {
-            int at[8];
+            constexpr int C = SB < 8 ? SB : 8;
+            int at[C];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) at[c] = ke && a8 + c < s ? __ldg(P.fv + f0 + a8 + c) * W + w : -1;
+            for (int c = 0; c < C; ++c) at[c] = ke && a8 + c < s ? __ldg(P.fv + f0 + a8 + c) * W + w : -1;
 #pragma unroll
-            for (int c = 0; c < 8; ++c) xp[a8 + c] = at[c] >= 0 ? P.P[at[c]] : 0u;
+            for (int c = 0; c < C; ++c) xp[a8 + c] = at[c] >= 0 ? P.P[at[c]] : 0u;
         }
     }
     if constexpr (SB <= 16) {
@@ -376,12 +385,12 @@ __device__ __forceinline__ void bs_prepare(const GomParams &P, const BsMap &M, c
         I.nz = nz;
     }
     {
-        uint32_t x[SB];
+        uint32_t x[TB];
 #pragma unroll
-        for (int a = 0; a < SB; ++a) x[a] = xp[a];
-        transpose_lane<SB>(x); // block column c of x[r]: the pattern of individual 32 w + SB c + r
-        if (SB < 32) nx <<= 32 - SB;
-        if constexpr (SB == 8) {
+        for (int a = 0; a < TB; ++a) x[a] = a < SB ? xp[a < SB ? a : 0] : 0u;
+        transpose_lane<TB>(x); // block column c of x[r]: the pattern of individual 32 w + TB c + r
+        if (TB < 32) nx <<= 32 - TB;
+        if constexpr (TB == 8) {
 #pragma unroll
             for (int c = 3; c >= 0; --c) {
                 uint32_t ent[4]; // two entries each
@@ -396,7 +405,7 @@ __device__ __forceinline__ void bs_prepare(const GomParams &P, const BsMap &M, c
                 nx >>= 8;
                 *reinterpret_cast<uint4 *>(tab + 16 * slot + 4 * c) = make_uint4(ent[0], ent[1], ent[2], ent[3]);
             }
-        } else if constexpr (SB == 16) {
+        } else if constexpr (TB == 16) {
 #pragma unroll
             for (int c = 1; c >= 0; --c) {
 #pragma unroll
@@ -438,21 +447,21 @@ __device__ __forceinline__ void bs_prepare(const GomParams &P, const BsMap &M, c
             for (int cc = 0; cc < 4; ++cc) {
                 const uint32_t d = (uint32_t)(i0 + cc + 1) + __umulhi(pick(r4, cc), (uint32_t)(p - 1));
                 const uint32_t st = min(d, d - (uint32_t)p); // d < p: d - p wraps above d
-                if constexpr (SB == 8) {
+                if constexpr (TB == 8) {
                     en[cc] = reinterpret_cast<const uint16_t *>(tab)[32 * b2 + st];
                 } else {
                     const uint32_t k3 = (uint32_t)b2 + (st >> 5), at = 32 * k3 + ((st + k3) & 31);
                     en[cc] = tab[at];
-                    if constexpr (SB == 32) en2[cc] = tab[1024 + at];
+                    if constexpr (TB == 32) en2[cc] = tab[1024 + at];
                 }
             }
-            if constexpr (SB == 8) {
+            if constexpr (TB == 8) {
                 *reinterpret_cast<uint2 *>(res + 16 * k2 + (((c >> 1) ^ ((k2 >> 1) & 3)) << 2) + ((c & 1) << 1)) =
                     make_uint2(__byte_perm(en[0], en[1], 0x5410), __byte_perm(en[2], en[3], 0x5410));
             } else {
                 uint32_t *at = res + 32 * k2 + ((c ^ (k2 & 7)) << 2);
                 *reinterpret_cast<uint4 *>(at) = make_uint4(en[0], en[1], en[2], en[3]);
-                if constexpr (SB == 32) *reinterpret_cast<uint4 *>(at + 1024) = make_uint4(en2[0], en2[1], en2[2], en2[3]);
+                if constexpr (TB == 32) *reinterpret_cast<uint4 *>(at + 1024) = make_uint4(en2[0], en2[1], en2[2], en2[3]);
             }
         }
     }
@@ -496,10 +505,10 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const BsMap &M, cons
                                         BsLane<FitShared> &L, long long *s_f, unsigned long long *s_fc)
 {
     const int slot = M.slot;
-    const int W = P.W, p = P.p, S = min(P.bs_S, SB);
+    const int W = P.W, p = P.p, S = SB < 8 ? SB : min(P.bs_S, SB);
     const int w = M.w, b2 = M.e * P.Wv, s = I.s;
     const bool ke = I.ke;
-    constexpr int EW = bs_entry_words(SB);
+    constexpr int EW = bs_entry_words(SB), TB = bs_table(SB);
     const uint32_t *tab = M.sm;
     uint32_t *res = M.sm + 32 * EW;
     uint32_t *sF = res; // flip planes, once every lane has read its entries back
@@ -511,30 +520,31 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const BsMap &M, cons
 #pragma unroll
     for (int a8 = 0; a8 < SB; a8 += 8) {
         if (a8 < S) {
-            int at[8];
-            uint32_t xo[8];
+            constexpr int C = SB < 8 ? SB : 8;
+            int at[C];
+            uint32_t xo[C];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) at[c] = ke && a8 + c < s ? __ldg(P.fv + I.f0 + a8 + c) * W + w : -1;
+            for (int c = 0; c < C; ++c) at[c] = ke && a8 + c < s ? __ldg(P.fv + I.f0 + a8 + c) * W + w : -1;
 #pragma unroll
-            for (int c = 0; c < 8; ++c) xo[c] = at[c] >= 0 ? P.O[at[c]] : 0u;
+            for (int c = 0; c < C; ++c) xo[c] = at[c] >= 0 ? P.O[at[c]] : 0u;
             if constexpr (SB > 16) {
                 if (a8 == 0) chg = 0;
 #pragma unroll
-                for (int c = 0; c < 8; ++c) chg |= at[c] >= 0 ? xo[c] ^ P.P[at[c]] : 0u;
+                for (int c = 0; c < C; ++c) chg |= at[c] >= 0 ? xo[c] ^ P.P[at[c]] : 0u;
             }
 #pragma unroll
-            for (int c = 0; c < 8; ++c)
+            for (int c = 0; c < C; ++c)
                 if (a8 + c < S) sX[32 * (a8 + c) + slot] = xo[c];
         }
     }
 
     // the entries back as planes: t1[a] the starts' bits, then t2[a] the
     // fall-through patterns' bits; f1: the individuals whose start differs
-    uint32_t F[SB];
+    uint32_t F[TB];
     uint32_t f1 = 0, same = kFull; // same: the fall-through pattern is the individual's own in P
     {
-        uint32_t t2[SB];
-        if constexpr (SB == 8) {
+        uint32_t t2[TB];
+        if constexpr (TB == 8) {
             const int sw = (slot >> 1) & 3;
 #pragma unroll
             for (int h = 0; h < 2; ++h) { // chunk i holds individuals 8 i .. 8 i + 7; half h of each
@@ -556,9 +566,9 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const BsMap &M, cons
                     t2[r + 1] = __byte_perm(h0, h1, 0x7632);
                 }
             }
-            transpose_lane<SB>(F);
-            transpose_lane<SB>(t2);
-        } else if constexpr (SB == 16) {
+            transpose_lane<TB>(F);
+            transpose_lane<TB>(t2);
+        } else if constexpr (TB == 16) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) { // individuals 4 i .. + 3 and 16 + 4 i .. + 3
                 const uint4 u = *reinterpret_cast<const uint4 *>(res + 32 * slot + ((i ^ (slot & 7)) << 2));
@@ -572,8 +582,8 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const BsMap &M, cons
                 t2[4 * i + 2] = __byte_perm(u.z, v.z, 0x7632);
                 t2[4 * i + 3] = __byte_perm(u.w, v.w, 0x7632);
             }
-            transpose_lane<SB>(F);
-            transpose_lane<SB>(t2);
+            transpose_lane<TB>(F);
+            transpose_lane<TB>(t2);
         } else {
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
@@ -583,7 +593,7 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const BsMap &M, cons
                 F[4 * i + 2] = u.z;
                 F[4 * i + 3] = u.w;
             }
-            transpose_lane<SB>(F);
+            transpose_lane<TB>(F);
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const uint4 u = *reinterpret_cast<const uint4 *>(res + 1024 + 32 * slot + ((i ^ (slot & 7)) << 2));
@@ -592,7 +602,7 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const BsMap &M, cons
                 t2[4 * i + 2] = u.z;
                 t2[4 * i + 3] = u.w;
             }
-            transpose_lane<SB>(t2);
+            transpose_lane<TB>(t2);
         }
 #pragma unroll
         for (int a = 0; a < SB; ++a)
