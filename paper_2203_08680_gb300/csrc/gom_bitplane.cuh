@@ -94,7 +94,10 @@ constexpr int kEdgeWeight = 12;        // |w|: bits 12 .. 27
 // edges in two pairs on UB + 2 planes each, the pairs' sum on UB + 3, and one
 // chain over all NP planes; the four carries of one that complements need
 // (neg) go into the four chains.  148 logic instructions for UB = 8, NP = 13,
-// against 4 x 42 for four chains over all planes.
+// against 4 x 42 for four chains over all planes.  The logic pipe is the
+// busier one: for 8-bit weights one edge of a pair selects by a multiplication
+// (torus1000 20.4 -> 19.9 ms a pass, random 12-regular 13.2 -> 12.8; with more
+// weight bits the extra instructions cost more, torus317 1.74 -> 1.83).
 template <int NP, int UB>
 __device__ __forceinline__ void add_signed4(uint32_t (&D)[NP], const uint32_t (&pos)[4], const uint32_t (&neg)[4],
                                             const int2 (&ed)[4])
@@ -107,9 +110,16 @@ __device__ __forceinline__ void add_signed4(uint32_t (&D)[NP], const uint32_t (&
         uint32_t carry = n0;
 #pragma unroll
         for (int t = 0; t < UB + 2; ++t) {
-            const bool w0 = (ed[2 * h].y & (1 << (kEdgeWeight + (t < UB ? t : 0)))) != 0;
-            const bool w1 = (ed[2 * h + 1].y & (1 << (kEdgeWeight + (t < UB ? t : 0)))) != 0;
-            const uint32_t i0 = t < UB && w0 ? pos[2 * h] : n0, i1 = t < UB && w1 ? pos[2 * h + 1] : n1;
+            uint32_t i0 = n0, i1 = n1;
+            if (t < UB) {
+                if (UB > 8) {
+                    i0 = (ed[2 * h].y & (1 << (kEdgeWeight + t))) != 0 ? pos[2 * h] : n0;
+                } else { // n0 + m (n0 - pos), m = -1 or 0: the select on the multiplier's pipe
+                    const int m = (int)((uint32_t)ed[2 * h].y << (31 - kEdgeWeight - t)) >> 31;
+                    i0 = (uint32_t)m * (n0 - pos[2 * h]) + n0;
+                }
+                i1 = (ed[2 * h + 1].y & (1 << (kEdgeWeight + t))) != 0 ? pos[2 * h + 1] : n1;
+            }
             A[h][t] = i0 ^ i1 ^ carry;
             carry = (i0 & i1) | (i0 & carry) | (i1 & carry);
         }
