@@ -28,7 +28,8 @@ template <int SB, int R, int UB>
 __device__ __noinline__ void batch_variant_bs(const GomParams &P, const VGrid V, GomBarrier *bar, int G,
                                               int64_t target, const RunShared &S)
 {
-    bs_generations<SB, R, UB, false>(P, V, bar, G, target, reinterpret_cast<unsigned long long *>(S.dyn),
+    const GomParams Q = P; // a private copy: in shared memory every store to it might change a parameter
+    bs_generations<SB, R, UB, false, false>(Q, V, bar, G, target, reinterpret_cast<unsigned long long *>(S.dyn),
                              S.dyn, S.f, S.cnt, nullptr);
 }
 
@@ -36,7 +37,8 @@ template <int R, int UB>
 __device__ __noinline__ void batch_variant_multi(const GomParams &P, const VGrid V, GomBarrier *bar, int G,
                                                  int64_t target, const RunShared &S)
 {
-    bs_multi_generations<R, UB>(P, V, bar, G, target, reinterpret_cast<unsigned long long *>(S.dyn), S.dyn, S.f,
+    const GomParams Q = P;
+    bs_multi_generations<R, UB, false>(Q, V, bar, G, target, reinterpret_cast<unsigned long long *>(S.dyn), S.dyn, S.f,
                                      S.cnt);
 }
 

@@ -769,10 +769,10 @@ __device__ __forceinline__ void bs_finish_generation(const GomParams &P, BsLane<
 // are set up after it); fit, w: the lane's fitness planes and their word; s_f, s_cnt: the block's
 // fitness accumulators and counters; s_fc: the learned filter's block
 // counters (LEARN only).
-// mix(t, c, g, open, L) mixes the group at position t, colour c, calling open()
+// FI: the Forced Improvement option exists here.  mix(t, c, g, open, L) mixes the group at position t, colour c, calling open()
 // -- the wait at the barrier that opens the group -- once in every thread, and
 // is false when that gave up.
-template <int R, bool LEARN, class Mix>
+template <int R, bool LEARN, bool FI, class Mix>
 __device__ __forceinline__ void bs_run(const GomParams &P, const VGrid &V, GomBarrier *bar, int G, int64_t target,
                                        unsigned long long *s_keys, uint32_t *fit, int w, long long *s_f,
                                        unsigned long long *s_cnt, unsigned long long *s_fc, Mix mix)
@@ -811,26 +811,26 @@ __device__ __forceinline__ void bs_run(const GomParams &P, const VGrid &V, GomBa
             };
             if (!mix(t, P.order[t], g, open, L)) return;
             if (tr) P.trace[5 + 2 * t] = global_ns();
-            if (t + 1 < P.k) grid_arrive(&bar->count);
+            if (t + 1 < P.k) grid_arrive(&bar->count, nblk);
         }
         bs_finish_generation(P, L, s_f, s_cnt);
         acc_flush(P, s_f, s_cnt);
         if (LEARN) fc_flush(P, s_fc);
         if (!grid_barrier(&bar->count, &P.st->err, nblk, bnext, kBarrierNs)) return;
-        if (P.fi.on && !fi_generation<(R <= 12 ? 12 : 16)>(P, V, &bar->count, nblk, bnext, e, P.order, s_f, s_cnt)) return;
+        if (FI && P.fi.on && !fi_generation<(R <= 12 ? 12 : 16)>(P, V, &bar->count, nblk, bnext, e, P.order, s_f, s_cnt)) return;
         if (tr) P.trace[4 + 2 * P.k] = global_ns();
         ++g;
     }
     if (G > 0 && lead) phase_gen_end(P, target, g - 1, e, true);
 }
 
-template <int SB, int R, int UB, bool LEARN>
+template <int SB, int R, int UB, bool LEARN, bool FI = true>
 __device__ __forceinline__ void bs_generations(const GomParams &P, const VGrid &V, GomBarrier *bar, int G,
                                                int64_t target, unsigned long long *s_keys, uint32_t *regions,
                                                long long *s_f, unsigned long long *s_cnt, unsigned long long *s_fc)
 {
     const BsMap M = bs_map<LEARN>(P, V, regions);
-    bs_run<R, LEARN>(P, V, bar, G, target, s_keys, bs_fit(P, regions), M.w, s_f, s_cnt, s_fc,
+    bs_run<R, LEARN, FI>(P, V, bar, G, target, s_keys, bs_fit(P, regions), M.w, s_f, s_cnt, s_fc,
                      [&](int t, int c, uint32_t g, auto &open, BsLane<FitShared> &L) {
                          return phase_mix_bs<SB, R, UB, LEARN>(P, M, t, c, g, open, L, s_f, s_fc);
                      });

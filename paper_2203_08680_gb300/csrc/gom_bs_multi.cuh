@@ -419,14 +419,14 @@ __host__ __device__ __forceinline__ int bs_multi_words(int S, int wv, int warps,
     return warps * 32 * kFitPlanes + (items > big ? items : big);
 }
 
-template <int R, int UB>
+template <int R, int UB, bool FI = true>
 __device__ __forceinline__ void bs_multi_generations(const GomParams &P, const VGrid &V, GomBarrier *bar, int G,
                                                      int64_t target, unsigned long long *s_keys, uint32_t *area,
                                                      long long *s_f, unsigned long long *s_cnt)
 {
     uint32_t *regions = area + (blockDim.x >> 5) * 32 * kFitPlanes;
     const BsMap M = bs_map<false>(P, V, regions);
-    bs_run<R, false>(P, V, bar, G, target, s_keys, area + threadIdx.x / 32 * 32 * kFitPlanes + (threadIdx.x & 31), M.w,
+    bs_run<R, false, FI>(P, V, bar, G, target, s_keys, area + threadIdx.x / 32 * 32 * kFitPlanes + (threadIdx.x & 31), M.w,
                      s_f, s_cnt, nullptr, [&](int t, int c, uint32_t g, auto &open, BsLane<FitShared> &L) {
                          return phase_mix_multi<R, UB>(P, V, M, regions, t, c, g, open, L, s_f);
                      });

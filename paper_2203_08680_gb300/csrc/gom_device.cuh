@@ -184,6 +184,7 @@ __device__ bool grid_barrier(unsigned long long *count, int *err, unsigned nblk,
 {
     __shared__ int s_ok;
     __syncthreads();
+    if (nblk == 1) return true; // (a block of its own: its barrier is enough, the counter stays)
     if (threadIdx.x == 0) {
         red_add_release_u64(count, 1ull);
         s_ok = barrier_poll(count, err, nblk, next, limit_ns);
@@ -194,16 +195,17 @@ __device__ bool grid_barrier(unsigned long long *count, int *err, unsigned nblk,
 
 // The barrier in two halves: what a block does between them overlaps the other
 // blocks' arrival.  Both are called by every thread of the block.
-__device__ __forceinline__ void grid_arrive(unsigned long long *count)
+__device__ __forceinline__ void grid_arrive(unsigned long long *count, unsigned nblk)
 {
     __syncthreads();
-    if (threadIdx.x == 0) red_add_release_u64(count, 1ull);
+    if (threadIdx.x == 0 && nblk > 1) red_add_release_u64(count, 1ull);
 }
 
 __device__ bool grid_wait(unsigned long long *count, int *err, unsigned nblk, unsigned long long &next,
                           unsigned long long limit_ns)
 {
     __shared__ int s_ok;
+    if (nblk == 1) return true; // (the block met in grid_arrive)
     if (threadIdx.x == 0) s_ok = barrier_poll(count, err, nblk, next, limit_ns);
     __syncthreads();
     return s_ok;
