@@ -443,7 +443,7 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
         warps_per_block = static_cast<int>(std::min<int64_t>(kMixThreads / 32, kSmemBudget / (base_words * 4)));
     }
     if (warps_per_block < 1) return GOM_E_LIMIT;
-    c->mix_threads = 32 * warps_per_block;
+    c->mix_threads = c->run_threads = 32 * warps_per_block;
     // shared-memory words of a block's staging outside stage-all mode
     const int64_t block_words =
         blk ? base_words + (warps_per_block - 1) * xw_words : base_words * warps_per_block;
@@ -482,6 +482,22 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
             c->prm.stage_all = 1;
             c->can_persist = true;
             warp_words = all_words;
+            // a group that fits one larger block: its barriers stay inside the
+            // block and its rows in one SM's L1 (10x10 torus, p = 16: 49 -> 41
+            // us a generation against two blocks of eight warps)
+            const int64_t items = max_group * per;
+            const size_t block_smem = static_cast<size_t>(c->k) * all_words * 4 * items;
+            if (grid_all > 1 && items <= kRunThreads / 32 && block_smem <= static_cast<size_t>(kSmemBudget)) {
+                int occ_one = 0;
+                GOM_CUDA(c, raise_smem_limit(c->run_fn, block_smem));
+                GOM_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_one, c->run_fn, static_cast<int>(32 * items),
+                                                                          block_smem));
+                if (occ_one > 0) {
+                    c->run_threads = static_cast<int>(32 * items);
+                    c->run_smem = block_smem;
+                    c->grid_run = 1;
+                }
+            }
         } else {
             const size_t one_smem = std::max(keys_smem, static_cast<size_t>(block_words * 4));
             int grid_one = 0;
@@ -778,15 +794,16 @@ int gom_generation(gom_ctx_t *ctx, int32_t num_generations, int64_t target_fitne
             int gens = chunk;
             int64_t target = target_fitness;
             void *args[] = {&prm, &gens, &target};
-            if (use_bs(ctx) && ctx->run_ms_fn && !ctx->prm.learn)
-                GOM_CUDA(ctx, cudaLaunchCooperativeKernel(ctx->run_ms_fn, dim3(ctx->ms_grid), dim3(kBsThreads), args,
-                                                          ctx->ms_smem, ctx->stream));
-            else if (use_bs(ctx))
-                GOM_CUDA(ctx, cudaLaunchCooperativeKernel(ctx->run_bs_fn, dim3(ctx->bs_grid_run), dim3(ctx->bs_threads),
-                                                          args, ctx->bs_smem, ctx->stream));
-            else
-                GOM_CUDA(ctx, cudaLaunchCooperativeKernel(ctx->run_fn, dim3(ctx->grid_run), dim3(ctx->mix_threads),
-                                                          args, ctx->run_smem, ctx->stream));
+            const bool bs = use_bs(ctx), ms = bs && ctx->run_ms_fn && !ctx->prm.learn;
+            const int grid = ms ? ctx->ms_grid : bs ? ctx->bs_grid_run : ctx->grid_run;
+            if (ctx->bar_grid != grid) { // the barrier counts in multiples of its grid
+                GOM_CUDA(ctx, cudaMemsetAsync(ctx->prm.bar, 0, sizeof(GomBarrier), ctx->stream));
+                ctx->bar_grid = grid;
+            }
+            GOM_CUDA(ctx, cudaLaunchCooperativeKernel(
+                              ms ? ctx->run_ms_fn : bs ? ctx->run_bs_fn : ctx->run_fn, dim3(grid),
+                              dim3(ms ? kBsThreads : bs ? ctx->bs_threads : ctx->run_threads), args,
+                              ms ? ctx->ms_smem : bs ? ctx->bs_smem : ctx->run_smem, ctx->stream));
         } else {
             k_begin_call<<<1, 1, 0, ctx->stream>>>(ctx->prm, target_fitness);
             GOM_CUDA(ctx, cudaGetLastError());

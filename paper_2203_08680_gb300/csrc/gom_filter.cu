@@ -268,7 +268,7 @@ int gom_filter_set_mode(gom_ctx_t *ctx, int32_t mode)
     if (ctx->can_persist) {
         GOM_CUDA(ctx, raise_smem_limit(run, ctx->run_smem));
         int occ = 0;
-        GOM_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, run, ctx->mix_threads, ctx->run_smem));
+        GOM_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, run, ctx->run_threads, ctx->run_smem));
         if (static_cast<int64_t>(occ) * ctx->sms < ctx->grid_run) return GOM_E_STATE;
     }
     if (mode > 0) {

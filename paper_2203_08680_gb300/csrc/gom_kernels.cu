@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(1024) k_gen_end(GomParams P)
 }
 
 template <int WPI, typename MaskT, typename AccT, bool LEARN>
-__global__ void __launch_bounds__(kMixThreads, 3) k_run(GomParams P, int G, int64_t target)
+__global__ void __launch_bounds__(kRunThreads, 1) k_run(GomParams P, int G, int64_t target)
 {
     extern __shared__ __align__(16) uint32_t s_dyn[];
     __shared__ long long s_f[1024];
