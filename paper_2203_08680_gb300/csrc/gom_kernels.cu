@@ -241,7 +241,7 @@ __global__ void k_export_elite(GomParams P, uint8_t *out)
 // Packs uint8 rows in[i*n + v] into the bit-sliced O, copies the elitist, and
 // sets the state of an import: the given elitist fitness and generation
 // counter, the fitness array zeroed for the evaluation that follows.
-__global__ void __launch_bounds__(kRowThreads) k_import_pop(GomParams P, const uint8_t *in, const uint8_t *elite,
+__global__ void __launch_bounds__(kRowThreads, 4) k_import_pop(GomParams P, const uint8_t *in, const uint8_t *elite,
                                                             int64_t fe, int64_t g)
 {
     __shared__ __align__(16) uint32_t sm[row_words(32)];

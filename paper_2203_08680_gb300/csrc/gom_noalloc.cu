@@ -88,7 +88,7 @@ cudaError_t scratch_address(uint32_t **out)
     return cudaSuccess;
 }
 
-__global__ void __launch_bounds__(kRowThreads)
+__global__ void __launch_bounds__(kRowThreads, 4)
     k_noalloc_pack(const uint8_t *pop, int32_t n, int32_t p, int32_t W, uint32_t *words, int64_t *fit)
 {
     __shared__ __align__(16) uint32_t sm[row_words(32)];

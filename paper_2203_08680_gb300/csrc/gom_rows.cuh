@@ -15,7 +15,7 @@ namespace {
 // ---- rows <-> words.  Bound by memory: a warp moves 128 variables of 32
 // individuals (one word column) with 4 bytes a lane and row, and the block
 // turns the words of 128 variables through shared memory, so that both sides
-// are read and written in whole lines.  torus1000, p = 256: import 709 -> 169
+// are read and written in whole lines.  torus1000, p = 256: import 709 -> 92
 // us, export 600 -> 78 us (256 MB of rows; one byte a lane and row before).
 constexpr int kRowVars = 128;
 constexpr int kRowThreads = 256;
@@ -63,6 +63,7 @@ __device__ __forceinline__ void pack_rows(const uint8_t *in, int n, int p, int W
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int T = row_tiles(W), stride = row_stride(W), lw = __ffs(W) - 1;
     const uint8_t *end = in + (int64_t)p * n;
+    const bool aligned = !(n & 3) && !(reinterpret_cast<uintptr_t>(in) & 3); // then no word passes a row's end
     const int64_t tiles = (n + kRowVars - 1) / kRowVars;
     for (int64_t t0 = (int64_t)blockIdx.x * T; t0 < tiles; t0 += (int64_t)gridDim.x * T) {
         for (int task = wib; task < T * W; task += kRowThreads / 32) {
@@ -74,14 +75,20 @@ __device__ __forceinline__ void pack_rows(const uint8_t *in, int n, int p, int W
                 const uint32_t valid = n - v >= 4 ? 0x01010101u : 0x01010101u >> (8 * (4 - (int)(n - v)));
                 const uint8_t *at = in + 32 * (int64_t)w * n + v;
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    uint32_t x[8];
+                for (int k = 0; k < 4; k += 2) { // 16 rows' loads in flight
+                    uint32_t x[16];
+                    if (aligned) {
 #pragma unroll
-                    for (int b = 0; b < 8; ++b) x[b] = 8 * k + b < rows ? load4(at + (int64_t)(8 * k + b) * n, in, end) : 0u;
+                        for (int b = 0; b < 16; ++b)
+                            x[b] = 8 * k + b < rows ? __ldg(reinterpret_cast<const uint32_t *>(at + (int64_t)(8 * k + b) * n)) : 0u;
+                    } else {
 #pragma unroll
-                    for (int b = 0; b < 8; ++b) { // bit 7 of a byte: the byte is not zero
+                        for (int b = 0; b < 16; ++b) x[b] = 8 * k + b < rows ? load4(at + (int64_t)(8 * k + b) * n, in, end) : 0u;
+                    }
+#pragma unroll
+                    for (int b = 0; b < 16; ++b) { // bit 7 of a byte: the byte is not zero
                         const uint32_t nz = (((x[b] & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | x[b]) >> 7;
-                        acc[k] |= (nz & valid) << b;
+                        acc[k + (b >> 3)] |= (nz & valid) << (b & 7);
                     }
                 }
             }
@@ -157,8 +164,8 @@ __device__ __forceinline__ void unpack_rows(const uint32_t *words, int n, int p,
 // individual took about 12 for 32.  Weights go in bytes: a pass over the
 // edges per byte that any weight has (the first for |w| < 256).  A negative
 // weight counts where the edge is not cut, less |w| for everyone.
-// 1000x1000 torus, p = 256: 1638 -> 163 us; 200,000 vertices of degree 6, p =
-// 512: 918 -> 124 us.
+// 1000x1000 torus, p = 256: 1638 -> 155 us; 200,000 vertices of degree 6, p =
+// 512: 918 -> 119 us.
 constexpr int kCutPlanes = 24;
 constexpr int kCutFlush = 500; // four-edge steps: 500 * 4 * 255 * 32 slots < 2^24
 
@@ -261,40 +268,57 @@ __device__ __forceinline__ void cut_sums(const uint32_t *words, int n, int p, in
     for (int byte = 0; byte < 4; ++byte) {
         if (byte > 0 && !(all >> (8 * byte))) break;
         int steps = 0;
+        // one vertex a slot; the next one's row bounds and the next four edges
+        // are on their way while four edges' words arrive and are added
+        int64_t u = gwarp * E + slot, e, end;
+        int v[4], wt[4];
+        const auto row = [&](int64_t x, int64_t *from, int64_t *to) {
+            const bool have = in && x < n;
+            *from = have ? __ldg(row_ptr + x) : 0;
+            *to = have ? __ldg(row_ptr + x + 1) : 0;
+        };
+        const auto edges = [&](int64_t from, int64_t to) {
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                v[x] = from + x < to ? __ldg(col + from + x) : -1;
+                wt[x] = from + x < to ? __ldg(wgt + from + x) : 0;
+            }
+        };
+        row(u, &e, &end);
+        edges(e, end);
         for (int64_t u0 = gwarp * E; u0 < n; u0 += nwarps * E) {
-            const int64_t u = u0 + slot;
-            const bool have = in && u < n;
-            int64_t e = have ? __ldg(row_ptr + u) : 0;
-            const int64_t end = have ? __ldg(row_ptr + u + 1) : 0;
-            const uint32_t xu = have ? words[u * W + w] : 0u;
-            while (__any_sync(0xFFFFFFFFu, e < end)) {
-                int v[4], wt[4];
+            int64_t e2, end2;
+            row(u + nwarps * E, &e2, &end2);
+            const uint32_t xu = in && u < n ? words[u * W + w] : 0u;
+            for (bool more = true; more;) {
                 uint32_t d[4], mag[4];
 #pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    v[x] = e + x < end ? __ldg(col + e + x) : -1;
-                    wt[x] = e + x < end ? __ldg(wgt + e + x) : 0;
-                }
-#pragma unroll
                 for (int x = 0; x < 4; ++x) d[x] = v[x] > u ? words[(int64_t)v[x] * W + w] : 0u; // each edge once
+                uint32_t neg[4];
 #pragma unroll
                 for (int x = 0; x < 4; ++x) {
-                    const uint32_t neg = (uint32_t)(wt[x] >> 31);
-                    mag[x] = v[x] > u ? ((uint32_t)wt[x] ^ neg) - neg : 0u;
-                    d[x] ^= xu ^ neg;
+                    neg[x] = (uint32_t)(wt[x] >> 31);
+                    mag[x] = v[x] > u ? ((uint32_t)wt[x] ^ neg[x]) - neg[x] : 0u;
                     if (byte == 0) {
                         all |= mag[x];
-                        if (neg && v[x] > u && w == 0) neg_sum += wt[x];
+                        if (neg[x] && v[x] > u && w == 0) neg_sum += wt[x];
                     }
                     mag[x] >>= 8 * byte;
                 }
-                add_bytes4(acc, d, mag);
                 e += 4;
+                more = __any_sync(0xFFFFFFFFu, e < end);
+                edges(more ? e : e2, more ? end : end2);
+#pragma unroll
+                for (int x = 0; x < 4; ++x) d[x] ^= xu ^ neg[x];
+                add_bytes4(acc, d, mag);
                 if (++steps == kCutFlush) {
                     cut_flush(acc, Wv, slot, in ? w : Wv, E, 8 * byte, s_f);
                     steps = 0;
                 }
             }
+            u += nwarps * E;
+            e = e2;
+            end = end2;
         }
         if (byte == 0) all = __reduce_or_sync(0xFFFFFFFFu, all);
         cut_flush(acc, Wv, slot, in ? w : Wv, E, 8 * byte, s_f);
