@@ -247,12 +247,19 @@ int ctx_read_stats(gom_ctx *ctx, int32_t num, gom_gen_stats_t *host_stats, int32
     if (run_out) *run_out = run;
     if (host_stats) {
         std::memset(host_stats, 0, sizeof(gom_gen_stats_t) * num);
-        std::vector<GomDevStats> ring(kStatsCap);
-        GOM_CUDA(ctx, cudaMemcpyAsync(ring.data(), ctx->prm.stats, sizeof(GomDevStats) * kStatsCap,
-                                      cudaMemcpyDeviceToHost, ctx->stream));
+        // only the entries of this call, in at most two pieces of the ring
+        const int32_t n = std::min(run, num), first = static_cast<int32_t>(st.call_g0 % kStatsCap);
+        const int32_t head = std::min(n, kStatsCap - first);
+        std::vector<GomDevStats> ring(n);
+        if (head > 0)
+            GOM_CUDA(ctx, cudaMemcpyAsync(ring.data(), ctx->prm.stats + first, sizeof(GomDevStats) * head,
+                                          cudaMemcpyDeviceToHost, ctx->stream));
+        if (n > head)
+            GOM_CUDA(ctx, cudaMemcpyAsync(ring.data() + head, ctx->prm.stats, sizeof(GomDevStats) * (n - head),
+                                          cudaMemcpyDeviceToHost, ctx->stream));
         GOM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-        for (int32_t q = 0; q < run && q < num; ++q) {
-            const GomDevStats &S = ring[(st.call_g0 + q) % kStatsCap];
+        for (int32_t q = 0; q < n; ++q) {
+            const GomDevStats &S = ring[q];
             gom_gen_stats_t &H = host_stats[q];
             H.generation = S.generation;
             H.best_fitness = S.best;

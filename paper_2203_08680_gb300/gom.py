@@ -56,6 +56,15 @@ class GenStats(C.Structure):
         return {k: int(getattr(self, k)) for k, _ in self._fields_}
 
 
+_STATS_NAMES = [name for name, _ in GenStats._fields_]
+
+
+def _stats_dicts(arr, count: int):
+    """The first `count` entries of a GenStats array (int64 fields only) as dicts."""
+    rows = np.frombuffer(arr, dtype=np.int64).reshape(-1, len(_STATS_NAMES))[:count].tolist()
+    return [dict(zip(_STATS_NAMES, row)) for row in rows]
+
+
 _lib = None
 
 # (name, restype, argtypes) of every entry point declared in include/gom.h
@@ -326,7 +335,7 @@ def gom_generation(ctx: Ctx, num_generations: int, target_fitness: int = INT64_M
     arr = (GenStats * max(num_generations, 1))()
     run = C.c_int32()
     _check(load().gom_generation(ctx.h, num_generations, target_fitness, arr, C.byref(run)), "gom_generation", ctx)
-    return [arr[q].as_dict() for q in range(run.value)], int(run.value)
+    return _stats_dicts(arr, run.value), int(run.value)
 
 
 def gom_fitness(ctx: Ctx, d_fitness_out):
@@ -490,7 +499,7 @@ def gom_batch_stats(batch: Batch, b: int, capacity: int):
     arr = (GenStats * max(capacity, 1))()
     cnt = C.c_int32()
     _check(load().gom_batch_stats(batch.h, b, arr, capacity, C.byref(cnt)), "gom_batch_stats")
-    return [arr[q].as_dict() for q in range(cnt.value)]
+    return _stats_dicts(arr, cnt.value)
 
 
 def gom_batch_layout(batch: Batch, b: int):
