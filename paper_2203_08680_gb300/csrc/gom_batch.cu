@@ -96,6 +96,14 @@ bool batch_multi(const gom_ctx *c, const gom_batch_config_t &conf, int level)
     return level == 0 && c->run_ms_fn && conf.min_blocks == 2 && conf.warps_per_block >= 4;
 }
 
+// The element size a single-class bit-sliced instance runs as: its own, with
+// 16-bit weights the next of the classes the batched kernel has for them.
+int batch_bs_s(const gom_ctx *c)
+{
+    const int s = static_cast<int>(std::max<int64_t>(c->max_s, 1));
+    return c->bs_ub == 8 || s > 16 ? s : s <= 8 ? 8 : 16;
+}
+
 // Whether an instance on `warps` warps runs the bit-sliced phase (only in the
 // kernel with the larger register budget, min_blocks 2): as the caller set it
 // for the context, else where its largest group gives every warp four pairs or
@@ -210,7 +218,7 @@ int batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config_t *
                     max_warp_words, (gom_bs_multi_words(static_cast<int>(c->max_s), wv, conf.warps_per_block, c->prm.ms_edges) +
                                      conf.warps_per_block - 1) / conf.warps_per_block);
             else
-                max_warp_words = std::max<int64_t>(max_warp_words, c->prm.bs_words);
+                max_warp_words = std::max<int64_t>(max_warp_words, gom_bs_warp_words(batch_bs_s(c)));
         }
         f_words = 2 * 32 * maxW;
         const int64_t slices = std::max<int64_t>(int64_t(8) * maxk, int64_t(4) * max_warp_words * conf.warps_per_block);
@@ -291,6 +299,10 @@ int batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config_t *
         const bool use_bs = batch_bits(c, conf, level, int64_t(nb[b]) * conf.warps_per_block);
         if (use_bs) {
             const bool multi = batch_multi(c, conf, level);
+            if (!multi) {
+                B->params[b].bs_S = batch_bs_s(c);
+                B->params[b].bs_words = gom_bs_warp_words(batch_bs_s(c));
+            }
             I.variant = multi ? kVarMulti : kVarBits;
             I.bs_r = c->bs_r;
             I.bs_ub = multi ? c->ms_ub : c->bs_ub;

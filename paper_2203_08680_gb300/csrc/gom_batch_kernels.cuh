@@ -84,16 +84,13 @@ __global__ void __launch_bounds__(kMixThreads, MINB)
     if (MINB == 2 && I.variant == kVarBits) { // the bit-sliced phase needs the larger register budget
         if constexpr (MINB == 2) {
             // fewer instances than the single-instance kernels have, the next wider planes for the rest
-            // (the variant's class lays its rows out, so S = 5 and 7 keep theirs)
             const int cls = bs_class(sP.bs_S);
-            if (cls == 5)
-                I.bs_ub == 8 ? batch_variant_bs<5, 16, 8>(sP, V, bar, G, I.target, S)
-                             : batch_variant_bs<5, 20, 16>(sP, V, bar, G, I.target, S);
-            else if (cls == 7)
-                I.bs_ub == 8 ? batch_variant_bs<7, 16, 8>(sP, V, bar, G, I.target, S)
-                             : batch_variant_bs<7, 20, 16>(sP, V, bar, G, I.target, S);
-            else if (I.bs_ub == 8)
-                cls == 8    ? batch_variant_bs<8, 16, 8>(sP, V, bar, G, I.target, S)
+            if (I.bs_ub == 8)
+                cls == 5    ? batch_variant_bs<5, 16, 8>(sP, V, bar, G, I.target, S)
+                : cls == 7  ? batch_variant_bs<7, 16, 8>(sP, V, bar, G, I.target, S)
+                : cls == 8  ? batch_variant_bs<8, 16, 8>(sP, V, bar, G, I.target, S)
+                : cls == 10 ? batch_variant_bs<10, 16, 8>(sP, V, bar, G, I.target, S)
+                : cls == 13 ? batch_variant_bs<13, 16, 8>(sP, V, bar, G, I.target, S)
                 : cls == 16 ? batch_variant_bs<16, 16, 8>(sP, V, bar, G, I.target, S)
                             : batch_variant_bs<32, 16, 8>(sP, V, bar, G, I.target, S);
             else

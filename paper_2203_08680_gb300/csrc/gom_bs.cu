@@ -114,6 +114,8 @@ const void *gom_run_bs_kernel(int s, int r, int ub, bool learn)
     case 5: return gom_run_bs5(r, ub, learn);
     case 7: return gom_run_bs7(r, ub, learn);
     case 8: return gom_run_bs8(r, ub, learn);
+    case 10: return gom_run_bs10(r, ub, learn);
+    case 13: return gom_run_bs13(r, ub, learn);
     case 16: return gom_run_bs16(r, ub, learn);
     default: return gom_run_bs32(r, ub, learn);
     }
@@ -125,6 +127,8 @@ const void *gom_mix_bs_kernel(int s, int r, int ub, bool learn)
     case 5: return gom_mix_bs5(r, ub, learn);
     case 7: return gom_mix_bs7(r, ub, learn);
     case 8: return gom_mix_bs8(r, ub, learn);
+    case 10: return gom_mix_bs10(r, ub, learn);
+    case 13: return gom_mix_bs13(r, ub, learn);
     case 16: return gom_mix_bs16(r, ub, learn);
     default: return gom_mix_bs32(r, ub, learn);
     }

@@ -101,14 +101,18 @@ __device__ __forceinline__ int next_run_start(const uint32_t *rs, uint32_t nz, i
 }
 
 // The kernels' element classes: instances for elements of at most SB = 5, 7, 8,
-// 16 or 32 variables (5 and 7: the neighbourhoods of degree 4 and 6; with the
-// rows known at compile time a generation of torus1000, p = 256, takes 9 %
-// less than in the class of 8).
-__host__ __device__ constexpr int bs_class(int S) { return S <= 5 ? 5 : S <= 7 ? 7 : S <= 8 ? 8 : S <= 16 ? 16 : 32; }
+// 10, 13, 16 or 32 variables.  Up to 13 the rows are known at compile time (the
+// neighbourhoods of degree 4, 6 and 7, 8 and 9, 12): a generation of torus1000,
+// p = 256, takes 9 % less in the class of 5 than in that of 8, one of random
+// 12-regular graphs 5 % less in the class of 13 than in that of 16.
+__host__ __device__ constexpr int bs_class(int S)
+{
+    return S <= 5 ? 5 : S <= 7 ? 7 : S <= 8 ? 8 : S <= 10 ? 10 : S <= 13 ? 13 : S <= 16 ? 16 : 32;
+}
 
 // Rows of a class's shared arrays: the class's in the small ones, else those of
 // the model's largest element.
-__host__ __device__ constexpr int bs_rows(int S) { return S <= 8 ? bs_class(S) : S; }
+__host__ __device__ constexpr int bs_rows(int S) { return S <= 13 ? bs_class(S) : S; }
 
 // Variables of a pattern in the class's tables: entries of 2 bytes (P_d in the
 // low byte, N_d in the high one), 4 bytes (halves) or 8 bytes (P_d, N_d) for
@@ -288,7 +292,7 @@ __device__ __forceinline__ void bs_prepare(const GomParams &P, const BsMap &M, c
                                            uint32_t g, BsItem &I)
 {
     const int lane = threadIdx.x & 31, slot = M.slot;
-    const int W = P.W, Wv = P.Wv, p = P.p, S = SB < 8 ? SB : min(P.bs_S, SB);
+    const int W = P.W, Wv = P.Wv, p = P.p, S = SB <= 13 ? SB : min(P.bs_S, SB);
     const int e = M.e, w = M.w, b2 = e * Wv; // b2: the element's first slot
     const bool ke = M.in && k0 + e < k1;     // this lane's pair exists
     int q = k0 + e;
@@ -339,9 +343,10 @@ __device__ __forceinline__ void bs_prepare(const GomParams &P, const BsMap &M, c
             constexpr int C = SB < 8 ? SB : 8;
             int at[C];
 #pragma unroll
-            for (int c = 0; c < C; ++c) at[c] = ke && a8 + c < s ? __ldg(P.fv + f0 + a8 + c) * W + w : -1;
+            for (int c = 0; c < C; ++c) at[c] = a8 + c < SB && ke && a8 + c < s ? __ldg(P.fv + f0 + a8 + c) * W + w : -1;
 #pragma unroll
-            for (int c = 0; c < C; ++c) xp[a8 + c] = at[c] >= 0 ? P.P[at[c]] : 0u;
+            for (int c = 0; c < C; ++c)
+                if (a8 + c < SB) xp[a8 + c < SB ? a8 + c : 0] = at[c] >= 0 ? P.P[at[c]] : 0u;
         }
     }
     if constexpr (SB <= 16) {
@@ -505,7 +510,7 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const BsMap &M, cons
                                         BsLane<FitShared> &L, long long *s_f, unsigned long long *s_fc)
 {
     const int slot = M.slot;
-    const int W = P.W, p = P.p, S = SB < 8 ? SB : min(P.bs_S, SB);
+    const int W = P.W, p = P.p, S = SB <= 13 ? SB : min(P.bs_S, SB);
     const int w = M.w, b2 = M.e * P.Wv, s = I.s;
     const bool ke = I.ke;
     constexpr int EW = bs_entry_words(SB), TB = bs_table(SB);
@@ -524,7 +529,7 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const BsMap &M, cons
             int at[C];
             uint32_t xo[C];
 #pragma unroll
-            for (int c = 0; c < C; ++c) at[c] = ke && a8 + c < s ? __ldg(P.fv + I.f0 + a8 + c) * W + w : -1;
+            for (int c = 0; c < C; ++c) at[c] = a8 + c < SB && ke && a8 + c < s ? __ldg(P.fv + I.f0 + a8 + c) * W + w : -1;
 #pragma unroll
             for (int c = 0; c < C; ++c) xo[c] = at[c] >= 0 ? P.O[at[c]] : 0u;
             if constexpr (SB > 16) {

@@ -41,13 +41,17 @@ const void *gom_run_multi_kernel(int ub);
 int gom_bs_multi_words(int max_s, int wv, int warps, int edges);
 // Packs the dependency lists into the bit-sliced path's edge lists (P.bdep).
 __global__ void k_bs_edges(GomParams P, int2 *bdep);
-// The instances of one element class (5, 7, 8, 16 or 32 variables at most).
+// The instances of one element class (5, 7, 8, 10, 13, 16 or 32 variables at most).
 const void *gom_run_bs5(int r, int ub, bool learn);
 const void *gom_mix_bs5(int r, int ub, bool learn);
 const void *gom_run_bs7(int r, int ub, bool learn);
 const void *gom_mix_bs7(int r, int ub, bool learn);
 const void *gom_run_bs8(int r, int ub, bool learn);
 const void *gom_mix_bs8(int r, int ub, bool learn);
+const void *gom_run_bs10(int r, int ub, bool learn);
+const void *gom_mix_bs10(int r, int ub, bool learn);
+const void *gom_run_bs13(int r, int ub, bool learn);
+const void *gom_mix_bs13(int r, int ub, bool learn);
 const void *gom_run_bs16(int r, int ub, bool learn);
 const void *gom_mix_bs16(int r, int ub, bool learn);
 const void *gom_run_bs32(int r, int ub, bool learn);
