@@ -639,7 +639,7 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
             most_pairs = std::max(most_pairs, count[1] + count[2] + count[3]);
             most_units = std::max(most_units, count[0] + (count[1] + count[2] + count[3]));
         }
-        const int wpb = kBsThreads / 32;
+        const int wpb = kMsThreads / 32;
         const size_t smem = std::max(static_cast<size_t>(256 * c->W) +
                                          sizeof(uint32_t) * gom_bs_multi_words(static_cast<int>(tabs.max_s), wv, wpb,
                                                                                static_cast<int>(large_edges)),
@@ -648,7 +648,7 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
         int occ_s = 0;
         if ((top == 0 || 2 * below >= c->m) && smem <= static_cast<size_t>(kSmemBudget)) {
             GOM_CUDA(c, raise_smem_limit(fn, smem));
-            GOM_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_s, fn, kBsThreads, smem));
+            GOM_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_s, fn, kMsThreads, smem));
         }
         if (occ_s > 0) {
             c->run_ms_fn = fn;
@@ -657,7 +657,9 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
             c->ms_edges = small_edges;
             c->prm.ms_edges = static_cast<int32_t>(large_edges);
             const int64_t warps = static_cast<int64_t>(c->sms) * occ_s * wpb;
-            bs_split(wv, std::max<int64_t>(most_pairs, 1), small_edges, warps, wpb, &c->prm.bs_lsh, &c->prm.bs_nwi);
+            // (tiles of at most four warps: the per-launch path's blocks have four)
+            bs_split(wv, std::max<int64_t>(most_pairs, 1), small_edges, warps, kBsThreads / 32, &c->prm.bs_lsh,
+                     &c->prm.bs_nwi);
             // a block for every large element and small element of a group up to one per SM, then four tiles a block
             c->ms_grid = static_cast<int>(std::min<int64_t>(
                 static_cast<int64_t>(c->sms) * occ_s,
@@ -809,7 +811,7 @@ int gom_generation(gom_ctx_t *ctx, int32_t num_generations, int64_t target_fitne
             }
             GOM_CUDA(ctx, cudaLaunchCooperativeKernel(
                               ms ? ctx->run_ms_fn : bs ? ctx->run_bs_fn : ctx->run_fn, dim3(grid),
-                              dim3(ms ? kBsThreads : bs ? ctx->bs_threads : ctx->run_threads), args,
+                              dim3(ms ? kMsThreads : bs ? ctx->bs_threads : ctx->run_threads), args,
                               ms ? ctx->ms_smem : bs ? ctx->bs_smem : ctx->run_smem, ctx->stream));
         } else {
             k_begin_call<<<1, 1, 0, ctx->stream>>>(ctx->prm, target_fitness);

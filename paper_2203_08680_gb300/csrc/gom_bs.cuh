@@ -155,9 +155,9 @@ struct BsMap {
     uint32_t *sm;     // the tile's shared region
 };
 
-// The tile's map; `regions` is the block's first warp region.
+// The tile's map; `regions` is the block's first warp region, `words` a region's size.
 template <bool LEARN>
-__device__ __forceinline__ BsMap bs_map(const GomParams &P, const VGrid &V, uint32_t *regions)
+__device__ __forceinline__ BsMap bs_map(const GomParams &P, const VGrid &V, uint32_t *regions, int words)
 {
     BsMap M;
     const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -172,24 +172,29 @@ __device__ __forceinline__ BsMap bs_map(const GomParams &P, const VGrid &V, uint
     M.w = M.slot - M.e * P.Wv;
     M.sub = lane & ((1 << M.lsh) - 1);
     M.in = M.e < M.E;
-    M.sm = regions + tb * M.nwi * P.bs_words;
+    M.sm = regions + tb * M.nwi * words;
     return M;
 }
 
 // Waits for the tile's threads (every thread of the tile calls it): a warp, a
-// whole block of four warps, or half of one on a named barrier.  The barrier
-// numbers are constants: a number in a register makes the compiler reserve all
-// 16 of a block, and an SM's 64 then hold four blocks.
+// whole block, or some of its warps on a named barrier.  The barrier numbers
+// are constants: a number in a register makes the compiler reserve all 16 of a
+// block, and an SM's 64 then hold four blocks.
 __device__ __forceinline__ void tile_sync(const BsMap &M)
 {
-    if (M.nwi == 1)
+    const int n = 32 * M.nwi;
+    if (M.nwi == 1) {
         __syncwarp();
-    else if (M.nwi == kBsThreads / 32)
+    } else if (n == (int)blockDim.x) {
         __syncthreads();
-    else if (threadIdx.x < kBsThreads / 2)
-        asm volatile("bar.sync 1, 64;" ::: "memory");
-    else
-        asm volatile("bar.sync 2, 64;" ::: "memory");
+    } else {
+        switch ((int)(threadIdx.x >> 5) / M.nwi) { // at most four tiles of several warps in a block of eight
+        case 0: asm volatile("bar.sync 1, %0;" ::"r"(n) : "memory"); break;
+        case 1: asm volatile("bar.sync 2, %0;" ::"r"(n) : "memory"); break;
+        case 2: asm volatile("bar.sync 3, %0;" ::"r"(n) : "memory"); break;
+        default: asm volatile("bar.sync 4, %0;" ::"r"(n) : "memory"); break;
+        }
+    }
 }
 
 // Learned filter bookkeeping after a bit-sliced item (warp-wide): each
@@ -834,7 +839,7 @@ __device__ __forceinline__ void bs_generations(const GomParams &P, const VGrid &
                                                int64_t target, unsigned long long *s_keys, uint32_t *regions,
                                                long long *s_f, unsigned long long *s_cnt, unsigned long long *s_fc)
 {
-    const BsMap M = bs_map<LEARN>(P, V, regions);
+    const BsMap M = bs_map<LEARN>(P, V, regions, P.bs_words);
     bs_run<R, LEARN, FI>(P, V, bar, G, target, s_keys, bs_fit(P, regions), M.w, s_f, s_cnt, s_fc,
                      [&](int t, int c, uint32_t g, auto &open, BsLane<FitShared> &L) {
                          return phase_mix_bs<SB, R, UB, LEARN>(P, M, t, c, g, open, L, s_f, s_fc);

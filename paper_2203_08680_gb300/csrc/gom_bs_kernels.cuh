@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(kBsThreads, bs_blocks(SB)) k_mix_bs(GomParams 
     if (P.st->done) return;
     fc_zero(s_fc);
     acc_zero(P, s_f, s_cnt);
-    const BsMap M = bs_map<LEARN>(P, whole_grid(), s_dyn + 64 * P.W);
+    const BsMap M = bs_map<LEARN>(P, whole_grid(), s_dyn + 64 * P.W, P.bs_words);
     BsLane<FitShared> L;
     L.fit.v = bs_fit(P, s_dyn + 64 * P.W);
     bs_lane_zero(L, M.w);

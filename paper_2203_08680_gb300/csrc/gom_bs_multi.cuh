@@ -13,7 +13,7 @@
 // call for four starts and one 16-byte table entry per pattern; the flip
 // planes by the inverse transposes; then the element's edges split over the
 // block's warps and their plane sums added.  Group of a 100x100 torus' tree of
-// bound 128 (p = 1,024; 25 elements above 64 variables, 900 below 9): 85 -> 23
+// bound 128 (p = 1,024; 25 elements above 64 variables, 900 below 9): 85 -> 19
 // us against a block per element and scalar deltas for every size.
 #pragma once
 
@@ -415,7 +415,7 @@ __device__ __forceinline__ bool phase_mix_multi(const GomParams &P, const VGrid 
 // warps' fitness planes, then the warps' item regions or a large element's.
 __host__ __device__ __forceinline__ int bs_multi_words(int S, int wv, int warps, bool large, int edges)
 {
-    const int items = warps * bs_warp_words(S), big = large ? bs_large_words(wv, warps, edges) : 0;
+    const int items = warps * (bs_warp_words(S) - 32 * kFitPlanes), big = large ? bs_large_words(wv, warps, edges) : 0;
     return warps * 32 * kFitPlanes + (items > big ? items : big);
 }
 
@@ -425,7 +425,7 @@ __device__ __forceinline__ void bs_multi_generations(const GomParams &P, const V
                                                      long long *s_f, unsigned long long *s_cnt)
 {
     uint32_t *regions = area + (blockDim.x >> 5) * 32 * kFitPlanes;
-    const BsMap M = bs_map<false>(P, V, regions);
+    const BsMap M = bs_map<false>(P, V, regions, P.bs_words - 32 * kFitPlanes); // (the planes stand ahead)
     bs_run<R, false, FI>(P, V, bar, G, target, s_keys, area + threadIdx.x / 32 * 32 * kFitPlanes + (threadIdx.x & 31), M.w,
                      s_f, s_cnt, nullptr, [&](int t, int c, uint32_t g, auto &open, BsLane<FitShared> &L) {
                          return phase_mix_multi<R, UB>(P, V, M, regions, t, c, g, open, L, s_f);

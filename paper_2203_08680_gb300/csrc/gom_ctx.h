@@ -188,7 +188,7 @@ inline bool bs_pays(int wv, int64_t max_group, int64_t max_s, bool stage_all, in
 {
     if (stage_all && (wv == 1 || max_group * wv <= 1024)) return false;
     if (max_s <= 16 || max_s > 64) return true;
-    return !(wv == 1 && max_group <= 4 * warps) && max_group * wv > 256;
+    return !(wv == 1 && max_group <= 4 * warps) && max_group * wv > 512;
 }
 
 // Raises a kernel's dynamic shared memory limit to at least `bytes`, never

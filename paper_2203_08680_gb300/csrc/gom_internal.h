@@ -181,7 +181,8 @@ struct GomFI {
 constexpr int kStatsCap = 1024;    // per-generation counters kept on the device
 constexpr int kMixThreads = 256;   // mixing kernel block size (8 warps)
 constexpr int kRunThreads = 768;   // largest block of the per-lane persistent kernel (as many registers as three of 256)
-constexpr int kBsThreads = 128;    // bit-sliced kernels' block size (4 warps; 5 blocks per SM)
+constexpr int kBsThreads = 128;    // bit-sliced kernels' block size (4 warps)
+constexpr int kMsThreads = 256;    // block of the bit-sliced kernels by element class (8 warps)
 constexpr int kStageAllMaxK = 128; // most colour groups of the stage-all mode (group order held per block)
 constexpr uint32_t kTagInit = 0x494E4954u;
 constexpr uint32_t kTagDonor = 0x444F4E52u;
