@@ -1,6 +1,6 @@
 """In-tree build of libgom.so (the CUDA library behind include/gom.h).
 
-Compiles the two CUDA translation units with nvcc for sm_103a only and the
+Compiles the CUDA translation units with nvcc for sm_103a only and the
 host set-up code with g++, in parallel, then links one shared library next to
 this file.  No cmake; a rebuild happens only when a source is newer than the
 library.

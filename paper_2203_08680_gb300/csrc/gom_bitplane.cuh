@@ -41,28 +41,6 @@ __device__ __forceinline__ void transpose_lane(uint32_t (&x)[NR])
 // x & (bit t of u ? ~0 : 0), for a per-lane weight u.
 __device__ __forceinline__ uint32_t bit_mask(uint32_t x, uint32_t u, int t) { return ((u >> t) & 1u) ? x : 0u; }
 
-// acc += u * x over R bit-planes (ripple carry; u < 2^UB; the sum stays below
-// 2^R by the caller's bound, so the last carry is always zero).
-template <int R, int UB, int NA>
-__device__ __forceinline__ void add_weighted(uint32_t (&acc)[NA], uint32_t x, uint32_t u)
-{
-    static_assert(NA >= R, "accumulator narrower than R");
-    uint32_t carry = 0;
-#pragma unroll
-    for (int t = 0; t < R; ++t) {
-        if (t < UB) {
-            const uint32_t in = bit_mask(x, u, t);
-            const uint32_t a = acc[t];
-            acc[t] = a ^ in ^ carry;
-            carry = (a & in) | (a & carry) | (in & carry);
-        } else {
-            const uint32_t a = acc[t];
-            acc[t] = a ^ carry;
-            carry = a & carry;
-        }
-    }
-}
-
 // D += u * pos - u * neg over NP bit-planes, two's complement (pos and neg
 // disjoint; u < 2^UB).  A lane that subtracts adds the complement of u with a
 // carry of one in: its planes are ~u below UB, all ones above (the sign

@@ -1,9 +1,10 @@
 // gom_bs.cuh -- the bit-sliced mixing path of parallel GOM for weighted Max-Cut:
-// its device code, shared by its own kernels (gom_bs.cu) and the batched
-// kernel (gom_kernels.cu).  Anonymous namespace: each translation unit that
+// its device code, shared by its own kernels (gom_bs_kernels.cuh), those by
+// element class (gom_bs_multi.cuh) and the batched kernel
+// (gom_batch_kernels.cuh).  Anonymous namespace: each translation unit that
 // includes it compiles its own copy.
 //
-// Same generations as the per-lane path of gom_kernels.cu (Alg. 3; every
+// Same generations as the per-lane path of gom_lane.cuh (Alg. 3; every
 // trial of Alg. 2 decided by the exact integer delta), with the partial
 // evaluation, the acceptance and the fitness bookkeeping done on bit-planes:
 // one 32-bit register holds one bit of 32 individuals, so one logic
@@ -16,9 +17,8 @@
 // repeat phase 0 and split the donor draws and the element's edges), and an
 // element whose lanes pass one warp takes 2 or 4 warps of a block (BsMap).
 // Per item:
-//   phase 0  (lane = pair) the parent's current rows on F_j into shared
-//            memory, the generation-start rows of P on F_j in registers; the
-//            run starts of P's patterns (bit d: pattern d differs from pattern
+//   phase 0  (lane = pair) the generation-start rows of P on F_j; the run
+//            starts of P's patterns (bit d: pattern d differs from pattern
 //            d - 1, cyclically); then, by a bit transpose inside the lane, the
 //            pattern P_d of each of its 32 individuals, and by one backward
 //            walk over them the pattern N_d of the next run start after d: one
@@ -26,7 +26,8 @@
 //   phase 1  (lane = 4 individuals of a pair) the donor search of Sec. 4.2: one
 //            Philox call gives 4 starts; one table entry per trial holds the
 //            start's pattern and the pattern the search falls through to when
-//            the start equals the parent.  (Lane = pair) the 32 entries come
+//            the start equals the parent.  So far everything comes from P: this
+//            is bs_prepare, the rest bs_item.  (Lane = pair) the 32 entries come
 //            back through the inverse transpose as bit-planes T1_a (the
 //            starts' bits) and T2_a (the fall-through's), and the flip planes
 //            F_a (bit b: individual b flips variable a) are a plane select;
@@ -55,7 +56,8 @@
 // 2.27 to 1.31 ms against tables of packed patterns transposed across the warp
 // with a run-start search per trial; one flat edge list per element and chains
 // over four edges took it to 1.10 ms (103 warp instructions per 32 trials, the
-// ALU pipe busy 65 % of the cycles).
+// ALU pipe busy 65 % of the cycles), instances with the rows known at compile
+// time and selects shared with the multiply pipe to 0.98 ms.
 //
 // Elements of one colour group share no variable and no edge (LMIG
 // colouring), so the rows a pair reads and writes belong to it alone during
