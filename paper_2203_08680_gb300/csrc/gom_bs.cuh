@@ -641,6 +641,7 @@ __device__ __forceinline__ void bs_item(const GomParams &P, const BsMap &M, cons
             hd |= Fa;
             sF[32 * a + slot] = Fa;
         }
+    __syncwarp(); // every lane of a pair has stored its planes: the first one may correct them
     // An individual that is itself the run start the search falls through to
     // is skipped (a donor is another individual).  Its start equals the parent
     // and the fall-through is its own pattern in P, another one: only an

@@ -1,0 +1,54 @@
+"""Which path a call takes and what it leaves behind, against the CPU oracle: shared lanes of the bit-sliced mixing, launches
+that follow one another on different kernels."""
+import numpy as np
+import pytest
+
+from paper_2203_08680_gb300 import gom
+from paper_2203_08680_gb300 import instances as I
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from test_gpu_bs_items import _windows  # noqa: E402
+from test_gpu_parity import _assert_same_state, _assert_same_stats, _gpu_state  # noqa: E402
+
+
+def _few_rows(oracle, g, p, rows, seed):
+    """A population of `rows` distinct rows, its cut weights and the best one's index."""
+    rng = np.random.default_rng(seed)
+    base = rng.integers(0, 2, (rows, g.n), dtype=np.uint8)
+    pop = base[rng.integers(0, rows, p)]
+    f = np.array([oracle.cut_value(g, x) for x in pop], dtype=np.int64)
+    return pop, f, int(f.argmax())
+
+
+def _load(P, run, pop, f, best):
+    P.set_population(torch.from_numpy(pop).cuda(), torch.from_numpy(pop[best]).cuda(), int(f[best]), 0)
+    run.load(pop, f, pop[best], int(f[best]), 0)
+
+
+def _steps(P, run, gens, generation=None):
+    """`gens` generations of both, every one compared."""
+    for gen in range(gens):
+        stats = generation(1) if generation else P.generation(1)[0]
+        _assert_same_stats(stats[0], run.generation())
+        _assert_same_state(_gpu_state(P), run.get(), f"generation {gen}")
+    assert np.array_equal(P.fitness().cpu().numpy(), run.get()["f"])
+
+
+@pytest.mark.parametrize("s,degree", [(5, 12), (12, 8), (24, 6)])
+@pytest.mark.parametrize("p", [4, 33, 150])
+def test_lanes_of_a_pair_share_its_corrected_flips(oracle, s, degree, p):
+    """Groups of a few elements with many edges, so that up to 32 lanes share a pair, and populations of two rows,
+    where individuals often are the run start that their own search falls through to: the pair's first lane corrects
+    the flip planes that all its lanes have stored."""
+    g = I.random_regular(60, degree, seed=s + p, wmin=-20, wmax=100)
+    ep, ev = _windows(g.n, s)
+    P = gom.Population(g, p, 3, fos=gom.gom_fos_create(g.n, ep, ev), bitsliced=True)
+    k, co = oracle.color(g, ep, ev)
+    run = oracle.Run(g, ep, ev, co, k, p, 3)
+    _load(P, run, *_few_rows(oracle, g, p, 2, 7 * s + p))
+    _steps(P, run, 10)
