@@ -54,7 +54,7 @@ Layout make_layout(int64_t n, int32_t p, int64_t nadj, int64_t m, int64_t total_
     L.eqw = take(sizeof(uint32_t) * 2 * W);
     L.xe = take(n);
     L.st = take(sizeof(GomDevState));
-    L.bar = take(sizeof(GomBarrier));
+    L.bar = take(sizeof(GomBarrier) * kBarriers);
     L.trace = take(sizeof(unsigned long long) * (5 + 2 * static_cast<size_t>(std::max<int32_t>(k, 1))));
     L.stats = take(sizeof(GomDevStats) * kStatsCap);
     L.order = take(sizeof(int32_t) * std::max<int32_t>(k, 1));
@@ -805,10 +805,7 @@ int gom_generation(gom_ctx_t *ctx, int32_t num_generations, int64_t target_fitne
             void *args[] = {&prm, &gens, &target};
             const bool bs = use_bs(ctx), ms = bs && ctx->run_ms_fn && !ctx->prm.learn;
             const int grid = ms ? ctx->ms_grid : bs ? ctx->bs_grid_run : ctx->grid_run;
-            if (ctx->bar_grid != grid) { // the barrier counts in multiples of its grid
-                GOM_CUDA(ctx, cudaMemsetAsync(ctx->prm.bar, 0, sizeof(GomBarrier), ctx->stream));
-                ctx->bar_grid = grid;
-            }
+            prm.bar += ms ? 2 : bs ? 1 : 0; // each path's own counter: it counts in multiples of the path's grid
             GOM_CUDA(ctx, cudaLaunchCooperativeKernel(
                               ms ? ctx->run_ms_fn : bs ? ctx->run_bs_fn : ctx->run_fn, dim3(grid),
                               dim3(ms ? kMsThreads : bs ? ctx->bs_threads : ctx->run_threads), args,

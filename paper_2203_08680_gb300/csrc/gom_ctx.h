@@ -19,7 +19,6 @@ struct gom_ctx {
     size_t mix_smem = 0;          // its dynamic shared memory per block
     int mix_threads = kMixThreads; // its block size (fewer warps for very large elements)
     int run_threads = kMixThreads; // the persistent kernel's
-    int bar_grid = 0;             // the grid whose launches the persistent kernels' barrier counter holds
     const void *run_fn = nullptr; // persistent generation kernel (same instance parameters)
     size_t run_smem = 0;          // its dynamic shared memory (staging or the k group keys)
     int grid_run = 0;             // its grid: co-resident blocks only

@@ -94,10 +94,11 @@ struct GomDevState {
     int32_t pad_;
 };
 
-struct GomBarrier { // grid barrier of the persistent kernel: monotonic arrival count
+struct GomBarrier { // grid barrier of a persistent kernel: monotonic arrival count
     unsigned long long count;
     unsigned long long pad;
 };
+constexpr int kBarriers = 3; // a context's: per-lane, bit-sliced, bit-sliced by element classes
 
 // One instance of a batched launch (gom_batch_*): its blocks, kernel variant
 // and target; gens_run and err are filled after each call.
@@ -228,7 +229,7 @@ struct GomParams {
     uint32_t *eqw;     // [2][W] flags P[i] == x_e of generation g in buffer g mod 2
     uint8_t *xe;       // [n] elitist
     GomDevState *st;
-    GomBarrier *bar;
+    GomBarrier *bar;         // [kBarriers] at init; a launch gets its own path's (batched: its instance's)
     unsigned long long *trace; // [5 + 2k] phase stamps of k_run, or null (off)
     GomDevStats *stats;  // [kStatsCap] ring indexed by generation
     int32_t *order;      // [k] colour visited at position t

@@ -52,3 +52,32 @@ def test_lanes_of_a_pair_share_its_corrected_flips(oracle, s, degree, p):
     run = oracle.Run(g, ep, ev, co, k, p, 3)
     _load(P, run, *_few_rows(oracle, g, p, 2, 7 * s + p))
     _steps(P, run, 10)
+
+
+@pytest.mark.parametrize("bound,side,p", [(0, 40, 96), (10, 30, 70), (64, 30, 300)])
+def test_captured_launch_replayed_between_other_paths(oracle, bound, side, p):
+    """A generation captured on the default path and replayed after, before and between generations of the per-lane
+    path, whose persistent kernel has another grid: each path's barrier counter stays a multiple of its own grid."""
+    g = I.torus2d(side, seed=bound + p)
+    stream = torch.cuda.Stream()
+    fos = gom.gom_build_fos(g, gom.GOM_FOS_BFLT, bound) if bound else None
+    ep, ev = oracle.build_bflt(g, bound) if bound else oracle.build_fos(g)
+    k, co = oracle.color(g, ep, ev)
+    run = oracle.Run(g, ep, ev, co, k, p, 5)
+    with torch.cuda.stream(stream):
+        P = gom.Population(g, p, 5, fos=fos, stream=stream, persistent=True)
+        if not bound:
+            gom.gom_set_option(P.ctx, gom.GOM_OPT_BITSLICED, 1)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        P.generation(1, want_stats=False)
+    gom.gom_set_option(P.ctx, gom.GOM_OPT_BITSLICED, 0)
+    with torch.cuda.stream(stream):
+        for step in "drdrrddr":
+            if step == "r":
+                graph.replay()
+            else:
+                P.generation(1, want_stats=False)
+            run.generation()
+            assert P.generation_counter() == run.get()["g"]  # (an error word here is a barrier that gave up)
+            _assert_same_state(_gpu_state(P), run.get(), step)
