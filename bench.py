@@ -353,6 +353,8 @@ def run_gpu(args, wl, rank, world, local):
     m, k = P.m, P.k
     persistent = bool(gom.gom_get_option(P.ctx, gom.GOM_OPT_PERSISTENT))
     bitsliced = bool(gom.gom_get_option(P.ctx, gom.GOM_OPT_BITSLICED))
+    by_class = bitsliced and bflt > 32  # elements above 32 variables: on bit-planes in the persistent kernel only
+    mix_bits = bitsliced and not by_class
     trials_per_step = p * m
     ex = gom.gom_fos_export(P.fos)
     mix_bytes = mixing_bytes_per_generation(g, ex["elem_ptr"], ex["elem_vars"], p)
@@ -379,13 +381,14 @@ def run_gpu(args, wl, rank, world, local):
     step_ms = [a.elapsed_time(b) for a, b in zip(ev0, ev1)]
     launches_per_step = gom.gom_launches_per_generation(P.ctx) + (0 if persistent else 1)
     if persistent:
-        dom = {"kernel": "k_run_bs (persistent generation kernel, bit-sliced mixing)" if bitsliced else
+        dom = {"kernel": "k_run_multi (persistent generation kernel, bit-sliced mixing by element class)" if by_class else
+               "k_run_bs (persistent generation kernel, bit-sliced mixing)" if bitsliced else
                "k_run (persistent generation kernel)", "bytes_per_launch": gen_bytes,
                "avg_ms": sum(step_ms) / len(step_ms), "launches": args.steps}
     else:
         mix_ms, mix_launches = gom.gom_read_timing(P.ctx)
         gom.gom_set_timing(P.ctx, False)
-        dom = {"kernel": "k_mix_bs" if bitsliced else "k_mix", "bytes_per_launch": mix_bytes / k,
+        dom = {"kernel": "k_mix_bs" if mix_bits else "k_mix", "bytes_per_launch": mix_bytes / k,
                "avg_ms": mix_ms / max(mix_launches, 1), "launches": mix_launches}
     dist_barrier(world)
     total_ms = dist_max(sum(step_ms), world)
@@ -405,7 +408,7 @@ def run_gpu(args, wl, rank, world, local):
         peak, peak_kind = peaks()
         avg = mix_ms / max(mix_launches, 1)
         ach = (mix_bytes / k) / (avg / 1e3) / 1e9
-        mix = {"kernel": "k_mix_bs" if bitsliced else "k_mix", "avg_launch_ms": avg, "launches": mix_launches,
+        mix = {"kernel": "k_mix_bs" if mix_bits else "k_mix", "avg_launch_ms": avg, "launches": mix_launches,
                "algorithmic_bytes_per_launch": mix_bytes / k, "achieved_gbs": ach, "frac": ach / peak}
         del Q
 
@@ -435,7 +438,7 @@ def run_gpu(args, wl, rank, world, local):
                                  "sample": f"{sgens} {swhat} from initialisation ({sel:.1f} s)"}}
     line = finish(args, wl, rank, world, desc, p, m, k, value, total_ms, dom, mix, ttt, e2e,
                   launches_per_step, clk, cpu, persistent)
-    line["config"]["mixing"] = "bit-sliced" if bitsliced else "per-lane"
+    line["config"]["mixing"] = "bit-sliced" if (bitsliced if persistent else mix_bits) else "per-lane"
     return line
 
 

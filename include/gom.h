@@ -83,22 +83,25 @@ extern "C" {
                              warps take more; the default).  Same results either way */
 
 #define GOM_OPT_BITSLICED 4 /* mixing on bit-planes: each lane owns 32 individuals of one element and
-                               takes the partial evaluation, the acceptance and the fitness
-                               bookkeeping as bit-plane arithmetic on them (one logic instruction
-                               works on 32 trials); the donor search stays per individual.
-                               Available for elements of at most 32 variables, |w| <= 255 and
-                               element weight sums (of |w| over their edges) below 2^16; the
-                               default where available except for the smallest problems (groups
-                               of a few hundred population words, or one-word populations of
-                               elements above 16 variables that do not fill the GPU)
-                               (GOM_E_STATE when set to 1 where unavailable).  Same results
-                               either way; the learned filter works on both.  A batched launch
-                               follows the value the caller set for the context, else runs
-                               bit-sliced the instances whose largest group gives each of their
-                               warps four (element, word) pairs or more (only with min_blocks 2).
-                               Weights up to 65,535 with element sums below 2^20 run on bit-planes
-                               by default as well; there the option reads 0 and can only be set
-                               to 0 (the per-lane mixing) */
+                               takes the donor search (from tables made inside the lane), the
+                               partial evaluation, the acceptance and the fitness bookkeeping as
+                               bit-plane arithmetic on them (one logic instruction works on 32
+                               trials).  Available for |w| <= 65,535 and element weight sums (of
+                               |w| over their edges) below 2^20, elements above 32 variables on
+                               the persistent path only (the per-generation graph mixes those per
+                               lane); GOM_E_STATE when set to 1 where unavailable.  The default
+                               where available except for the smallest problems (a colour group
+                               of at most 1,024 population words, or any one-word population,
+                               whose groups are all staged at once; models of elements of 17 to 64
+                               variables with groups of at most 512 words, or with one-word
+                               populations that do not fill the GPU).  Reads the selection in
+                               force.  Same results either way.  The learned filter works on both
+                               for elements of at most 32 variables, |w| <= 255 and sums below
+                               2^16, beyond that per lane.  A batched launch follows the value
+                               the caller set for the context, else runs bit-sliced the instances
+                               whose largest group gives each of their warps four (element, word)
+                               pairs or more (only with min_blocks 2; elements above 32 variables
+                               with at least 4 warps per block) */
 
 #define GOM_OPT_FORCED_IMPROVEMENT 5 /* 1: Forced Improvement (Sec. 4, Alg. 1) after each generation's
                                         mixing, in this library's parallel reading (the paper's

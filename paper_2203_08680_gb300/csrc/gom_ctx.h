@@ -26,8 +26,7 @@ struct gom_ctx {
     bool persistent = false;      // current path: k_run (true) or the per-generation graph
     // the bit-sliced mixing path (gom_bs.cu), where the FOS and weights allow it
     bool bs_can = false;          // available for this context
-    bool bs_ok = false;           // and within the option's limits (8-bit weights): the caller may switch it on, and
-                                  //   the learned filter runs on it
+    bool bs_ok = false;           // and the learned filter runs on it (elements of at most 32 variables, 8-bit weights)
     bool bs_on = false;           // selected (GOM_OPT_BITSLICED)
     int bs_set = -1;              // GOM_OPT_BITSLICED as the caller set it (-1: never set; batched launches
                                   //   then choose by the instance's share of warps)

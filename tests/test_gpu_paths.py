@@ -81,3 +81,33 @@ def test_captured_launch_replayed_between_other_paths(oracle, bound, side, p):
             run.generation()
             assert P.generation_counter() == run.get()["g"]  # (an error word here is a barrier that gave up)
             _assert_same_state(_gpu_state(P), run.get(), step)
+
+
+@pytest.mark.parametrize("bound,side,p,wmax,late", [(0, 60, 96, 255, 1), (0, 60, 96, 3000, 1), (0, 60, 96, 65535, 1),
+                                                    (64, 30, 512, 100, 1), (100, 24, 40, 100, 1), (100, 24, 40, 2000, 1),
+                                                    (0, 8, 16, 3000, 0)])
+def test_mixing_option_reads_and_restores_the_path(oracle, bound, side, p, wmax, late):
+    """GOM_OPT_BITSLICED reads the path in force for every model that runs on bit-planes (`late`: the default), writing
+    back what was read changes nothing, and each value can be set again; the same generations on either path."""
+    g = I.torus2d(side, seed=side + wmax, wmin=-wmax // 2, wmax=wmax)
+    fos = gom.gom_build_fos(g, gom.GOM_FOS_BFLT, bound) if bound else None
+    ep, ev = oracle.build_bflt(g, bound) if bound else oracle.build_fos(g)
+    k, co = oracle.color(g, ep, ev)
+    run = oracle.Run(g, ep, ev, co, k, p, 4)
+    P = gom.Population(g, p, 4, fos=fos)
+    assert gom.gom_get_option(P.ctx, gom.GOM_OPT_BITSLICED) == late
+    gom.gom_set_option(P.ctx, gom.GOM_OPT_BITSLICED, late)
+    for value in (late, 0, 1, 0, 1):
+        gom.gom_set_option(P.ctx, gom.GOM_OPT_BITSLICED, value)
+        assert gom.gom_get_option(P.ctx, gom.GOM_OPT_BITSLICED) == value
+        _steps(P, run, 1)
+
+
+def test_mixing_option_refused_past_every_width():
+    """Weights past 65,535: no bit-planes, 1 is refused and 0 stands."""
+    P = gom.Population(I.torus2d(12, seed=1, wmin=1, wmax=70000), 40, 1)
+    assert gom.gom_get_option(P.ctx, gom.GOM_OPT_BITSLICED) == 0
+    with pytest.raises(gom.GomError) as ei:
+        gom.gom_set_option(P.ctx, gom.GOM_OPT_BITSLICED, 1)
+    assert ei.value.code == -7
+    gom.gom_set_option(P.ctx, gom.GOM_OPT_BITSLICED, 0)
