@@ -353,8 +353,8 @@ __device__ __forceinline__ void bs_large_item(const GomParams &P, const BsItem &
 // P.ms_list[P.ms_ptr[5 c + h] .. P.ms_ptr[5 c + h + 1]), h = 0 large, 1 to 3
 // at most 32, 16 and 8 variables.  Block b of the (virtual) grid takes the
 // large elements b, b + nblk, ...; then, and at once in the other blocks, the
-// tiles claim the small items, the larger classes first (tiles of several
-// warps take them in a static stride).  The first one of either kind is
+// tiles claim the small items, the larger classes first (without P.dyn, and
+// tiles of several warps, take them in a static stride).  The first one of either kind is
 // prepared before open().
 template <int R, int UB, class Open>
 __device__ __forceinline__ bool phase_mix_multi(const GomParams &P, const VGrid &V, const BsMap &M, uint32_t *regions,
@@ -365,7 +365,7 @@ __device__ __forceinline__ bool phase_mix_multi(const GomParams &P, const VGrid 
     const int c0 = cp[0], c1 = cp[1], c2 = cp[2], c3 = cp[3], c4 = cp[4], E = M.E, nl = c1 - c0;
     const int n1 = (c2 - c1 + E - 1) / E, n2 = n1 + (c3 - c2 + E - 1) / E, n3 = n2 + (c4 - c3 + E - 1) / E;
     const int lane = threadIdx.x & 31;
-    const bool dyn = M.nwi == 1;
+    const bool dyn = P.dyn && M.nwi == 1;
     bool first = true;
     BsItem I;
     for (int x = V.blk; x < nl; x += V.nblk) { // block-uniform
