@@ -243,7 +243,8 @@ int ctx_read_stats(gom_ctx *ctx, int32_t num, gom_gen_stats_t *host_stats, int32
     GOM_CUDA(ctx, cudaMemcpyAsync(&st, ctx->prm.st, sizeof(st), cudaMemcpyDeviceToHost, ctx->stream));
     GOM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     if (st.err) return GOM_E_TIMEOUT;
-    const int32_t run = static_cast<int32_t>(st.g - st.call_g0);
+    // (none where an import has set the counter back behind the last call's start)
+    const int32_t run = std::max(static_cast<int32_t>(st.g - st.call_g0), 0);
     if (run_out) *run_out = run;
     if (host_stats) {
         std::memset(host_stats, 0, sizeof(gom_gen_stats_t) * num);

@@ -132,3 +132,25 @@ def test_item_schedule_of_the_bit_sliced_paths(oracle, bound, dynamic):
     assert len(at) == 1
     claims = words[at[0] + rows:at[0] + 2 * rows].ravel()[:k]
     assert claims.all() if dynamic else not claims.any()
+
+
+def test_batch_counters_after_an_import_of_an_earlier_generation(oracle):
+    """A batch made generations 3 to 7, then one instance is set back to generation 0: it has no counters of a call
+    until the next one."""
+    g = I.torus2d(12, seed=3)
+    P = gom.Population(g, 40, 2)
+    pop, _, fe = P.population()
+    xe, _ = P.elite()
+    P.generation(3)
+    ws = torch.empty(gom.gom_batch_workspace_bytes(1) + 256, dtype=torch.uint8, device="cuda")
+    batch = gom.gom_batch_create([P.ctx], None, ws[(-ws.data_ptr()) % 256:])
+    gom.gom_batch_generation(batch, 4)
+    assert [s["generation"] for s in gom.gom_batch_stats(batch, 0, 8)] == [3, 4, 5, 6]
+    P.set_population(pop, xe, fe, 0)
+    assert gom.gom_batch_stats(batch, 0, 8) == []
+    gom.gom_batch_generation(batch, 2)
+    ep, ev = oracle.build_fos(g)
+    k, co = oracle.color(g, ep, ev)
+    want = oracle.Run(g, ep, ev, co, k, 40, 2).run(2)
+    for a, o in zip(gom.gom_batch_stats(batch, 0, 8), want):
+        _assert_same_stats(a, o)
