@@ -353,9 +353,13 @@ __device__ __forceinline__ void bs_large_item(const GomParams &P, const BsItem &
 // P.ms_list[P.ms_ptr[5 c + h] .. P.ms_ptr[5 c + h + 1]), h = 0 large, 1 to 3
 // at most 32, 16 and 8 variables.  Block b of the (virtual) grid takes the
 // large elements b, b + nblk, ...; then, and at once in the other blocks, the
-// tiles claim the small items, the larger classes first (without P.dyn, and
-// tiles of several warps, take them in a static stride).  The first one of either kind is
-// prepared before open().
+// tiles claim the small items, the larger classes first (without P.dyn they
+// take them in a static stride).  Tiles of several warps claim as well: in a
+// static stride the blocks with a large element came late to their share of the
+// small ones (tree of bound 64 on the 50x50 torus, p = 64: 311 us a generation
+// against 208, of bound 100 on a random 6-regular graph of 1,000 vertices, p =
+// 512: 1,302 against 778).  The first one of either kind is prepared before
+// open().
 template <int R, int UB, class Open>
 __device__ __forceinline__ bool phase_mix_multi(const GomParams &P, const VGrid &V, const BsMap &M, uint32_t *regions,
                                                 int t, int c, uint32_t g, Open open, BsLane<FitShared> &L,
@@ -364,8 +368,9 @@ __device__ __forceinline__ bool phase_mix_multi(const GomParams &P, const VGrid 
     const int32_t *cp = P.ms_ptr + 5 * c;
     const int c0 = cp[0], c1 = cp[1], c2 = cp[2], c3 = cp[3], c4 = cp[4], E = M.E, nl = c1 - c0;
     const int n1 = (c2 - c1 + E - 1) / E, n2 = n1 + (c3 - c2 + E - 1) / E, n3 = n2 + (c4 - c3 + E - 1) / E;
-    const int lane = threadIdx.x & 31;
-    const bool dyn = P.dyn && M.nwi == 1;
+    __shared__ int s_claim[kMsThreads / 32]; // per tile of several warps
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, tb = wib / M.nwi;
+    const bool dyn = P.dyn, lead = lane == 0 && wib == tb * M.nwi;
     bool first = true;
     BsItem I;
     for (int x = V.blk; x < nl; x += V.nblk) { // block-uniform
@@ -375,9 +380,15 @@ __device__ __forceinline__ bool phase_mix_multi(const GomParams &P, const VGrid 
         bs_large_item<R, UB>(P, I, g, regions, L, s_f);
     }
     unsigned claim = 0;
-    if (dyn && lane == 0) claim = atomicAdd(&P.work[t], 1u);
+    if (dyn && lead) claim = atomicAdd(&P.work[t], 1u);
     for (int it = M.tile;; it += M.ntiles) {
-        if (dyn) it = (int)__shfl_sync(kFull, claim, 0);
+        if (dyn && M.nwi == 1) {
+            it = (int)__shfl_sync(kFull, claim, 0);
+        } else if (dyn) { // (read by all before the next is written: an item's first part or the group's end waits)
+            if (lead) s_claim[tb] = (int)claim;
+            tile_sync(M);
+            it = s_claim[tb];
+        }
         int cls = 0, k0 = 0, k1 = 0;
         if (it < n1) {
             cls = 32;
@@ -401,7 +412,7 @@ __device__ __forceinline__ bool phase_mix_multi(const GomParams &P, const VGrid 
         if (first && !open()) return false;
         first = false;
         if (!cls) return true;
-        if (dyn && lane == 0) claim = atomicAdd(&P.work[t], 1u);
+        if (dyn && lead) claim = atomicAdd(&P.work[t], 1u);
         if (cls == 8)
             bs_item<8, R, UB, false>(P, M, I, g, L, s_f, nullptr);
         else if (cls == 16)

@@ -113,17 +113,18 @@ def test_mixing_option_refused_past_every_width():
     gom.gom_set_option(P.ctx, gom.GOM_OPT_BITSLICED, 0)
 
 
-@pytest.mark.parametrize("bound", [0, 24, 100])
+@pytest.mark.parametrize("bound,p", [(0, 32), (24, 32), (100, 32), (24, 512), (100, 300)])
 @pytest.mark.parametrize("dynamic", [True, False])
-def test_item_schedule_of_the_bit_sliced_paths(oracle, bound, dynamic):
-    """GOM_OPT_DYNAMIC on one-warp tiles (a one-word population): claims leave their marks in the groups' counters,
-    which stand behind the group order in the workspace, the static stride leaves them zero; equal generations."""
+def test_item_schedule_of_the_bit_sliced_paths(oracle, bound, p, dynamic):
+    """GOM_OPT_DYNAMIC on one-warp tiles (a one-word population) and, by element class, on tiles of several warps:
+    claims leave their marks in the groups' counters, which stand behind the group order in the workspace, the static
+    stride leaves them zero; equal generations."""
     g = I.torus2d(24, seed=bound)
     fos = gom.gom_build_fos(g, gom.GOM_FOS_BFLT, bound) if bound else None
     ep, ev = oracle.build_bflt(g, bound) if bound else oracle.build_fos(g)
     k, co = oracle.color(g, ep, ev)
-    run = oracle.Run(g, ep, ev, co, k, 32, 6)
-    P = gom.Population(g, 32, 6, fos=fos, persistent=True, dynamic=dynamic, bitsliced=True)
+    run = oracle.Run(g, ep, ev, co, k, p, 6)
+    P = gom.Population(g, p, 6, fos=fos, persistent=True, dynamic=dynamic, bitsliced=True)
     _steps(P, run, 3)
     raw = P.workspace.cpu().numpy()[(-P.workspace.data_ptr()) % 256:]
     words = raw[:len(raw) // 256 * 256].view(np.int32).reshape(-1, 64)
