@@ -90,14 +90,16 @@ extern "C" {
                                |w| over their edges) below 2^20, elements above 32 variables on
                                the persistent path only (the per-generation graph mixes those per
                                lane); GOM_E_STATE when set to 1 where unavailable.  The default
-                               where available except for the smallest problems (a colour group
-                               of at most 1,024 population words, or any one-word population,
-                               whose groups are all staged at once; models of elements of 17 to 64
-                               variables with groups of at most 512 words, or with one-word
-                               populations that do not fill the GPU).  Reads the selection in
-                               force.  Same results either way.  The learned filter works on both
-                               for elements of at most 32 variables, |w| <= 255 and sums below
-                               2^16, beyond that per lane.  A batched launch follows the value
+                               where available and measured as the faster: not for small problems
+                               whose groups are all staged at once, nor for small populations or
+                               groups of models with elements of 17 to 64 variables.  Reads the
+                               selection, the default or as set.  (Where it was not set, linkage
+                               trees at small populations mix per lane on the per-generation
+                               graph all the same, and with the learned filter on bit-planes mix
+                               the large groups only.)  Same results either way.  The learned
+                               filter works on both for elements of at most 32 variables, |w| <=
+                               255 and sums below 2^16, beyond that per lane.
+                               A batched launch follows the value
                                the caller set for the context, else runs bit-sliced the instances
                                whose largest group gives each of their warps four (element, word)
                                pairs or more (only with min_blocks 2; elements above 32 variables

@@ -153,7 +153,7 @@ int build_graph(gom_ctx *ctx, bool timed, cudaGraph_t *out_graph, cudaGraphExec_
         }
         ts[t] = t;
         void *args2[] = {&prm, &ts[t]};
-        if (use_bs(ctx) && ctx->mix_bs_fn)
+        if (use_bs_one(ctx))
             e = add_kernel(g, &node, last, ctx->mix_bs_fn, ctx->bs_grid_mix, ctx->bs_threads, ctx->bs_smem, args2);
         else
             e = add_kernel(g, &node, last, ctx->mix_fn, ctx->grid_mix, ctx->mix_threads, ctx->mix_smem, args2);
@@ -218,7 +218,7 @@ int accumulate_timing(gom_ctx *ctx)
 int rebuild_graphs(gom_ctx *ctx)
 {
     // the learned filter's counting unit and list mode follow the mixing path in use
-    const bool bs = use_bs(ctx) && ctx->mix_bs_fn;
+    const bool bs = use_bs_one(ctx);
     ctx->prm.flt.compact = bs ? 1 : 0;
     ctx->prm.flt.items_per_elem =
         bs || !ctx->prm.split ? 1 : (ctx->prm.Wv + ctx->wpi - 1) / std::max(ctx->wpi, 1);
@@ -421,10 +421,10 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
     int dev = 0;
     GOM_CUDA(c, cudaGetDevice(&dev));
     GOM_CUDA(c, cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev));
-    // Work split for the whole grid (~24 resident warps per SM).
+    // Work split for the whole grid.
     const int wv = (pop + 31) / 32;
     int wpi = 1, split = 0;
-    item_split(c->W, pop, max_group, static_cast<int64_t>(c->sms) * 24, variant, &wpi, &split);
+    item_split(c->W, pop, max_group, static_cast<int64_t>(c->sms) * kLaneWarps, variant, &wpi, &split);
     // Block mode (the 128-bit instances, 4 or more word groups per element):
     // the warps of a block stage each element once, together, and share its
     // word groups -- rather than every (element, word group) item staging the
@@ -551,6 +551,26 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
         GOM_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_f, gom_fi_kernel(2, c->fi_r), 256, 0));
         c->fi_grid = std::max(1, c->sms * std::max(occ_f, 1));
     }
+    int ms_ub = 0; // weight bits of the by-class instances, 0 where there are none
+    if (max_w < 256 && tabs.max_abs_w < (int64_t(1) << 16))
+        ms_ub = 8;
+    else if (max_w < 65536 && tabs.max_abs_w < (int64_t(1) << 20))
+        ms_ub = 16;
+    MixShape shape{wv, max_group, tabs.max_s, tabs.max_edges, ms_ub, c->k, 0, false, c->prm.stage_all != 0,
+                   static_cast<int64_t>(c->sms) * kLaneWarps};
+    {
+        int64_t small = 0;
+        for (int32_t col = 0; col < c->k; ++col) {
+            int32_t most = 0;
+            for (int64_t q = fos->cptr[col]; q < fos->cptr[col + 1]; ++q) {
+                const int32_t s = tabs.hdr[8 * q + 3] & 0xFF;
+                most = std::max(most, s);
+                small += s <= 8;
+            }
+            shape.headed += most > 16;
+        }
+        shape.mixed = tabs.max_s > 8 && 2 * small >= c->m;
+    }
     {
         int R = 0, UB = 0;
         if (coop && variant == kVarNarrow && bs_planes(max_w, tabs.max_abs_w, &R, &UB)) {
@@ -563,8 +583,6 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
             const void *rf = gom_run_bs_kernel(S, R, UB, false), *mf = gom_mix_bs_kernel(S, R, UB, false);
             const void *rfl = gom_run_bs_kernel(S, R, UB, true), *mfl = gom_mix_bs_kernel(S, R, UB, true);
             if (wpb >= 1 && smem <= static_cast<size_t>(kSmemBudget)) {
-                const int E = 32 / wv;
-                const int64_t items = (max_group + E - 1) / E;
                 for (const void *fn : {rf, mf, rfl, mfl})
                     if (fn) GOM_CUDA(c, raise_smem_limit(fn, smem));
                 int occ_r = 0, occ_m = 0, occ_rl = 0, occ_ml = 0;
@@ -597,8 +615,9 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
                         std::min<int64_t>(static_cast<int64_t>(c->sms) * occ_m, need), kMaxMixBlocks));
                     c->prm.bs_S = S;
                     c->prm.bs_words = static_cast<int32_t>(ww);
-                    c->bs_on = bs_pays(wv, max_group, tabs.max_s, c->prm.stage_all != 0,
-                                       static_cast<int64_t>(c->sms) * occ_r * wpb);
+                    c->bs_on = bs_pays(shape);
+                    c->bs_one = bs_one_class_pays(shape);
+                    c->bs_learn = bs_learn_pays(c->W, max_group, c->sms);
                 }
             }
         }
@@ -609,11 +628,6 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
     // one class with more resident warps is the faster: 237 against 256 us a
     // generation for the 200x200 torus' tree of bound 10, p = 300)
     std::vector<int32_t> ms_list, ms_ptr;
-    int ms_ub = 0;
-    if (max_w < 256 && tabs.max_abs_w < (int64_t(1) << 16))
-        ms_ub = 8;
-    else if (max_w < 65536 && tabs.max_abs_w < (int64_t(1) << 20))
-        ms_ub = 16;
     if (coop && ms_ub && tabs.max_s > 16 && (c->bs_can || tabs.max_s > 32)) {
         const auto cls = [&](int64_t q) {
             const int s = tabs.hdr[8 * q + 3] & 0xFF;
@@ -669,7 +683,7 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
             c->prm.bs_words = gom_bs_warp_words(c->prm.bs_S);
             if (!c->bs_can) {
                 c->bs_can = true;
-                c->bs_on = bs_pays(wv, max_group, tabs.max_s, c->prm.stage_all != 0, warps);
+                c->bs_on = bs_pays(shape);
             }
         }
     }
@@ -804,7 +818,7 @@ int gom_generation(gom_ctx_t *ctx, int32_t num_generations, int64_t target_fitne
             int gens = chunk;
             int64_t target = target_fitness;
             void *args[] = {&prm, &gens, &target};
-            const bool bs = use_bs(ctx), ms = bs && ctx->run_ms_fn && !ctx->prm.learn;
+            const bool ms = use_ms(ctx), bs = !ms && use_bs_run(ctx);
             const int grid = ms ? ctx->ms_grid : bs ? ctx->bs_grid_run : ctx->grid_run;
             prm.bar += ms ? 2 : bs ? 1 : 0; // each path's own counter: it counts in multiples of the path's grid
             GOM_CUDA(ctx, cudaLaunchCooperativeKernel(
@@ -966,10 +980,10 @@ int gom_set_option(gom_ctx_t *ctx, int32_t option, int64_t value)
     if (option == GOM_OPT_BITSLICED) {
         if (value != 0 && value != 1) return GOM_E_ARG;
         if (value && !ctx->bs_can) return GOM_E_STATE;
+        const bool one = use_bs_one(ctx);
         ctx->bs_set = static_cast<int>(value); // batched launches follow it too
-        if (ctx->bs_on == (value != 0)) return GOM_OK;
         ctx->bs_on = value != 0;
-        return rebuild_graphs(ctx); // the graphs hold the mixing kernel
+        return use_bs_one(ctx) == one ? GOM_OK : rebuild_graphs(ctx); // the graphs hold the mixing kernel
     }
     if (option == GOM_OPT_FORCED_IMPROVEMENT) {
         if (value != 0 && value != 1) return GOM_E_ARG;

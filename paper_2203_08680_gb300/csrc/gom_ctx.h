@@ -28,6 +28,8 @@ struct gom_ctx {
     bool bs_can = false;          // available for this context
     bool bs_ok = false;           // and the learned filter runs on it (elements of at most 32 variables, 8-bit weights)
     bool bs_on = false;           // selected (GOM_OPT_BITSLICED)
+    bool bs_one = true;           // the one-class kernels pay (bs_one_class_pays)
+    bool bs_learn = false;        // the learned filter's do (bs_learn_pays)
     int bs_set = -1;              // GOM_OPT_BITSLICED as the caller set it (-1: never set; batched launches
                                   //   then choose by the instance's share of warps)
     const void *run_bs_fn = nullptr, *mix_bs_fn = nullptr; // the instances for the learned filter's mode
@@ -73,9 +75,18 @@ struct gom_ctx {
 };
 
 
-// The bit-sliced path runs the context's generations: selected, and with the
-// learned filter on within its instances' limits.
-inline bool use_bs(const gom_ctx *ctx) { return ctx->bs_on && (ctx->bs_ok || !ctx->prm.learn); }
+// The bit-sliced path runs the context's generations: by element class where
+// the model has that (persistent, without the learned filter), else in one
+// class.  The per-generation graph and the learned filter have their own
+// defaults, where the caller has not set the option (use_bs_one: the graph's
+// kernels, and with the filter the persistent one too).
+inline bool use_ms(const gom_ctx *ctx) { return ctx->bs_on && ctx->run_ms_fn && !ctx->prm.learn; }
+inline bool use_bs_one(const gom_ctx *ctx)
+{
+    const bool learn = ctx->prm.learn != 0, dflt = learn ? ctx->bs_learn : ctx->bs_on && ctx->bs_one;
+    return ctx->run_bs_fn && (ctx->bs_ok || !learn) && (ctx->bs_set >= 0 ? ctx->bs_set == 1 : dflt);
+}
+inline bool use_bs_run(const gom_ctx *ctx) { return ctx->prm.learn ? use_bs_one(ctx) : ctx->bs_on && ctx->run_bs_fn; }
 
 // Weight and sum widths of the bit-sliced instances for |w| <= max_w and
 // element sums of |w| <= max_abs_w; false where there is none.
@@ -170,23 +181,79 @@ inline void bs_split(int wv, int64_t max_group, int64_t max_edges, int64_t warps
     }
 }
 
-// Whether the bit-sliced path is the faster one where both are available, for
-// a largest colour group of `max_group` elements of wv words, the largest of
-// max_s variables, on `warps` resident bit-sliced warps.  Microseconds per
-// generation, per-lane / bit-sliced (late generations): 2D torus 100 p = 256
-// 111 / 70, p = 64 56 / 51; 3D torus 50 p = 128 1046 / 312; random 12-regular
-// 60,000 p = 512 5459 / 3372; 2D torus 300 p = 1,024 also 6 times faster.  The
-// per-lane path wins where it stages every group at once and a group is no
-// more than a few hundred words (2D torus 10 p = 16 50 / 58, 50 p = 64 58 / 62),
-// and for models with elements of 17 to 64 variables where the population has
-// one word and does not fill the warps (linkage tree of bound 30, 100x100 torus,
-// p = 32: 142 / 239) or a group has a few hundred words (20x20 torus, p = 100,
-// bound 30 147 / 193, bound 64 208 / 304; p = 512 253 / 194 and 416 / 315).
-inline bool bs_pays(int wv, int64_t max_group, int64_t max_s, bool stage_all, int64_t warps)
+// What the choice between the two mixing paths goes by: population words of an
+// element, elements of the largest colour group, variables and edges of the
+// largest element, weight bits of the bit-plane instances, the colour groups
+// and those of them that hold an element above 16 variables, whether half of
+// the elements have at most 8 variables and the largest more (linkage trees),
+// whether the per-lane path stages all groups at once, and its resident warps.
+struct MixShape {
+    int64_t wv, max_group, max_s, max_edges;
+    int ub;
+    int64_t groups, headed;
+    bool mixed, stage_all;
+    int64_t lane_warps;
+};
+
+// Whether the bit-sliced path is the faster one where both are available: its
+// persistent kernels, over tori, random regular graphs of degree 3 to 12 and
+// their linkage trees of bounds 2 to 128, p = 2 to 1,024 (figures: microseconds
+// per generation, per lane / bit-sliced).
+// - Up to 16 variables it is, from small groups on (2D torus 100, p = 256 111 /
+//   70; 3D torus 50, p = 128 1046 / 312; random 12-regular 60,000, p = 512
+//   5459 / 3372), unless the per-lane path has staged every group: then at one
+//   word (2D torus 75, p = 32 73 / 75; singletons 23 / 30), in groups of at most
+//   1,024 words (2D torus 10, p = 32 45 / 59), and up to six words where the
+//   groups have few edges (singletons of the 50x50 torus, p = 64 15 / 19, 4 edges
+//   times 2,500 words; of a random 10-regular graph of 3,000, p = 128 48 / 43).
+//   Linkage trees in the class of 16 (bounds 14 to 16): up to four words, in all
+//   but small groups five, only from one and a half waves of per-lane warps on
+//   (bound 14, random 6-regular 4,000, p = 128 170 / 232; 75x75 torus, p = 160
+//   153 / 171; 100x100 torus, p = 128 255 / 182).
+// - Above 64 variables it is (a block takes a large element; tree of bound 70,
+//   50x50 torus, p = 64 296 / 213; random 5-regular 40,000, p = 64 1408 / 1120).
+// - From 17 to 64 variables its tables are at their widest, and one block of
+//   eight warps fills an SM.  Up to four words the per-lane path splits elements
+//   by word and wins while those items fit one wave of its warps (tree of bound
+//   24, 50x50 torus, p = 64 121 / 140; 150x150, p = 64 236 / 169; at three and four
+//   words three quarters of a wave: bound 30, 75x75, p = 128 180 / 171), and
+//   where most groups hold an element above 16 variables (bound 40, random
+//   5-regular 40,000, p = 64 618 / 749).  Above four words its items take four
+//   words each and bit-planes win (bound 30, 50x50, p = 256 211 / 168), but not in groups
+//   of at most 512 words (bound 30, random 3-regular 300, p = 256 161 / 173), nor
+//   with 16-bit weights, whose adders are twice as long, up to 32 variables and
+//   12 words in one wave (bound 24, 50x50, p = 160 283 / 304).
+inline bool bs_pays(const MixShape &m)
 {
-    if (stage_all && (wv == 1 || max_group * wv <= 1024)) return false;
-    if (max_s <= 16 || max_s > 64) return true;
-    return !(wv == 1 && max_group <= 4 * warps) && max_group * wv > 512;
+    const int64_t words = m.max_group * m.wv;
+    if (m.stage_all && (m.wv == 1 || words <= 1024 || (m.wv <= 6 && words * m.max_edges <= 19000))) return false;
+    if (m.max_s <= 16 && m.max_s > 13 && m.mixed && (m.wv <= 4 || (m.wv == 5 && 2 * words > m.lane_warps)))
+        return 2 * words > 3 * m.lane_warps;
+    if (m.max_s <= 16 || m.max_s > 64) return true;
+    if (m.wv <= 4) return words > m.lane_warps * (m.wv <= 2 ? 4 : 3) / 4 && 5 * m.headed <= 3 * m.groups;
+    return words > 512 && !(m.ub > 8 && m.max_s <= 32 && m.wv <= 12 && words <= m.lane_warps);
+}
+
+// The same for the per-generation graph's kernels, which take all elements in
+// the largest one's class.  In linkage trees, where that class is wide and most
+// elements are small, per lane is the faster up to five words for 9 to 16
+// variables (bound 12, 150x150 torus, p = 32 153 / 190; bound 14, 75x75, p = 160
+// 177 / 211) and up to 15 words above (bound 30, 50x50, p = 64 158 / 275, p = 256
+// 249 / 293, p = 512 as fast).
+inline bool bs_one_class_pays(const MixShape &m)
+{
+    if (!m.mixed) return true;
+    return m.max_s <= 16 ? m.wv > 5 || 2 * m.max_group * m.wv > 3 * m.lane_warps : m.wv > 15;
+}
+
+// The same for the learned filter's kernels, whose bookkeeping takes one lane
+// per pair and whole warps: rows of at most 16 words, and items for at least a
+// quarter of 20 warps per SM (random 10-regular 3,000, p = 32 1,634 / 4,824; random
+// 16-regular 20,000, p = 1,024 19.3 / 29.6 ms).
+inline bool bs_learn_pays(int64_t W, int64_t max_group, int64_t sms)
+{
+    const int64_t E = 32 / W;
+    return W <= 16 && 4 * ((max_group + E - 1) / E) >= 20 * sms;
 }
 
 // Raises a kernel's dynamic shared memory limit to at least `bytes`, never

@@ -180,6 +180,7 @@ struct GomFI {
 };
 
 constexpr int kStatsCap = 1024;    // per-generation counters kept on the device
+constexpr int kLaneWarps = 24;     // resident warps per SM of the per-lane mixing kernels, about
 constexpr int kMixThreads = 256;   // mixing kernel block size (8 warps)
 constexpr int kRunThreads = 768;   // largest block of the per-lane persistent kernel (as many registers as three of 256)
 constexpr int kBsThreads = 128;    // bit-sliced kernels' block size (4 warps)

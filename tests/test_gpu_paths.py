@@ -155,3 +155,15 @@ def test_batch_counters_after_an_import_of_an_earlier_generation(oracle):
     want = oracle.Run(g, ep, ev, co, k, 40, 2).run(2)
     for a, o in zip(gom.gom_batch_stats(batch, 0, 8), want):
         _assert_same_stats(a, o)
+
+
+@pytest.mark.parametrize("bound,kind,side,p,late", [
+    (0, 0, 100, 64, 1), (0, 0, 100, 32, 0), (0, 0, 10, 16, 0), (0, 0, 50, 128, 1), (0, 1, 50, 64, 0), (0, 1, 33, 128, 0),
+    (14, 0, 50, 64, 0), (10, 0, 50, 300, 1), (24, 0, 50, 64, 0), (24, 0, 50, 128, 0), (48, 0, 33, 128, 0),
+    (48, 0, 33, 256, 1), (24, 0, 100, 128, 1), (64, 0, 150, 64, 1), (100, 0, 22, 64, 1), (128, 0, 30, 1024, 1)])
+def test_default_mixing_path(bound, kind, side, p, late):
+    """The default on either side of the lines where one path was measured as the faster."""
+    g = I.torus2d(side, seed=1)
+    fos = gom.gom_build_fos(g, gom.GOM_FOS_BFLT, bound) if bound else None
+    P = gom.Population(g, p, 1, kind=gom.GOM_FOS_SINGLETON if kind else gom.GOM_FOS_NEIGHBOURHOOD, fos=fos)
+    assert gom.gom_get_option(P.ctx, gom.GOM_OPT_BITSLICED) == late
