@@ -618,6 +618,7 @@ int gom_init_population(const gom_graph_t *g, const gom_fos_t *fos, int32_t pop,
                     c->bs_on = bs_pays(shape);
                     c->bs_one = bs_one_class_pays(shape);
                     c->bs_learn = bs_learn_pays(c->W, max_group, c->sms);
+                    c->bs_fi = wv > 1 || max_group > 1024;
                 }
             }
         }

@@ -163,13 +163,22 @@ __device__ __forceinline__ void planes_add(uint32_t (&x)[32], long long *f)
 
 // Adds the lane's accumulated deltas into the block's fitness accumulators
 // s_f[32 w + b] (one shared atomic per individual with a non-zero sum) and
-// clears them.
+// clears them.  In Forced Improvement few individuals have any: bit by bit, and
+// nothing for a lane without (a launch per group: 75x75 torus, p = 32, 15
+// groups, 185 us a generation with a transpose in every lane, 154 so).
 __device__ __forceinline__ void bs_flush(BsLane<FitRegs> &L, long long *s_f)
 {
-    uint32_t x[32];
+    uint32_t any = 0;
 #pragma unroll
-    for (int t = 0; t < 32; ++t) x[t] = t < kFitPlanes ? L.fit.v[t < kFitPlanes ? t : 0] : 0u;
-    planes_add(x, s_f + 32 * L.w);
+    for (int t = 0; t < kFitPlanes; ++t) any |= L.fit.v[t];
+    while (any) {
+        const int b = __ffs(any) - 1;
+        any &= any - 1;
+        unsigned v = 0;
+#pragma unroll
+        for (int t = 0; t < kFitPlanes; ++t) v |= ((L.fit.v[t] >> b) & 1u) << t;
+        atomicAdd(reinterpret_cast<unsigned long long *>(&s_f[32 * L.w + b]), (unsigned long long)v);
+    }
 #pragma unroll
     for (int t = 0; t < kFitPlanes; ++t) L.fit.v[t] = 0;
     L.since_flush = 0;

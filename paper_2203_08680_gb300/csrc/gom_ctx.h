@@ -30,6 +30,10 @@ struct gom_ctx {
     bool bs_on = false;           // selected (GOM_OPT_BITSLICED)
     bool bs_one = true;           // the one-class kernels pay (bs_one_class_pays)
     bool bs_learn = false;        // the learned filter's do (bs_learn_pays)
+    bool bs_fi = true;            // the persistent one does with Forced Improvement on: not with one-word populations
+                                  //   in groups of at most 1,024, whose FI steps are most of the time and want the
+                                  //   per-lane kernel's grid (random 6-regular 4,000, p = 32, generation 40: 672 us
+                                  //   per lane, 773; 2D torus 300, p = 32 197, 94)
     int bs_set = -1;              // GOM_OPT_BITSLICED as the caller set it (-1: never set; batched launches
                                   //   then choose by the instance's share of warps)
     const void *run_bs_fn = nullptr, *mix_bs_fn = nullptr; // the instances for the learned filter's mode
@@ -86,7 +90,11 @@ inline bool use_bs_one(const gom_ctx *ctx)
     const bool learn = ctx->prm.learn != 0, dflt = learn ? ctx->bs_learn : ctx->bs_on && ctx->bs_one;
     return ctx->run_bs_fn && (ctx->bs_ok || !learn) && (ctx->bs_set >= 0 ? ctx->bs_set == 1 : dflt);
 }
-inline bool use_bs_run(const gom_ctx *ctx) { return ctx->prm.learn ? use_bs_one(ctx) : ctx->bs_on && ctx->run_bs_fn; }
+inline bool use_bs_run(const gom_ctx *ctx)
+{
+    if (ctx->prm.learn) return use_bs_one(ctx);
+    return ctx->bs_on && ctx->run_bs_fn && (!ctx->prm.fi.on || ctx->bs_fi || ctx->bs_set == 1);
+}
 
 // Weight and sum widths of the bit-sliced instances for |w| <= max_w and
 // element sums of |w| <= max_abs_w; false where there is none.

@@ -167,3 +167,26 @@ def test_default_mixing_path(bound, kind, side, p, late):
     fos = gom.gom_build_fos(g, gom.GOM_FOS_BFLT, bound) if bound else None
     P = gom.Population(g, p, 1, kind=gom.GOM_FOS_SINGLETON if kind else gom.GOM_FOS_NEIGHBOURHOOD, fos=fos)
     assert gom.gom_get_option(P.ctx, gom.GOM_OPT_BITSLICED) == late
+
+
+@pytest.mark.parametrize("bound,side,p", [(0, 30, 32), (0, 40, 96), (10, 20, 200), (24, 30, 300), (64, 20, 200), (100, 16, 40)])
+@pytest.mark.parametrize("persistent", [True, False])
+def test_forced_improvement_on_the_default_path(oracle, bound, side, p, persistent):
+    """Forced Improvement where the mixing option was never set: per lane, bit-sliced, and by element class."""
+    from test_gpu_fi import KEYS, _same, _state
+    g = I.torus2d(side, seed=bound + p)
+    fos = gom.gom_build_fos(g, gom.GOM_FOS_BFLT, bound) if bound else None
+    ep, ev = oracle.build_bflt(g, bound) if bound else oracle.build_fos(g)
+    k, co = oracle.color(g, ep, ev)
+    run = oracle.Run(g, ep, ev, co, k, p, 8)
+    run.set_fi(True, 2)
+    P = gom.Population(g, p, 8, fos=fos, persistent=persistent, forced_improvement=True, fi_nis=2)
+    seen = 0
+    for gen in range(8):
+        want = run.generation()
+        got = P.generation(1)[0][0]
+        seen += want["fi_individuals"]
+        for gk, ok in KEYS:
+            assert got[gk] == want[ok], (gen, gk, got, want)
+        _same(_state(P), run.get(), f"gen {gen}")
+    assert seen > 0
