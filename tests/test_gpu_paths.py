@@ -172,7 +172,8 @@ def test_default_mixing_path(bound, kind, side, p, late):
 @pytest.mark.parametrize("bound,side,p", [(0, 30, 32), (0, 40, 96), (10, 20, 200), (24, 30, 300), (64, 20, 200), (100, 16, 40)])
 @pytest.mark.parametrize("persistent", [True, False])
 def test_forced_improvement_on_the_default_path(oracle, bound, side, p, persistent):
-    """Forced Improvement where the mixing option was never set: per lane, bit-sliced, and by element class."""
+    """Forced Improvement where the mixing option was never set: per lane, bit-sliced, and by element class, until
+    individuals have entered it (in the oracle's runs too)."""
     from test_gpu_fi import KEYS, _same, _state
     g = I.torus2d(side, seed=bound + p)
     fos = gom.gom_build_fos(g, gom.GOM_FOS_BFLT, bound) if bound else None
@@ -182,7 +183,7 @@ def test_forced_improvement_on_the_default_path(oracle, bound, side, p, persiste
     run.set_fi(True, 2)
     P = gom.Population(g, p, 8, fos=fos, persistent=persistent, forced_improvement=True, fi_nis=2)
     seen = 0
-    for gen in range(8):
+    for gen in range(18):
         want = run.generation()
         got = P.generation(1)[0][0]
         seen += want["fi_individuals"]
