@@ -745,7 +745,7 @@ struct RunShared {
     int *order;                 // [kStageAllMaxK] stage-all group order
 };
 
-template <int WPI, typename MaskT, typename AccT, bool LEARN>
+template <int WPI, typename MaskT, typename AccT, bool LEARN, bool FI = true>
 __device__ void run_generations(const GomParams &P, const VGrid V, GomBarrier *bar, int G, int64_t target,
                                 const RunShared &S)
 {
@@ -804,7 +804,7 @@ __device__ void run_generations(const GomParams &P, const VGrid V, GomBarrier *b
         count_flush(S.cnt, n_dl, n_acc, n_imp);
         acc_flush(P, S.f, S.cnt);
         if (!grid_barrier(&bar->count, &P.st->err, nblk, bnext, kBarrierNs)) return;
-        if (P.fi.on && !fi_generation<16>(P, V, &bar->count, nblk, bnext, e, all ? S.order : P.order, S.f, S.cnt))
+        if (FI && P.fi.on && !fi_generation<16>(P, V, &bar->count, nblk, bnext, e, all ? S.order : P.order, S.f, S.cnt))
             return;
         if (tr) P.trace[4 + 2 * P.k] = global_ns();
         ++g;
