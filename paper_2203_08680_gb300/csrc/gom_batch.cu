@@ -197,6 +197,7 @@ int batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config_t *
     int32_t f_words = 0;
     int64_t smem = 0;
     int total = 0, level = 0;
+    std::vector<int32_t> nb;
     for (;; ++level) {
         int maxW = 1, maxk = 1;
         int64_t max_warp_words = 8;
@@ -230,8 +231,20 @@ int batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config_t *
             GOM_CUDA(nullptr, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, static_cast<size_t>(smem)));
             total = conf.max_blocks > 0 ? std::min(sms * occ, conf.max_blocks) : sms * occ;
         }
-        if (total >= num) break;
-        if (level == 2) return GOM_E_LIMIT;
+        if (total >= num) {
+            // shared out: where that leaves every instance per lane, sized and shared out
+            // again without the bit-sliced phases' room (60 trees of bound 128 over
+            // 14x14 tori, p = 32: 152 blocks of eight warps with the element classes'
+            // regions, 304 without; 343 -> 292 us a generation)
+            nb = allocate_blocks(cs, total, conf, level, weights);
+            bool any = false;
+            for (int32_t b = 0; b < num; ++b)
+                any |= batch_bits(cs[b], conf, level, int64_t(nb[b]) * conf.warps_per_block);
+            if (any || level == 2 || conf.min_blocks != 2) break;
+            level = 1;
+        } else if (level == 2) {
+            return GOM_E_LIMIT;
+        }
     }
 
     std::unique_ptr<gom_batch> bt(new (std::nothrow) gom_batch());
@@ -250,7 +263,6 @@ int batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config_t *
     B->d_inst = reinterpret_cast<GomBatchInst *>(base + L.inst);
     B->d_bars = reinterpret_cast<GomBarrier *>(base + L.bars);
 
-    const std::vector<int32_t> nb = allocate_blocks(cs, total, conf, level, weights);
     B->params.resize(num);
     B->inst.resize(num);
     int32_t blk = 0;

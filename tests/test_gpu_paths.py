@@ -191,3 +191,26 @@ def test_forced_improvement_on_the_default_path(oracle, bound, side, p, persiste
             assert got[gk] == want[ok], (gen, gk, got, want)
         _same(_state(P), run.get(), f"gen {gen}")
     assert seen > 0
+
+
+def test_batch_of_per_lane_instances_takes_no_room_for_bit_planes(oracle):
+    """60 small linkage trees, whose shares of the warps leave them per lane: the launch has more than the one block
+    of eight warps per SM that the regions of the element classes would leave, and the trees' generations are their
+    own; with few instances the same trees are on bit-planes."""
+    ws = torch.empty(gom.gom_batch_workspace_bytes(60) + 256, dtype=torch.uint8, device="cuda")
+    ws = ws[(-ws.data_ptr()) % 256:]
+    graphs = [I.torus2d(14, seed=i) for i in range(60)]
+    pops = [gom.Population(g, 32, i, fos=gom.gom_build_fos(g, gom.GOM_FOS_BFLT, 128)) for i, g in enumerate(graphs)]
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for part, config in ((pops, (8, 2, 0, 300)), (pops[:2], (8, 2, 2, 300))):
+        batch = gom.gom_batch_create([P.ctx for P in part], config, ws)
+        grid = gom.gom_batch_layout(batch, 0)[2]
+        assert grid > sms if len(part) == 60 else grid == 2
+        gom.gom_batch_generation(batch, 3)
+        del batch
+    for i in (0, 1, 59):
+        ep, ev = oracle.build_bflt(graphs[i], 128)
+        k, co = oracle.color(graphs[i], ep, ev)
+        run = oracle.Run(graphs[i], ep, ev, co, k, 32, i)
+        run.run(6 if i < 2 else 3)
+        _assert_same_state(_gpu_state(pops[i]), run.get(), f"instance {i}")
