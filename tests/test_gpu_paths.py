@@ -214,3 +214,47 @@ def test_batch_of_per_lane_instances_takes_no_room_for_bit_planes(oracle):
         run = oracle.Run(graphs[i], ep, ev, co, k, 32, i)
         run.run(6 if i < 2 else 3)
         _assert_same_state(_gpu_state(pops[i]), run.get(), f"instance {i}")
+
+
+def _batch_of(P, config):
+    ws = torch.empty(gom.gom_batch_workspace_bytes(1) + 256, dtype=torch.uint8, device="cuda")
+    batch = gom.gom_batch_create([P.ctx], config, ws[(-ws.data_ptr()) % 256:])
+
+    def generation(num):
+        gom.gom_batch_generation(batch, num)
+        return gom.gom_batch_stats(batch, 0, num)
+    return generation
+
+
+@pytest.mark.parametrize("degree,wmax", [(4, 1000), (6, 1000), (7, 500), (9, 700), (12, 300), (15, 280),
+                                         (4, 65535), (6, 20000), (7, 20000), (9, 10000), (12, 6000), (15, 4000),
+                                         (20, 2000)])
+@pytest.mark.parametrize("path", ["persistent", "graph", "batch"])
+def test_wide_weights_on_bit_planes(oracle, degree, wmax, path):
+    """Weights of 9 to 12 bits with sums below 2^16 (but the last row), then of up to 16 bits with sums below 2^20, in
+    every element class; on bit-planes by request, the batch on one warp, whose fitness planes fill up between
+    flushes."""
+    g = I.random_regular(240, degree, seed=degree + wmax, wmin=-wmax, wmax=wmax)
+    g.weight[:] = np.where(np.abs(g.weight) > wmax * 9 // 10, np.sign(g.weight) * wmax, g.weight)
+    P = gom.Population(g, 70, 5, persistent=path != "graph", bitsliced=True)
+    assert gom.gom_get_option(P.ctx, gom.GOM_OPT_BITSLICED) == 1
+    ep, ev = oracle.build_fos(g)
+    k, co = oracle.color(g, ep, ev)
+    run = oracle.Run(g, ep, ev, co, k, 70, 5)
+    _steps(P, run, 5, _batch_of(P, (1, 2, 1, 300)) if path == "batch" else None)
+
+
+@pytest.mark.parametrize("bound,p,wmax", [(17, 64, 3000), (24, 300, 300), (40, 65, 3000), (64, 512, 3000), (100, 70, 300),
+                                          (128, 1024, 2000), (128, 32, 2000)])
+@pytest.mark.parametrize("path", ["persistent", "batch"])
+def test_wide_weights_by_element_class(oracle, bound, p, wmax, path):
+    """Linkage trees with 9- to 12-bit weights of either sign, by element class: the persistent kernel and one block of
+    a batch, whose warps pass the sixteen items between two flushes of 20-bit sums."""
+    g = I.torus2d(20, seed=bound + p, wmin=-wmax, wmax=wmax)
+    ep, ev = oracle.build_bflt(g, bound)
+    P = gom.Population(g, p, 9, fos=gom.gom_build_fos(g, gom.GOM_FOS_BFLT, bound), bitsliced=True)
+    assert gom.gom_get_option(P.ctx, gom.GOM_OPT_BITSLICED) == 1
+    k, co = oracle.color(g, ep, ev)
+    run = oracle.Run(g, ep, ev, co, k, p, 9)
+    _load(P, run, *_few_rows(oracle, g, p, 5, bound))
+    _steps(P, run, 4, _batch_of(P, (4, 2, 1, 300)) if path == "batch" else None)
