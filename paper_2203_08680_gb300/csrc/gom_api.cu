@@ -871,7 +871,11 @@ int gom_get_population(gom_ctx_t *ctx, uint8_t *d_pop, int64_t *d_fit, int64_t *
 {
     if (!ctx) return GOM_E_ARG;
     if (d_pop) {
-        k_export_pop<<<ctx->grid_io, kRowThreads, 0, ctx->stream>>>(ctx->prm, d_pop);
+        if (export_small(ctx->n, ctx->p, ctx->W, d_pop))
+            k_export_small<<<static_cast<int>(std::min<int64_t>((int64_t(ctx->n) * ctx->p + 255) / 256, ctx->sms * 4)), 256, 0,
+                             ctx->stream>>>(ctx->prm, d_pop);
+        else
+            k_export_pop<<<ctx->grid_io, kRowThreads, 0, ctx->stream>>>(ctx->prm, d_pop);
         GOM_CUDA(ctx, cudaGetLastError());
     }
     if (d_fit)

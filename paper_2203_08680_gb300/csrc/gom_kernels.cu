@@ -230,6 +230,16 @@ __global__ void __launch_bounds__(kRowThreads) k_export_pop(GomParams P, uint8_t
     unpack_rows(P.O, P.n, P.p, P.W, out, sm);
 }
 
+// The same, one byte a thread, for small populations (export_small).
+__global__ void k_export_small(GomParams P, uint8_t *out)
+{
+    const int64_t total = (int64_t)P.p * P.n;
+    for (int64_t idx = gthread(); idx < total; idx += gthreads()) {
+        const int64_t i = idx / P.n, v = idx - i * P.n;
+        out[idx] = (uint8_t)((P.O[v * P.W + (i >> 5)] >> (i & 31)) & 1u);
+    }
+}
+
 __global__ void k_export_elite(GomParams P, uint8_t *out)
 {
     const int improved = P.st->improved;

@@ -75,5 +75,6 @@ __global__ void k_filter_select(GomParams P, int compact);
 __global__ void k_filter_scan(GomParams P, int nwarps);
 __global__ void k_filter_compact(GomParams P);
 __global__ void k_export_pop(GomParams P, uint8_t *out);
+__global__ void k_export_small(GomParams P, uint8_t *out);
 __global__ void k_export_elite(GomParams P, uint8_t *out);
 __global__ void k_import_pop(GomParams P, const uint8_t *in, const uint8_t *elite, int64_t fe, int64_t g);

@@ -55,6 +55,18 @@ __device__ __forceinline__ void transpose_bytes(uint32_t (&x)[4])
     x[3] = __byte_perm(h0, h1, 0x7632);
 }
 
+// Whether the export goes one byte a thread: rows in whole lines take a block a
+// tile of 128 variables, which has its word columns of 32 rows one after another (11
+// us for up to 8 words, twice as long for 16, 1.7 times for rows that are not
+// word-aligned), and a small population has few tiles.  One byte a thread takes 6 us and 4 a
+// MB: n = 1,089, p = 1,024 12 us against 48, n = 100, p = 256 6 / 11, n = 10,000, p =
+// 256 14 / 11.
+inline bool export_small(int64_t n, int p, int W, const void *out)
+{
+    const bool aligned = !(n & 3) && !(reinterpret_cast<uintptr_t>(out) & 3);
+    return n * p <= (int64_t)(aligned ? 1400000 : 2800000) * (W <= 8 ? 1 : W / 8);
+}
+
 // Packs rows in[p][n] (any non-zero byte is a 1) into words[n][W]; bits of
 // individuals past p are zero.  Called by every thread of the grid's blocks
 // (kRowThreads each); sm: row_words(W) words.

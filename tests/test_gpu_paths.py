@@ -258,3 +258,17 @@ def test_wide_weights_by_element_class(oracle, bound, p, wmax, path):
     run = oracle.Run(g, ep, ev, co, k, p, 9)
     _load(P, run, *_few_rows(oracle, g, p, 5, bound))
     _steps(P, run, 4, _batch_of(P, (4, 2, 1, 300)) if path == "batch" else None)
+
+
+@pytest.mark.parametrize("n,p,shift", [(28003, 101, 1), (28003, 101, 0), (30001, 100, 2), (12003, 1024, 3), (20004, 100, 0),
+                                       (20004, 100, 3), (9001, 700, 1), (9001, 300, 0), (100, 64, 0), (101, 64, 1)])
+def test_rows_out_on_either_side_of_the_size_rule(n, p, shift):
+    """The export in whole lines (the larger sizes: ragged tiles, rows and buffers off the 4-byte words) and one byte a
+    thread."""
+    P = gom.Population(I.empty_graph(n), p, 3, kind=gom.GOM_FOS_SINGLETON)
+    pop = torch.from_numpy(np.random.default_rng(n + p).integers(0, 2, (p, n), dtype=np.uint8)).cuda()
+    P.set_population(pop, pop[0].clone(), 0, 0)
+    out = torch.full((p * n + 8,), 9, dtype=torch.uint8, device="cuda")
+    gom.gom_get_population(P.ctx, out[shift:shift + p * n])
+    assert torch.equal(out[shift:shift + p * n].view(p, n), pop)
+    assert (out[:shift] == 9).all() and (out[shift + p * n:] == 9).all()
