@@ -121,7 +121,7 @@ extern "C" int gom_fitness_noalloc(const int64_t *d_row_ptr, const int32_t *d_co
     if (scratch_address(&scratch) != cudaSuccess) return GOM_E_CUDA;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     // eight (four) resident blocks a SM cover a GB300; fewer where the problem is small
-    const int64_t tiles = (num_vertices + kRowVars - 1) / kRowVars / row_tiles(W) + 1;
+    const int64_t tiles = ((num_vertices + kRowVars - 1) / kRowVars / row_tiles(W) + 1) * (W > 8 ? W / 8 : 1);
     k_noalloc_pack<<<static_cast<int>(tiles < 1216 ? tiles : 1216), kRowThreads, 0, s>>>(d_pop, num_vertices, pop, W, scratch,
                                                                                       d_fitness_out);
     if (cudaGetLastError() != cudaSuccess) return GOM_E_CUDA;
