@@ -398,7 +398,8 @@ typedef struct gom_batch gom_batch_t;
 
 typedef struct gom_batch_config {
     int32_t warps_per_block; /* 1, 2, 4 or 8 */
-    int32_t min_blocks;      /* register budget: 2 (128 registers a thread, no spills) or 3 (85) */
+    int32_t min_blocks;      /* register budget: 2 (128 registers a thread, the bit-sliced phases
+                                among its variants) or 3 (80; more warps per SM, per lane only) */
     int32_t max_blocks;      /* most blocks of the launch (0: every block that can be resident) */
     int32_t item_cost;       /* block allocation: a warp's time for one element is taken as
                                 item_cost + (population words) x (variables + edges), so

@@ -299,7 +299,7 @@ int batch_create(gom_ctx_t *const *ctxs, int32_t num, const gom_batch_config_t *
         P.learn = 0; // the learned filter is not active inside batched launches
         P.fi.on = 0; // nor Forced Improvement (refused above)
         P.bar = B->d_bars + b; // (P.trace: the context's phase trace, when switched on)
-        // (one-warp tiles: the blocks' named barriers are left to the block-mode instances)
+        // (one-warp tiles: an instance has few blocks, and its groups give each warp pairs of its own)
         if (c->bs_can) bs_split(wv, c->max_group, c->run_ms_fn ? c->ms_edges : c->max_edges, int64_t(nb[b]) * conf.warps_per_block, 1, &P.bs_lsh, &P.bs_nwi);
         B->params[b] = P;
         GomBatchInst &I = B->inst[b];

@@ -53,8 +53,9 @@ __device__ __noinline__ void batch_variant_multi(const GomParams &P, const VGrid
 // kernel variant, target and generation count (at most G).  The dynamic shared memory holds the block's
 // fitness accumulators (f_words 32-bit words, 32 W of the widest instance)
 // and then the warps' staging slices.
-// MINB: resident blocks of 256 threads the register budget is cut for (2: no
-// spills, 3: more warps per SM).
+// MINB: resident blocks of 256 threads the register budget is cut for (2: 128
+// registers, the per-lane functions spill 30 to 160 bytes, the bit-sliced ones
+// 460 to 940; 3: 80 registers and more warps per SM, 260 to 460 bytes).
 template <int MINB>
 __global__ void __launch_bounds__(kMixThreads, MINB)
     k_batch(const GomParams *Ps, const GomBatchInst *inst, GomBarrier *bars, int B, int G, int f_words)

@@ -55,9 +55,9 @@
 // read inside the lane took a generation of the 1000x1000 torus (p = 256) from
 // 2.27 to 1.31 ms against tables of packed patterns transposed across the warp
 // with a run-start search per trial; one flat edge list per element and chains
-// over four edges took it to 1.10 ms (103 warp instructions per 32 trials, the
-// ALU pipe busy 65 % of the cycles), instances with the rows known at compile
-// time and selects shared with the multiply pipe to 0.98 ms.
+// over four edges took it to 1.10 ms, instances with the rows known at compile
+// time and selects shared with the multiply pipe to 0.98 ms (103 warp
+// instructions per 32 trials, the ALU pipe busy 65 % of the cycles).
 //
 // Elements of one colour group share no variable and no edge (LMIG
 // colouring), so the rows a pair reads and writes belong to it alone during
@@ -136,7 +136,9 @@ __host__ __device__ __forceinline__ int bs_warp_words(int S)
 }
 
 // Blocks per SM the kernels' registers are cut for, by element class: what the
-// regions leave of an SM's shared memory (34, 54 and 90 KB a block).
+// regions leave of an SM's shared memory (34, 54 and 90 KB a block).  Measured
+// for 8-bit weights (torus1000: 5 blocks of 96 registers 25.5 ms a pass, 6 of 80
+// 25.1); the 20-bit sums of 5 to 8 variables spill about 210 bytes at 80.
 constexpr int bs_blocks(int SB) { return SB <= 8 ? 6 : SB <= 16 ? 4 : 2; }
 
 // This lane's fitness planes; `regions` is the block's first warp region.
@@ -739,7 +741,7 @@ __device__ __forceinline__ BsGroup bs_group(const GomParams &P, const BsMap &M, 
 // One colour group (position t) on the bit-sliced path: items of E consecutive
 // elements; tile x takes item x first -- prepared before `open`, the barrier
 // that opens the group (false: it gave up) --, then items ntiles + the claims
-// it draws from work[t] (P.dyn, one-warp tiles), one ahead, or x + ntiles, x +
+// it draws from work[t] (P.dyn; one-warp tiles, of equal items), one ahead, or x + ntiles, x +
 // 2 ntiles, ... (static stride).
 template <int SB, int R, int UB, bool LEARN, class Open>
 __device__ __forceinline__ bool phase_mix_bs(const GomParams &P, const BsMap &M, int t, int c, uint32_t g, Open open,
